@@ -4,8 +4,8 @@ Translation units and their floating-point flags:
   lbm_ref.cu, lbm_measure.cu,  -fmad=false: the canonical-order kernels must not
   lbm_adjoint.cu               contract a*b+c into an FMA (bit-exact FP64 path;
                                the adjoint recomputes the same forward values)
-  lbm_fused.cu, lbm_batch.cu   FMA allowed: the production FP32 step (one domain; many
-                               instances in one persistent launch)
+  lbm_fused.cu, lbm_tile.cu,   FMA allowed: the production FP32 step (one domain, large or
+  lbm_batch.cu                 small; many instances in one persistent launch)
   lbm_api.cu                   host code and launch orchestration
 Units compile in parallel; only stale objects are rebuilt.
 """
@@ -26,11 +26,12 @@ UNITS = {
     "lbm_ref.cu": ["-fmad=false"],
     "lbm_measure.cu": ["-fmad=false"],
     "lbm_fused.cu": [],
+    "lbm_tile.cu": [],
     "lbm_noalloc.cu": [],
     "lbm_batch.cu": [],
     "lbm_adjoint.cu": ["-fmad=false"],
 }
-HEADERS = [os.path.join(CSRC, h) for h in ("lbm_internal.h", "lbm_node.cuh", "lbm_ref_node.cuh")] + [
+HEADERS = [os.path.join(CSRC, h) for h in ("lbm_internal.h", "lbm_fused.h", "lbm_node.cuh", "lbm_ref_node.cuh")] + [
     os.path.join(ROOT, "include", "lbm.h")]
 
 

@@ -30,8 +30,7 @@
 #include <math.h>
 #include <stdlib.h>
 
-#include "lbm_internal.h"
-#include "lbm_node.cuh"
+#include "lbm_fused.h"
 
 namespace {
 
@@ -59,23 +58,6 @@ struct Cfg {
   static constexpr int MIN_CTAS = 4;                            // register budget per thread
 };
 constexpr unsigned long long kWaitNs = 2000000000ull;  // 2 s per bounded wait
-
-struct FusedArgs {
-  int nx, ny, walls, wetting, n_iter, kind;
-  int nstrips, nrows, y0;
-  long long total;
-  int stages;
-  float b4, RT2, a2, r1, r2, pc0, pc1, pc2;    // EOS constants (b/4, -2RT, 2a; Eq. 11 break-
-                                                // points and slopes folded into -2U)
-  float A, omA, pre, halfA, rho_max, ghost_max; // force / Q constants, bounds
-  lbm_node::RateK k;                            // relaxation constants
-  float Gw;
-  long long eoff[9];  // byte offset of plane a's destination from (row y, column x) of plane 0 for an
-                      // interior node: 4 (a n + e_ay nx + e_ax) (streaming without wrap or bounce-back)
-  const double *coef;
-  float *fout;
-  int *flag;
-};
 
 __device__ __forceinline__ unsigned smem_u32(const void *p) {
   return (unsigned)__cvta_generic_to_shared(p);
@@ -127,7 +109,7 @@ struct Seq {
   long long u, u1;
   int strip, v, vend, ya, yb;
   bool has;
-  __device__ void start(const FusedArgs &P) {
+  __device__ void start(const lbm_fused_args &P) {
     if (u >= u1) { has = false; return; }
     strip = (int)(u / P.nrows);
     int r0 = (int)(u - (long long)strip * P.nrows);
@@ -140,16 +122,16 @@ struct Seq {
     u += cnt;
     has = true;
   }
-  __device__ void init(const FusedArgs &P, long long a, long long b) { u = a; u1 = b; start(P); }
-  __device__ void next(const FusedArgs &P) {
+  __device__ void init(const lbm_fused_args &P, long long a, long long b) { u = a; u1 = b; start(P); }
+  __device__ void next(const lbm_fused_args &P) {
     if (v < vend) ++v; else start(P);
   }
-  __device__ bool solid(const FusedArgs &P) const { return P.walls && (v == 0 || v == P.ny - 1); }
+  __device__ bool solid(const lbm_fused_args &P) const { return P.walls && (v == 0 || v == P.ny - 1); }
 };
 
 template <bool UNIT, int NC, int MCW, int KIND>
 __global__ void __launch_bounds__(NCONS, Cfg<NC>::MIN_CTAS)
-    k_fused(const __grid_constant__ CUtensorMap tm_main, const __grid_constant__ CUtensorMap tm_halo, FusedArgs P) {
+    k_fused(const __grid_constant__ CUtensorMap tm_main, const __grid_constant__ CUtensorMap tm_halo, lbm_fused_args P) {
   static_assert(NC == 2, "two columns per thread: one lane pair");
   constexpr int W = Cfg<NC>::W, WIN = Cfg<NC>::WIN, WP = Cfg<NC>::WP, MAIN_BYTES = Cfg<NC>::MAIN_BYTES;
   constexpr int STAGE_BYTES = Cfg<NC>::STAGE_BYTES;
@@ -535,7 +517,7 @@ size_t smem_bytes(int stages) {
 // the eight specialisations: collision (unit or general rates) x wetting
 // rule (geometric or Martys-Chen) x EOS (Carnahan-Starling or Eq. 11), each
 // fixed at compile time so that no branch is left in the per-node arithmetic
-typedef void (*FusedKernel)(CUtensorMap, CUtensorMap, FusedArgs);
+typedef void (*FusedKernel)(CUtensorMap, CUtensorMap, lbm_fused_args);
 template <bool UNIT, int MCW>
 FusedKernel pick_kind(int kind) {
   return kind == LBM_EOS_CARNAHAN_STARLING ? (FusedKernel)k_fused<UNIT, kNC, MCW, LBM_EOS_CARNAHAN_STARLING>
@@ -566,6 +548,11 @@ int lbm_fused_plan(lbm_ctx *C) {
   // the diag(0,1,...,1) relaxation of Sec. 3.1 takes the specialised collision
   const lbm_dev_params &D = C->dp;
   C->fused_unit = D.s[1] == 1.0 && D.s[2] == 1.0 && D.s[4] == 1.0 && D.s[7] == 1.0;
+  lbm_tile_plan(C);
+  if (C->tile_rows) {
+    C->fused_ok = 1;
+    return 1;
+  }
   const void *kern = (const void *)kernel_ptr(C->fused_unit, D.wetting == LBM_WET_MARTYS_CHEN, D.eos_kind);
   int dev = 0, nsm = 0, occ = 0, optin = 0;
   cudaGetDevice(&dev);
@@ -608,54 +595,11 @@ int lbm_fused_plan(lbm_ctx *C) {
 
 namespace {
 
-// Launch arguments of a context's step (all but the destination array).
-FusedArgs fused_args(const lbm_ctx *C) {
-  FusedArgs P;
-  const lbm_dev_params &D = C->dp;
-  const int W = C->tile_w;
-  P.nx = C->nx;
-  P.ny = C->ny;
-  P.walls = C->walls;
-  P.wetting = D.wetting;
-  P.n_iter = D.n_iter;
-  P.kind = D.eos_kind;
-  P.nstrips = (C->nx + W - 1) / W;
-  P.nrows = C->walls ? C->ny - 2 : C->ny;
-  P.y0 = C->walls ? 1 : 0;
-  P.total = (long long)P.nstrips * P.nrows;
-  P.stages = C->tile_stages;
-  P.b4 = (float)(0.25 * D.b);
-  P.RT2 = (float)(-2.0 * D.R * D.T);
-  P.a2 = (float)(2.0 * D.a);
-  P.r1 = (float)D.r1;
-  P.r2 = (float)D.r2;
-  P.pc0 = (float)(-2.0 * (D.thv - 1.0 / 3.0));
-  P.pc1 = (float)(-2.0 * (D.thm - D.thv));
-  P.pc2 = (float)(-2.0 * (D.thl - D.thm));
-  P.A = (float)D.A;
-  P.omA = (float)(1.0 - D.A);
-  P.pre = (float)(-0.5 * D.kappa);
-  P.halfA = (float)(0.5 * D.A);
-  P.rho_max = (float)fmin(D.rho_max, 3.0e38);
-  P.ghost_max = (float)fmin(D.ghost_max, 3.0e38);
-  P.k = lbm_node::rate_consts(D.s);
-  P.Gw = (float)D.Gw;
-  {
-    const long long n = (long long)C->nx * C->ny, nx = C->nx;
-    const int ex[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1}, ey[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
-    for (int k = 0; k < 9; ++k) P.eoff[k] = 4 * (k * n + ey[k] * nx + ex[k]);
-  }
-  P.coef = C->d_coef;
-  P.fout = nullptr;
-  P.flag = C->d_flag;
-  return P;
-}
-
 // Launched with programmatic stream serialisation (the kernel orders its own
 // global accesses after the previous grid with griddepcontrol.wait), so that
 // back-to-back steps overlap one grid's tail with the next grid's launch and
 // set-up; LBM_FUSED_PDL=0 turns it off.
-cudaError_t launch_fused(lbm_ctx *C, const CUtensorMap &tm, const CUtensorMap &th, const FusedArgs &P,
+cudaError_t launch_fused(lbm_ctx *C, const CUtensorMap &tm, const CUtensorMap &th, const lbm_fused_args &P,
                          unsigned long long *launches) {
   static const int pdl = [] {
     const char *e = getenv("LBM_FUSED_PDL");
@@ -680,18 +624,20 @@ cudaError_t launch_fused(lbm_ctx *C, const CUtensorMap &tm, const CUtensorMap &t
 }  // namespace
 
 cudaError_t lbm_fused_step(lbm_ctx *C, int src, unsigned long long *launches) {
-  FusedArgs P = fused_args(C);
+  if (C->tile_rows) return lbm_tile_step(C, C->f[src], C->f[src ^ 1], launches);
+  lbm_fused_args P = lbm_make_fused_args(C);
   P.fout = (float *)C->f[src ^ 1];
   return launch_fused(C, *(const CUtensorMap *)C->tmaps[2 * src], *(const CUtensorMap *)C->tmaps[2 * src + 1], P,
                       launches);
 }
 
 cudaError_t lbm_fused_step_between(lbm_ctx *C, const void *src, void *dst, unsigned long long *launches) {
+  if (C->tile_rows) return lbm_tile_step(C, src, dst, launches);
   CUtensorMap tm, th;
   if (!encode(&tm, const_cast<void *>(src), C->nx, C->ny, C->tile_w) ||
       !encode(&th, const_cast<void *>(src), C->nx, C->ny, HB))
     return cudaErrorInvalidValue;
-  FusedArgs P = fused_args(C);
+  lbm_fused_args P = lbm_make_fused_args(C);
   P.fout = (float *)dst;
   return launch_fused(C, tm, th, P, launches);
 }

@@ -71,6 +71,7 @@ struct lbm_ctx {
   // fused kernel plan
   int fused_ok, fused_unit;  // fused kernel usable; unit-rate specialisation
   int fused_cols;            // columns per thread of the fused kernel
+  int tile_rows;             // rows per tile of the small-domain kernel, 0: the ring kernel runs
   int tile_w, tile_blocks, tile_stages, fused_smem;
   unsigned char tmaps[4][128];   // CUtensorMap for f[0], f[1]: main box, halo box
   // lbm_step graphs, captured at the first lbm_step for both starting arrays:
@@ -104,6 +105,10 @@ cudaError_t lbm_fused_step(lbm_ctx *C, int src, unsigned long long *launches);
 // The same step between any two state arrays of the context's shape (16-byte
 // aligned): the adjoint's recorded forward and its segment replays.
 cudaError_t lbm_fused_step_between(lbm_ctx *C, const void *src, void *dst, unsigned long long *launches);
+
+// ---- lbm_tile.cu: the FP32 step of small domains ------------------------------
+void lbm_tile_plan(lbm_ctx *C);  // sets tile_rows (0: not for this domain) and the tile_* shape
+cudaError_t lbm_tile_step(const lbm_ctx *C, const void *src, void *dst, unsigned long long *launches);
 
 // ---- lbm_adjoint.cu: discrete adjoint ---------------------------------------
 void lbm_adjoint_free_tape(lbm_ctx *C);

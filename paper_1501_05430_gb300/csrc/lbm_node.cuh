@@ -88,11 +88,11 @@ __device__ __forceinline__ float4 eos_node(const PT &P, float rho) {
 }
 
 // Eqs. 19-21 ghost entry at column x from the boundary-row densities rl, ri1,
-// rr (at x-1, x, x+1) and the second-row density ri2 (at x); gx indexes the
-// wall coefficients; top: 0 or 1.
+// rr (at x-1, x, x+1), the second-row density ri2 (at x) and the wall
+// coefficients cc = sin(pi/2 - theta), cot = tan(pi/2 - theta).
 template <int KIND = -1, class PT>
-__device__ __forceinline__ float4 ghost_value(const PT &P, float rl, float ri1, float rr, float ri2, int gx, int top) {
-  float cc = (float)P.coef[top * P.nx + gx], cot = (float)P.coef[(2 + top) * P.nx + gx];
+__device__ __forceinline__ float4 ghost_rule(const PT &P, float rl, float ri1, float rr, float ri2, float cc,
+                                             float cot) {
   float aa = rr - rl, g;
   if (P.n_iter <= 0) {
     g = fmaf(cot, fabsf(aa), ri2);
@@ -106,6 +106,12 @@ __device__ __forceinline__ float4 ghost_value(const PT &P, float rl, float ri1, 
   }
   g = fminf(fmaxf(g, 0.0f), P.ghost_max);
   return g < P.rho_max ? eos_node<KIND>(P, g) : make_float4(g, 0.0f, 0.0f, 0.0f);  // psi = U = 0 at rho_max
+}
+
+// The same with the coefficients of column gx; top: 0 or 1.
+template <int KIND = -1, class PT>
+__device__ __forceinline__ float4 ghost_value(const PT &P, float rl, float ri1, float rr, float ri2, int gx, int top) {
+  return ghost_rule<KIND>(P, rl, ri1, rr, ri2, (float)P.coef[top * P.nx + gx], (float)P.coef[(2 + top) * P.nx + gx]);
 }
 
 // The same from window rows: r1 boundary row, r2 second row, column c stored

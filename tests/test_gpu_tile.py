@@ -1,0 +1,85 @@
+"""The small-domain kernel of the FP32 step (one tile per CTA) against the ring
+kernel: the same per-node operations on the same values, so the same bits, and
+the same verdict on an unstable state.  (Both are compared with the oracle in
+test_gpu_parity.py.)"""
+import numpy as np
+import pytest
+
+from paper_1501_05430_gb300 import inputs as I
+from paper_1501_05430_gb300 import lbm as L
+
+from helpers import Case
+
+pytestmark = pytest.mark.gpu
+
+PW10 = (0.25, -0.02, 0.3, 1.1216073327407194, 9.540106186999981)
+MODELS = {
+    "geometric": dict(),
+    "eq19": dict(n_iter=0),
+    "general_rates": dict(rates=dict(s_e=0.8, s_eps=0.9, s_j=1.0, s_q=1.1), tau=0.8),
+    "martys_chen": dict(wetting=1, G_w=-0.2),
+    "martys_chen_general": dict(wetting=1, G_w=-0.2, tau=0.9),
+    "piecewise": dict(eos="pw", pw=PW10),
+    "piecewise_martys_chen_general": dict(eos="pw", pw=PW10, wetting=1, G_w=-0.1, tau=0.8),
+    "periodic": dict(walls=False),
+}
+# one and several strips with a ragged last one, bands with every remainder
+# (walled: ny - 2 rows), the smallest grid
+SIZES = [(4, 5), (64, 6), (60, 7), (68, 8), (132, 9), (260, 24), (128, 13)]
+
+
+def _context(c, f, monkeypatch, ring):
+    if ring:
+        monkeypatch.setenv("LBM_FUSED_STAGES", "3")
+    else:
+        monkeypatch.delenv("LBM_FUSED_STAGES", raising=False)
+    g = L.Lbm(c.nx, c.ny, c.geos, c.T, c.tau, theta=c.theta, walls=c.walls, params=c.params, torch_state=False)
+    assert g.info.kernel_in_use == L.LBM_KERNEL_FUSED
+    assert (g.info.tile_stages > 0) == ring
+    g.set_f(f)
+    return g
+
+
+def _case(nx, ny, seed, **kw):
+    rng = np.random.default_rng(seed)
+    c = Case(nx, ny, theta=rng.uniform(np.deg2rad(20), np.deg2rad(160), (ny, nx)), precision=32, **kw)
+    rho = I.droplet_field(nx, ny, [(nx * 0.3, ny * 0.35, 0), (nx * 0.75, ny * 0.3, 1)], c.rho_v, c.rho_l)
+    return c, I.random_distributions(rho, seed, walls=c.walls)
+
+
+@pytest.mark.parametrize("nx,ny", SIZES)
+@pytest.mark.parametrize("name", list(MODELS))
+def test_tile_and_ring_kernels_give_the_same_bits(name, nx, ny, monkeypatch):
+    c, f = _case(nx, ny, nx + ny, **MODELS[name])
+    out = []
+    for ring in (False, True):
+        with _context(c, f, monkeypatch, ring) as g:
+            g.step(7)
+            out.append((g.f(), g.status()))
+    c.orc.close()
+    assert np.array_equal(out[0][0], out[1][0])
+    assert out[0][1] == out[1][1] == 0
+
+
+@pytest.mark.parametrize("nx,ny", [(128, 8300), (72, 30001)])
+def test_narrow_domains_above_2_20_nodes(nx, ny, monkeypatch):
+    """Tiles of six rows (the second: a size at which wide domains take the ring)."""
+    c, f = _case(nx, ny, 3, tau=0.8)
+    out = []
+    for ring in (False, True):
+        with _context(c, f, monkeypatch, ring) as g:
+            g.step(3)
+            out.append(g.f())
+    c.orc.close()
+    assert np.array_equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("y,x", [(1, 0), (3, 63), (4, 64), (8, 67)])
+def test_tile_kernel_flags_an_unstable_node(y, x, monkeypatch):
+    """A density of 0 in the first and last row and column of tiles."""
+    c, f = _case(68, 10, 5)
+    f[:, y, x] = 0.0
+    with _context(c, f, monkeypatch, False) as g:
+        g.step(1)
+        assert g.status() == L.LBM_EUNSTABLE
+    c.orc.close()
