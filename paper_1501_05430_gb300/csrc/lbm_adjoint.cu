@@ -435,7 +435,9 @@ int capture(lbm_ctx *C, cudaGraphExec_t *out, unsigned long long *launches, Fn f
     return LBM_ECUDA;
   }
   const unsigned long long l0 = C->launches;
+  C->capturing = 1;
   int st = fn();
+  C->capturing = 0;
   *launches = C->launches - l0;
   C->launches = l0;
   cudaError_t e = cudaStreamEndCapture(C->stream, &graph);

@@ -285,7 +285,9 @@ int capture_steps(lbm_ctx *C, int start, int G, cudaGraphExec_t *out) {
   }
   unsigned long long dummy = 0;
   cudaError_t e = cudaSuccess;
+  C->capturing = 1;
   for (int k = 0; k < G && e == cudaSuccess; ++k) e = launch_step(C, start ^ (k & 1), &dummy);
+  C->capturing = 0;
   cudaError_t e2 = cudaStreamEndCapture(C->stream, &graph);
   if (e == cudaSuccess) e = e2;
   if (e == cudaSuccess) e = cudaGraphInstantiate(out, graph, 0);

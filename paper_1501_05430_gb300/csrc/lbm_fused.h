@@ -13,6 +13,7 @@ struct lbm_fused_args {
   int nstrips, nrows, y0;
   long long total;
   int stages;
+  int pdl;  // tile kernel: launched as a programmatic dependent
   float b4, RT2, a2, r1, r2, pc0, pc1, pc2;    // EOS constants (b/4, -2RT, 2a; Eq. 11 break-
                                                 // points and slopes folded into -2U)
   float A, omA, pre, halfA, rho_max, ghost_max; // force / Q constants, bounds
@@ -41,6 +42,7 @@ inline lbm_fused_args lbm_make_fused_args(const lbm_ctx *C) {
   P.y0 = C->walls ? 1 : 0;
   P.total = (long long)P.nstrips * P.nrows;
   P.stages = C->tile_stages;
+  P.pdl = 0;
   P.b4 = (float)(0.25 * D.b);
   P.RT2 = (float)(-2.0 * D.R * D.T);
   P.a2 = (float)(2.0 * D.a);

@@ -80,6 +80,7 @@ struct lbm_ctx {
   // most one direct launch
   static constexpr int kMaxGraphs = 17;
   int ngraph, graphs_ready;
+  int capturing;             // the library is recording launches of this context into a graph
   int graph_len[kMaxGraphs];
   cudaGraphExec_t step_graph[2][kMaxGraphs];
 };
