@@ -89,9 +89,8 @@ __device__ void eos_derivs(const Mdl<R> &m, R rho, R &dp_drho, R &dp_dT) {
 }
 
 template <typename R>
-__global__ void k_adj_collide(lbm_dev_params P, const R *__restrict__ f, const R *__restrict__ fields,
+__global__ void k_adj_collide(Mdl<R> m, const R *__restrict__ f, const R *__restrict__ fields,
                               const R *__restrict__ lam_in, R *__restrict__ lam_out, R *__restrict__ aux) {
-  Mdl<R> m(P);
   size_t n = (size_t)m.nx * m.ny;
   size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
@@ -175,9 +174,8 @@ __global__ void k_adj_collide(lbm_dev_params P, const R *__restrict__ f, const R
 }
 
 template <typename R>
-__global__ void k_adj_psi(lbm_dev_params P, const R *__restrict__ fields, const R *__restrict__ aux,
+__global__ void k_adj_psi(Mdl<R> m, const R *__restrict__ fields, const R *__restrict__ aux,
                           R *__restrict__ rhob_out, double *__restrict__ tacc) {
-  Mdl<R> m(P);
   size_t n = (size_t)m.nx * m.ny;
   size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
@@ -250,10 +248,9 @@ __global__ void k_adj_psi(lbm_dev_params P, const R *__restrict__ fields, const 
 }
 
 template <typename R>
-__global__ void k_adj_ghost(lbm_dev_params P, const R *__restrict__ fields, const double *__restrict__ coef,
+__global__ void k_adj_ghost(Mdl<R> m, const R *__restrict__ fields, const double *__restrict__ coef,
                             const double *__restrict__ dcoef, const R *__restrict__ rhob,
                             double *__restrict__ gpart, double *__restrict__ dtheta) {
-  Mdl<R> m(P);
   int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= 2 * m.nx) return;
   int w = t / m.nx, x = t - w * m.nx;
@@ -317,9 +314,8 @@ __global__ void k_adj_ghost(lbm_dev_params P, const R *__restrict__ fields, cons
 }
 
 template <typename R>
-__global__ void k_adj_finish(lbm_dev_params P, R *__restrict__ lam, const R *__restrict__ rhob,
+__global__ void k_adj_finish(Mdl<R> m, R *__restrict__ lam, const R *__restrict__ rhob,
                              const double *__restrict__ gpart, int geo) {
-  Mdl<R> m(P);
   size_t n = (size_t)m.nx * m.ny;
   size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
@@ -406,20 +402,20 @@ int reverse_step(lbm_ctx *C, lbm_tape *T, const void *f, int lin) {
   const size_t n = (size_t)C->nx * C->ny;
   const int B = 256;
   const unsigned g = (unsigned)((n + B - 1) / B), gw = (unsigned)((2 * C->nx + B - 1) / B);
-  const lbm_dev_params &P = C->dp;
+  const Mdl<R> m(C->dp);
   const R *fields = (const R *)C->d_fields;
   ACK(lbm_ref_fields(C, f, C->d_fields, &C->launches));
   R *lam_in = (R *)T->lam[lin], *lam_out = (R *)T->lam[lin ^ 1];
-  k_adj_collide<R><<<g, B, 0, C->stream>>>(P, (const R *)f, fields, lam_in, lam_out, (R *)T->aux);
-  k_adj_psi<R><<<g, B, 0, C->stream>>>(P, fields, (const R *)T->aux, (R *)T->rhob, T->tacc);
+  k_adj_collide<R><<<g, B, 0, C->stream>>>(m, (const R *)f, fields, lam_in, lam_out, (R *)T->aux);
+  k_adj_psi<R><<<g, B, 0, C->stream>>>(m, fields, (const R *)T->aux, (R *)T->rhob, T->tacc);
   C->launches += 2;
-  const int geo = C->walls && P.wetting == LBM_WET_GEOMETRIC;
+  const int geo = C->walls && m.wetting == LBM_WET_GEOMETRIC;
   if (geo) {
-    k_adj_ghost<R><<<gw, B, 0, C->stream>>>(P, fields, C->d_coef, C->d_dcoef, (const R *)T->rhob, T->gpart,
+    k_adj_ghost<R><<<gw, B, 0, C->stream>>>(m, fields, C->d_coef, C->d_dcoef, (const R *)T->rhob, T->gpart,
                                             T->dtheta);
     ++C->launches;
   }
-  k_adj_finish<R><<<g, B, 0, C->stream>>>(P, lam_out, (const R *)T->rhob, T->gpart, geo);
+  k_adj_finish<R><<<g, B, 0, C->stream>>>(m, lam_out, (const R *)T->rhob, T->gpart, geo);
   ++C->launches;
   ACK(cudaGetLastError());
   return LBM_OK;

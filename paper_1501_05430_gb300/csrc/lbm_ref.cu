@@ -33,9 +33,8 @@ __device__ __forceinline__ R node_rho(const R *__restrict__ f, size_t n, size_t 
 // which the thread sums itself in the same order as their own threads do, or
 // the zero potential (Martys-Chen).
 template <typename R>
-__global__ void k_fields(lbm_dev_params P, const R *__restrict__ f, const double *__restrict__ coef,
+__global__ void k_fields(Mdl<R> m, const R *__restrict__ f, const double *__restrict__ coef,
                          R *__restrict__ fields, int *flag) {
-  Mdl<R> m(P);
   size_t n = (size_t)m.nx * m.ny;
   size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
@@ -82,9 +81,8 @@ __global__ void k_fields(lbm_dev_params P, const R *__restrict__ f, const double
 }
 
 template <typename R>
-__global__ void k_collide(lbm_dev_params P, const R *__restrict__ fin, R *__restrict__ fout,
+__global__ void k_collide(Mdl<R> m, const R *__restrict__ fin, R *__restrict__ fout,
                           const R *__restrict__ fields) {
-  Mdl<R> m(P);
   size_t n = (size_t)m.nx * m.ny;
   size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
@@ -110,9 +108,8 @@ __global__ void k_collide(lbm_dev_params P, const R *__restrict__ fin, R *__rest
 // Macroscopic outputs at every node: out7 = {ux, uy, Fx, Fy, Qxx, Qyy, Qxy}
 // (zero on the solid rows).
 template <typename R>
-__global__ void k_macro(lbm_dev_params P, const R *__restrict__ f, const R *__restrict__ fields,
+__global__ void k_macro(Mdl<R> m, const R *__restrict__ f, const R *__restrict__ fields,
                         double *__restrict__ out7) {
-  Mdl<R> m(P);
   size_t n = (size_t)m.nx * m.ny;
   size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
@@ -241,10 +238,10 @@ inline unsigned nblk(size_t n, int t) { return (unsigned)((n + t - 1) / t); }
 cudaError_t lbm_ref_fields(const lbm_ctx *C, const void *f, void *fields, unsigned long long *launches) {
   size_t n = (size_t)C->nx * C->ny;
   if (C->precision == 64)
-    k_fields<double><<<nblk(n, 256), 256, 0, C->stream>>>(C->dp, (const double *)f, C->d_coef, (double *)fields,
+    k_fields<double><<<nblk(n, 256), 256, 0, C->stream>>>(Mdl<double>(C->dp), (const double *)f, C->d_coef, (double *)fields,
                                                           C->d_flag);
   else
-    k_fields<float><<<nblk(n, 256), 256, 0, C->stream>>>(C->dp, (const float *)f, C->d_coef, (float *)fields,
+    k_fields<float><<<nblk(n, 256), 256, 0, C->stream>>>(Mdl<float>(C->dp), (const float *)f, C->d_coef, (float *)fields,
                                                          C->d_flag);
   ++*launches;
   return cudaGetLastError();
@@ -254,10 +251,10 @@ cudaError_t lbm_ref_collide(const lbm_ctx *C, const void *fin, void *fout, const
                             unsigned long long *launches) {
   size_t n = (size_t)C->nx * C->ny;
   if (C->precision == 64)
-    k_collide<double><<<nblk(n, 128), 128, 0, C->stream>>>(C->dp, (const double *)fin, (double *)fout,
+    k_collide<double><<<nblk(n, 128), 128, 0, C->stream>>>(Mdl<double>(C->dp), (const double *)fin, (double *)fout,
                                                            (const double *)fields);
   else
-    k_collide<float><<<nblk(n, 128), 128, 0, C->stream>>>(C->dp, (const float *)fin, (float *)fout,
+    k_collide<float><<<nblk(n, 128), 128, 0, C->stream>>>(Mdl<float>(C->dp), (const float *)fin, (float *)fout,
                                                           (const float *)fields);
   ++*launches;
   return cudaGetLastError();
@@ -267,9 +264,9 @@ cudaError_t lbm_ref_macro(const lbm_ctx *C, const void *f, const void *fields, d
                           unsigned long long *launches) {
   size_t n = (size_t)C->nx * C->ny;
   if (C->precision == 64)
-    k_macro<double><<<nblk(n, 128), 128, 0, C->stream>>>(C->dp, (const double *)f, (const double *)fields, out7);
+    k_macro<double><<<nblk(n, 128), 128, 0, C->stream>>>(Mdl<double>(C->dp), (const double *)f, (const double *)fields, out7);
   else
-    k_macro<float><<<nblk(n, 128), 128, 0, C->stream>>>(C->dp, (const float *)f, (const float *)fields, out7);
+    k_macro<float><<<nblk(n, 128), 128, 0, C->stream>>>(Mdl<float>(C->dp), (const float *)f, (const float *)fields, out7);
   ++*launches;
   return cudaGetLastError();
 }

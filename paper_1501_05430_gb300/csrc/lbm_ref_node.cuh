@@ -38,12 +38,16 @@ __device__ __forceinline__ double NRM(int k) {
   return t[k];
 }
 
+// The model constants in the kernels' precision, rounded once on the host and
+// passed by value: converted in the kernel, the two dozen double constants
+// cost every thread of a float kernel as many instructions of the FP64 pipe
+// (2 lanes per clock and SM), more than its arithmetic.
 template <typename R>
 struct Mdl {
   int nx, ny, walls, kind, n_iter, wetting;
   R a, b, Rg, T, thv, thm, thl, r1, r2, A, kappa, Gw, rho_max, ghost_max;
   R s[9];
-  __device__ explicit Mdl(const lbm_dev_params &P)
+  explicit Mdl(const lbm_dev_params &P)
       : nx(P.nx), ny(P.ny), walls(P.walls), kind(P.eos_kind), n_iter(P.n_iter), wetting(P.wetting),
         a((R)P.a), b((R)P.b), Rg((R)P.R), T((R)P.T), thv((R)P.thv), thm((R)P.thm), thl((R)P.thl),
         r1((R)P.r1), r2((R)P.r2), A((R)P.A), kappa((R)P.kappa), Gw((R)P.Gw), rho_max((R)P.rho_max),
