@@ -62,8 +62,8 @@ extern "C" {
 enum { LBM_EOS_CARNAHAN_STARLING = 0, LBM_EOS_PIECEWISE = 1 };
 enum { LBM_WET_GEOMETRIC = 0, LBM_WET_MARTYS_CHEN = 1 };
 /* Kernel choice for lbm_step: AUTO takes the fused single-pass kernel when the
- * context qualifies (FP32, nx % 4 == 0) and the unfused reference kernels
- * otherwise; REFERENCE forces the unfused kernels (the path that follows the
+ * context qualifies (FP32, nx % 4 == 0) and the canonical-order kernel
+ * otherwise; REFERENCE forces the canonical kernel (the path that follows the
  * canonical evaluation order, bit-identical to an FP64 CPU evaluation in the
  * same order); FUSED demands the fused kernel (LBM_EUNSUPPORTED if the
  * context does not qualify). */
@@ -310,7 +310,7 @@ int lbm_mass_noalloc(const void *f, int nx, int ny, int precision, int walls, do
  * (adjoint) of the step, with the initial state held fixed.  The recorded
  * forward and the segment replays of the backward sweep run the context's own
  * step kernel, so the recorded trajectory is the one lbm_step produces: at
- * precision 64 the canonical reference kernels (bit-identical to an FP64
+ * precision 64 the canonical kernel (bit-identical to an FP64
  * evaluation of the step in that order), at precision 32 the fused kernel when
  * the context uses it.  The reverse sweep transposes the canonical step at each
  * recorded state, so in FP32 the gradient is the canonical step's transpose

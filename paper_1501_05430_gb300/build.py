@@ -1,8 +1,8 @@
 """Build liblbm.so (the C-ABI library) in-tree with nvcc for sm_103a.
 
 Translation units and their floating-point flags:
-  lbm_ref.cu, lbm_measure.cu,  -fmad=false: the canonical-order kernels must not
-  lbm_adjoint.cu               contract a*b+c into an FMA (bit-exact FP64 path;
+  lbm_ref.cu, lbm_canon.cu,    -fmad=false: the canonical-order kernels must not
+  lbm_measure.cu,              contract a*b+c into an FMA (bit-exact FP64 path;
                                the adjoint recomputes the same forward values)
   lbm_fused.cu, lbm_tile.cu,   FMA allowed: the production FP32 step (one domain, large or
   lbm_batch.cu                 small; many instances in one persistent launch)
@@ -24,6 +24,7 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 UNITS = {
     "lbm_api.cu": [],
     "lbm_ref.cu": ["-fmad=false"],
+    "lbm_canon.cu": ["-fmad=false"],
     "lbm_measure.cu": ["-fmad=false"],
     "lbm_fused.cu": [],
     "lbm_tile.cu": [],

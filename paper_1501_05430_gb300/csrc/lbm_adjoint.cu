@@ -385,15 +385,14 @@ size_t rsize(const lbm_ctx *C) { return C->precision == 64 ? sizeof(double) : si
 
 // One forward step src -> dst with the context's own step kernel: the fused
 // FP32 kernel where the context runs it (so the recorded forward advances
-// exactly like lbm_step), else the canonical reference kernels.  The reverse
+// exactly like lbm_step), else the canonical kernel.  The reverse
 // kernels transpose the canonical step at the states this produces.
 int fwd_step(lbm_ctx *C, const void *src, void *dst) {
   if (C->kernel_in_use == LBM_KERNEL_FUSED) {
     ACK(lbm_fused_step_between(C, src, dst, &C->launches));
     return LBM_OK;
   }
-  ACK(lbm_ref_fields(C, src, C->d_fields, &C->launches));
-  ACK(lbm_ref_collide(C, src, dst, C->d_fields, &C->launches));
+  ACK(lbm_canon_step(C, src, dst, &C->launches));
   return LBM_OK;
 }
 

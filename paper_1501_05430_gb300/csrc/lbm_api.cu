@@ -261,12 +261,8 @@ int read_flags(lbm_ctx *C) {
 cudaError_t launch_step(lbm_ctx *C, int src, unsigned long long *launches) {
   const int dst = src ^ 1;
   if (C->kernel_in_use == LBM_KERNEL_FUSED) return lbm_fused_step(C, src, launches);
-  cudaError_t e = lbm_ref_fields(C, C->f[src], C->d_fields, launches);
-  if (e == cudaSuccess) e = lbm_ref_collide(C, C->f[src], C->f[dst], C->d_fields, launches);
-  return e;
+  return lbm_canon_step(C, C->f[src], C->f[dst], launches);
 }
-
-int launches_per_step(const lbm_ctx *C) { return C->kernel_in_use == LBM_KERNEL_FUSED ? 1 : 2; }
 
 // Steps per captured graph (even), or 0 when graphs are off or impossible
 // (the legacy default stream cannot be captured).
@@ -404,7 +400,6 @@ int create_impl(int nx, int ny, const lbm_eos *eos, double T, double tau, const 
 
   size_t n = (size_t)nx * ny, rs = real_size(P.precision);
   size_t need = 2 * 9 * n * rs;
-  int st = LBM_OK;
   if (state) {
     if (state_bytes < need || ((uintptr_t)state & 255)) { delete C; return LBM_EINVAL; }
     C->state = state;
@@ -461,10 +456,6 @@ int create_impl(int nx, int ny, const lbm_eos *eos, double T, double tau, const 
   if (P.precision == 32 && P.kernel != LBM_KERNEL_REFERENCE) lbm_fused_plan(C);
   if (P.kernel == LBM_KERNEL_FUSED && !C->fused_ok) { lbm_destroy(C); return LBM_EUNSUPPORTED; }
   C->kernel_in_use = C->fused_ok ? LBM_KERNEL_FUSED : LBM_KERNEL_REFERENCE;
-  if (C->kernel_in_use == LBM_KERNEL_REFERENCE && (st = ensure_fields(C)) != LBM_OK) {
-    lbm_destroy(C);
-    return st;
-  }
   if (cudaStreamSynchronize(C->stream) != cudaSuccess) { cudaGetLastError(); lbm_destroy(C); return LBM_ECUDA; }
   *out = C;
   return LBM_OK;
@@ -609,7 +600,7 @@ int lbm_step(lbm_ctx *C, int nsteps) {
       const int len = C->graph_len[k];
       while (nsteps - it >= len) {
         CK(cudaGraphLaunch(C->step_graph[C->cur][k], C->stream));
-        C->launches += (unsigned long long)len * launches_per_step(C);
+        C->launches += (unsigned long long)len;
         const long long before = C->steps;
         C->steps += len;
         it += len;

@@ -1,0 +1,469 @@
+// lbm_canon.cu -- the step in the canonical evaluation order (the one of
+// lbm_ref_node.cuh), one kernel per step: FP64 domains, and FP32 domains whose
+// width the fused kernels do not take.  Every result has the bits of the
+// plain form in lbm_ref_node.cuh (compiled, like it, without contraction); the
+// operations that cost most are only arranged anew:
+//  - a product by a power of two is exact, so the sum it goes into takes it as
+//    a fused multiply-add with the same single rounding, and such factors move
+//    freely through roundings (4 f_0 - 2 f_1 is twice 2 f_0 - f_1);
+//  - x / 3, x / 9, x / 36, x / 6, x / 12: one product and one fused
+//    multiply-add (div_const below) instead of a general division;
+//  - values that several sums use in the same order are formed once (prefixes
+//    of the inverse transform, psi^2, and, per node instead of per neighbour,
+//    the weighted psi and U of the FP64 kernel).
+// About 350 FP64 operations per node instead of 700, and one pass over the
+// populations instead of two and a pass over three fields (FP32: 72 bytes per
+// node instead of 132).  us per step, before -> now: FP64 100 x 60 29.6 -> 16.7,
+// 400 x 200 104 -> 79; FP32 1001 x 501 30.4 -> 15.6, 2047 x 1025 131 -> 56.
+// FP64 is bound by the FP64 pipe (0.5 lanes per clock and SM quarter), FP32 by
+// instruction issue and the FMA pipe.
+#include <math.h>
+
+#include "lbm_internal.h"
+
+namespace {
+
+// ---- values: one double, or a lane pair of floats -------------------------------
+// F2 holds two nodes of a row; its operations are the packed FP32 instructions,
+// each lane rounded like the scalar operation.
+struct F2 {
+  float2 v;
+};
+// The assembler joins a packed product and the packed sum it goes into to one
+// fused operation whatever their rounding modifiers say, so sums are written as
+// fused operations themselves, a * 1 + b with a factor that it cannot know.
+__constant__ float2 c_one = {1.0f, 1.0f}, c_minus = {-1.0f, -1.0f};
+__device__ __forceinline__ F2 operator+(F2 a, F2 b) { return {__ffma2_rn(a.v, c_one, b.v)}; }
+__device__ __forceinline__ F2 operator-(F2 a, F2 b) { return {__ffma2_rn(b.v, c_minus, a.v)}; }
+__device__ __forceinline__ F2 operator-(F2 a) { return F2{make_float2(0.0f, 0.0f)} - a; }
+__device__ __forceinline__ F2 operator*(F2 a, F2 b) { return {__fmul2_rn(a.v, b.v)}; }
+__device__ __forceinline__ F2 operator/(F2 a, F2 b) { return {make_float2(a.v.x / b.v.x, a.v.y / b.v.y)}; }
+__device__ __forceinline__ F2 vfma(F2 a, F2 b, F2 c) { return {__ffma2_rn(a.v, b.v, c.v)}; }
+__device__ __forceinline__ double vfma(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ float vfma(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ F2 root0(F2 a) {
+  return {make_float2(sqrtf(fmaxf(0.0f, a.v.x)), sqrtf(fmaxf(0.0f, a.v.y)))};
+}
+__device__ __forceinline__ double root0(double a) { return sqrt(fmax(0.0, a)); }
+__device__ __forceinline__ float root0(float a) { return sqrtf(fmaxf(0.0f, a)); }
+// a where x <= lim, else b
+__device__ __forceinline__ F2 where_le(F2 x, float lim, F2 a, F2 b) {
+  return {make_float2(x.v.x <= lim ? a.v.x : b.v.x, x.v.y <= lim ? a.v.y : b.v.y)};
+}
+template <class R>
+__device__ __forceinline__ R where_le(R x, R lim, R a, R b) {
+  return x <= lim ? a : b;
+}
+
+template <class V>
+struct Val;
+template <>
+struct Val<double> {
+  typedef double R;
+  static constexpr int N = 1;
+  __device__ __forceinline__ static double bc(double c) { return c; }
+  __device__ __forceinline__ static double lane(double v, int) { return v; }
+  __device__ __forceinline__ static void set(double &v, int, double x) { v = x; }
+};
+template <>
+struct Val<float> {
+  __device__ __forceinline__ static float bc(float c) { return c; }
+};
+template <>
+struct Val<F2> {
+  typedef float R;
+  static constexpr int N = 2;
+  __device__ __forceinline__ static F2 bc(float c) { return {make_float2(c, c)}; }
+  __device__ __forceinline__ static float lane(F2 v, int k) { return k ? v.v.y : v.v.x; }
+  __device__ __forceinline__ static void set(F2 &v, int k, float x) { (k ? v.v.y : v.v.x) = x; }
+};
+
+// Model constants, evaluated on the host in the kernel's precision in the order
+// in which the plain form evaluates them.
+template <class R>
+struct Canon {
+  int nx, ny, walls, kind, n_iter, wetting;
+  int strips, sw;                         // strips of sw columns
+  R b4, Rg, T, a;                         // Carnahan-Starling (b/4)
+  R thv, thm, thl, r1, r2, p1, p2;        // Eq. 11; its pressure at r1 and at r2
+  R A, omA, c2, pre, Gw, ss_dn, ss_up;    // 1 - A, A/2, -kappa/2, sum_a w_a S e_ay at the two walls
+  R s1, s2, s3, s4, s7, h1, h2, h3, h4, h7, h7x2, c15;  // rates, 1 - s/2, 2 (1 - s_7/2), 1.5 s_1
+  R rho_max, ghost_max;
+  R z3h, z3l, z9h, z9l, z36h, z36l, z6h, z6l, z12h, z12l;  // 1/d as a sum of two numbers
+
+  static void split(R d, R *h, R *l) {
+    *h = (R)1 / d;
+    *l = (R)fma(-d, *h, (R)1) / d;  // the remainder is exact
+  }
+  explicit Canon(const lbm_ctx *C) {
+    const lbm_dev_params &P = C->dp;
+    nx = P.nx, ny = P.ny, walls = P.walls, kind = P.eos_kind, n_iter = P.n_iter, wetting = P.wetting;
+    strips = sw = 0;
+    b4 = (R)P.b * (R)0.25, Rg = (R)P.R, T = (R)P.T, a = (R)P.a;
+    thv = (R)P.thv, thm = (R)P.thm, thl = (R)P.thl, r1 = (R)P.r1, r2 = (R)P.r2;
+    p1 = r1 * thv;
+    const R dp = (r2 - r1) * thm;
+    p2 = p1 + dp;
+    A = (R)P.A, omA = (R)1 - A, c2 = A * (R)0.5, pre = (R)P.kappa * ((R)-1 * (R)0.5), Gw = (R)P.Gw;
+    const R w1 = (R)1 / (R)3, w2 = (R)1 / (R)12;
+    ss_up = (w1 + w2) + w2;
+    ss_dn = -ss_up;
+    s1 = (R)P.s[1], s2 = (R)P.s[2], s3 = (R)P.s[3], s4 = (R)P.s[4], s7 = (R)P.s[7];
+    auto half = [](R s) {
+      const R t = (R)0.5 * s;
+      return (R)1 - t;
+    };
+    h1 = half(s1), h2 = half(s2), h3 = half(s3), h4 = half(s4), h7 = half(s7), h7x2 = (R)2 * h7, c15 = (R)1.5 * s1;
+    rho_max = (R)P.rho_max, ghost_max = (R)P.ghost_max;
+    split((R)3, &z3h, &z3l);
+    split((R)9, &z9h, &z9l);
+    split((R)36, &z36h, &z36l);
+    split((R)6, &z6h, &z6l);
+    split((R)12, &z12h, &z12l);
+  }
+};
+
+// x / d for d = 3, 6, 9, 12, 36, correctly rounded, from 1/d = h + l (Brisebarre,
+// Muller, Raina, "Accelerating correctly rounded floating-point division when
+// the divisor is known in advance", IEEE Trans. Computers 53, 2004).  Before its
+// rounding x h + RN(x l) is within 2^-2p (relative; p = 53 or 24) of x / d, and
+// x / d, whose odd denominator part is 3 or 9, is never nearer than 1/18 of a
+// last place to a midpoint between two numbers.
+template <class V, class R>
+__device__ __forceinline__ V div_const(V x, R h, R l) {
+  return vfma(x, Val<V>::bc(h), x * Val<V>::bc(l));
+}
+
+// psi and U of Eqs. 10-11.
+template <class V, class R>
+__device__ __forceinline__ void psi_U(const Canon<R> &m, V rho, V &psi, V &U) {
+  auto bc = [](R c) { return Val<V>::bc(c); };
+  V p;
+  if (m.kind == LBM_EOS_CARNAHAN_STARLING) {
+    const V eta = bc(m.b4) * rho, e2 = eta * eta, one = bc((R)1), om = one - eta;
+    const V num = ((one + eta) + e2) - e2 * eta, den = (om * om) * om;
+    p = (((rho * bc(m.Rg)) * bc(m.T)) * num) / den - (bc(m.a) * rho) * rho;
+  } else {
+    p = where_le(rho, m.r1, rho * bc(m.thv),
+                 where_le(rho, m.r2, bc(m.p1) + (rho - bc(m.r1)) * bc(m.thm),
+                          bc(m.p2) + (rho - bc(m.r2)) * bc(m.thl)));
+  }
+  U = p - div_const(rho, m.z3h, m.z3l);
+  psi = root0(bc((R)-2) * U);
+}
+
+// Ghost psi and U (Eqs. 19-21) from the densities around column x.
+template <class R>
+__device__ __forceinline__ void ghost(const Canon<R> &m, R rim1, R ri1, R rip1, R ri2, R c, R &psi, R &U) {
+  const R a = rip1 - rim1;
+  R g = ri2;
+  if (m.n_iter <= 0) {
+    g = ri2 + c * fabs(a);
+  } else {
+    const R aa = a * a;
+    R d = (R)2 * (ri2 - ri1);
+    for (int k = 0; k < m.n_iter; ++k) {
+      g = ri2 + c * sqrt(aa + d * d);
+      d = ri2 - g;
+    }
+  }
+  g = fmin(fmax(g, (R)0), m.ghost_max);
+  psi = U = (R)0;
+  if (g < m.rho_max) psi_U(m, g, psi, U);
+}
+
+// The neighbour values of a window: psi, psi^2, w psi, w U.
+template <class V>
+struct Nb {
+  V p, p2, tp, tu;
+};
+
+constexpr int kH = 32;       // lanes of a row; a lane pair is columns t, t + 32
+constexpr int kWP = kH + 4;  // window entries -2 .. kH + 1 at index i + 2
+
+template <class V, int R>
+struct Window;
+template <int R>
+struct Window<F2, R> {
+  F2 p[R + 2][kWP], u[R + 2][kWP];
+  __device__ __forceinline__ void put1(int row, int i, int lane, float psi, float U) {
+    Val<F2>::set(p[row][i], lane, psi);
+    Val<F2>::set(u[row][i], lane, U);
+  }
+  __device__ __forceinline__ void put(int row, int c, float psi, float U) {
+    if (c <= kH + 1) put1(row, c + 2, 0, psi, U);
+    if (c >= kH - 2) put1(row, c - kH + 2, 1, psi, U);
+  }
+  template <bool DIAG>
+  __device__ __forceinline__ Nb<F2> at(int row, int i) const {
+    const F2 w = Val<F2>::bc(DIAG ? 1.0f / 12.0f : 1.0f / 3.0f), a = p[row][i];
+    return {a, a * a, w * a, w * u[row][i]};
+  }
+};
+template <int R>
+struct Window<double, R> {
+  double p[R + 2][kWP], p2[R + 2][kWP], p1w[R + 2][kWP], p2w[R + 2][kWP], u1w[R + 2][kWP], u2w[R + 2][kWP];
+  __device__ __forceinline__ void put(int row, int c, double psi, double U) {
+    const int i = c + 2;
+    p[row][i] = psi;
+    p2[row][i] = psi * psi;
+    p1w[row][i] = (1.0 / 3.0) * psi;
+    p2w[row][i] = (1.0 / 12.0) * psi;
+    u1w[row][i] = (1.0 / 3.0) * U;
+    u2w[row][i] = (1.0 / 12.0) * U;
+  }
+  template <bool DIAG>
+  __device__ __forceinline__ Nb<double> at(int row, int i) const {
+    return {p[row][i], p2[row][i], DIAG ? p2w[row][i] : p1w[row][i], DIAG ? u2w[row][i] : u1w[row][i]};
+  }
+};
+
+// Force (Eq. 9, + Eq. 14 with ss = sum_a w_a S e_ay), Eq. 17 tensor and MRT
+// collision of the node(s) at window row `row`, entry i; f: populations, rho:
+// density, fs: post-collision populations.
+template <class V, class R, class W>
+__device__ __forceinline__ void collide(const Canon<R> &m, const W &win, int row, int i, const V (&f)[9], V rho,
+                                        R ss, V (&fs)[9]) {
+  auto bc = [](R c) { return Val<V>::bc(c); };
+  const V w1 = bc((R)1 / (R)3), w2 = bc((R)1 / (R)12);
+  V Fx, Fy, Qxx, Qyy, Qxy;
+  {
+    const Nb<V> n0 = win.template at<false>(row, i);
+    V spx, spy, sUx, sUy, xx1, yy1, xy1, xx2, yy2, xy2;
+    auto t1 = [&](const Nb<V> &n, V w) { return w * (n.p - n0.p); };
+    auto t2 = [&](const Nb<V> &n, V w) { return w * (n.p2 - n0.p2); };
+    Nb<V> n = win.template at<false>(row, i + 1);  // e1
+    spx = n.tp, sUx = n.tu, xx1 = t1(n, w1), xx2 = t2(n, w1);
+    n = win.template at<false>(row + 1, i);  // e2
+    spy = n.tp, sUy = n.tu, yy1 = t1(n, w1), yy2 = t2(n, w1);
+    n = win.template at<false>(row, i - 1);  // e3
+    spx = spx - n.tp, sUx = sUx - n.tu, xx1 = xx1 + t1(n, w1), xx2 = xx2 + t2(n, w1);
+    n = win.template at<false>(row - 1, i);  // e4
+    spy = spy - n.tp, sUy = sUy - n.tu, yy1 = yy1 + t1(n, w1), yy2 = yy2 + t2(n, w1);
+    n = win.template at<true>(row + 1, i + 1);  // e5
+    V a = t1(n, w2), b = t2(n, w2);
+    spx = spx + n.tp, sUx = sUx + n.tu, spy = spy + n.tp, sUy = sUy + n.tu;
+    xx1 = xx1 + a, xx2 = xx2 + b, yy1 = yy1 + a, yy2 = yy2 + b, xy1 = a, xy2 = b;
+    n = win.template at<true>(row + 1, i - 1);  // e6
+    a = t1(n, w2), b = t2(n, w2);
+    spx = spx - n.tp, sUx = sUx - n.tu, spy = spy + n.tp, sUy = sUy + n.tu;
+    xx1 = xx1 + a, xx2 = xx2 + b, yy1 = yy1 + a, yy2 = yy2 + b, xy1 = xy1 - a, xy2 = xy2 - b;
+    n = win.template at<true>(row - 1, i - 1);  // e7
+    a = t1(n, w2), b = t2(n, w2);
+    spx = spx - n.tp, sUx = sUx - n.tu, spy = spy - n.tp, sUy = sUy - n.tu;
+    xx1 = xx1 + a, xx2 = xx2 + b, yy1 = yy1 + a, yy2 = yy2 + b, xy1 = xy1 + a, xy2 = xy2 + b;
+    n = win.template at<true>(row - 1, i + 1);  // e8
+    a = t1(n, w2), b = t2(n, w2);
+    spx = spx + n.tp, sUx = sUx + n.tu, spy = spy - n.tp, sUy = sUy - n.tu;
+    xx1 = xx1 + a, xx2 = xx2 + b, yy1 = yy1 + a, yy2 = yy2 + b, xy1 = xy1 - a, xy2 = xy2 - b;
+    const V c1 = bc(m.omA) * n0.p, c2 = bc(m.c2), pre = bc(m.pre);
+    Fx = c1 * spx - bc(m.A) * sUx;
+    Fy = c1 * spy - bc(m.A) * sUy;
+    if (m.wetting == LBM_WET_MARTYS_CHEN) Fy = Fy - (bc(m.Gw) * n0.p) * bc(ss);
+    Qxx = pre * (c1 * xx1 + c2 * xx2);
+    Qyy = pre * (c1 * yy1 + c2 * yy2);
+    Qxy = pre * (c1 * xy1 + c2 * xy2);
+  }
+  const V half = bc((R)0.5), two = bc((R)2), m2 = bc((R)-2), four = bc((R)4), m4 = bc((R)-4), quarter = bc((R)0.25);
+  // moments (rho is the first), left to right in f_0 .. f_8
+  const V d13 = f[1] - f[3], d24 = f[2] - f[4];
+  V me = vfma(m4, f[0], -f[1]);
+  me = ((me - f[2]) - f[3]) - f[4];
+  me = vfma(two, f[8], vfma(two, f[7], vfma(two, f[6], vfma(two, f[5], me))));
+  V mp = ((vfma(two, f[0], -f[1]) - f[2]) - f[3]) - f[4];  // half of 4 f_0 - 2 f_1 - ...
+  mp = ((vfma(two, mp, f[5]) + f[6]) + f[7]) + f[8];
+  const V jx = (((d13 + f[5]) - f[6]) - f[7]) + f[8];
+  const V jy = (((d24 + f[5]) + f[6]) - f[7]) - f[8];
+  const V qx = ((vfma(m2, d13, f[5]) - f[6]) - f[7]) + f[8];
+  const V qy = ((vfma(m2, d24, f[5]) + f[6]) - f[7]) - f[8];
+  const V nn = ((f[1] - f[2]) + f[3]) - f[4];
+  const V no = ((f[5] - f[6]) + f[7]) - f[8];
+  const V vx = vfma(half, Fx, jx) / rho, vy = vfma(half, Fy, jy) / rho;
+  const V vx2 = vx * vx, vy2 = vy * vy, v3 = bc((R)3) * (vx2 + vy2);
+  const V vxF = vx * Fx, vyF = vy * Fy, S1 = bc((R)6) * (vxF + vyF);
+  const V rvx = rho * vx, rvy = rho * vy;
+  // m - s (m - meq) + (1 - s/2) S + C, divided by N
+  V r0 = div_const(rho, m.z9h, m.z9l);
+  V r1 = ((me - bc(m.s1) * (me - rho * (v3 - two))) + bc(m.h1) * S1) + bc(m.c15) * (Qxx + Qyy);
+  V r2 = (mp - bc(m.s2) * (mp - rho * (bc((R)1) - v3))) - bc(m.h2) * S1;
+  V r3 = (jx - bc(m.s3) * (jx - rvx)) + bc(m.h3) * Fx;
+  V r4 = (qx - bc(m.s4) * (qx + rvx)) - bc(m.h4) * Fx;
+  V r5 = (jy - bc(m.s3) * (jy - rvy)) + bc(m.h3) * Fy;
+  V r6 = (qy - bc(m.s4) * (qy + rvy)) - bc(m.h4) * Fy;
+  V r7 = ((nn - bc(m.s7) * (nn - rho * (vx2 - vy2))) + bc(m.h7x2) * (vxF - vyF)) - bc(m.s7) * (Qxx - Qyy);
+  V r8 = ((no - bc(m.s7) * (no - rho * (vx * vy))) + bc(m.h7) * (vx * Fy + vy * Fx)) - bc(m.s7) * Qxy;
+  r1 = div_const(r1, m.z36h, m.z36l);
+  r2 = div_const(r2, m.z36h, m.z36l);
+  r3 = div_const(r3, m.z6h, m.z6l);
+  r4 = div_const(r4, m.z12h, m.z12l);
+  r5 = div_const(r5, m.z6h, m.z6l);
+  r6 = div_const(r6, m.z12h, m.z12l);
+  // f* = M^T r; r7 and r8 still carry their factor 4
+  const V mq = bc((R)-0.25);
+  fs[0] = vfma(four, r2, vfma(m4, r1, r0));
+  const V ax = vfma(m2, r2, r0 - r1);
+  fs[1] = vfma(quarter, r7, vfma(m2, r4, ax + r3));
+  fs[2] = vfma(mq, r7, vfma(m2, r6, ax + r5));
+  fs[3] = vfma(quarter, r7, vfma(two, r4, ax - r3));
+  fs[4] = vfma(mq, r7, vfma(two, r6, ax - r5));
+  const V dg = vfma(two, r1, r0) + r2, dp = (dg + r3) + r4, dm = (dg - r3) - r4;
+  fs[5] = vfma(quarter, r8, (dp + r5) + r6);
+  fs[6] = vfma(mq, r8, (dm + r5) + r6);
+  fs[7] = vfma(quarter, r8, (dm - r5) - r6);
+  fs[8] = vfma(mq, r8, (dp - r5) - r6);
+}
+
+// Tile of m.sw columns x R rows per CTA of R + 3 warps: warps 0 .. R + 1 each
+// load one row (the tile's, the one above, the one below), the last one the
+// columns beside the tile.  Window row w holds row y0 - 1 + w.
+template <class V, int R>
+__global__ void __launch_bounds__((R + 3) * 32)
+    k_canon(Canon<typename Val<V>::R> m, const typename Val<V>::R *__restrict__ fin,
+            typename Val<V>::R *__restrict__ fout, const double *__restrict__ coef, int *flag) {
+  typedef typename Val<V>::R real;
+  constexpr int N = Val<V>::N;
+  static_assert(2 * (R + 2) + 4 <= 32, "one warp loads the columns beside the tile");
+  __shared__ Window<V, R> win;
+  __shared__ real wrho[R + 2][N * kH + 4];  // column c at c + 2
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int band = (int)(blockIdx.x / (unsigned)m.strips);
+  const int x0 = ((int)blockIdx.x - band * m.strips) * m.sw, wr = min(m.sw, m.nx - x0);
+  const int first = m.walls ? 1 : 0, last = m.walls ? m.ny - 1 : m.ny;  // fluid rows [first, last)
+  const int y0 = first + band * R;
+  const int nr = min(R, last - y0);
+  const size_t n = (size_t)m.nx * m.ny;
+  const bool geo = m.walls && m.wetting != LBM_WET_MARTYS_CHEN;
+  const bool low = geo && y0 == 1, high = geo && y0 + nr == m.ny - 1;  // the tile touches a wall with a ghost row
+
+  int w = warp, hc = 0;  // window row; column of a thread of the last warp
+  bool on = true;
+  if (warp == R + 2) {
+    const int k = lane - 2 * (R + 2);
+    w = lane >> 1;
+    hc = lane & 1 ? wr : -1;
+    if (k >= 0) {  // densities two columns out, which the ghost values one column out read
+      w = k >> 1 ? nr : 1;
+      hc = k & 1 ? wr + 1 : -2;
+      on = k < 4 && (k >> 1 ? high : low);
+    }
+  }
+  on = on && w <= nr + 1;
+  const int v = y0 - 1 + w;
+  const bool solid = m.walls && (v == 0 || v == m.ny - 1);
+  const int y = v < 0 ? v + m.ny : (v >= m.ny ? v - m.ny : v);
+  const bool row_warp = warp < R + 2;
+  bool act[N];
+#pragma unroll
+  for (int j = 0; j < N; ++j) act[j] = lane + j * kH < wr;  // a later one implies the earlier
+  int gx = x0 + hc;
+  gx = gx < 0 ? gx + m.nx : (gx >= m.nx ? gx - m.nx : gx);
+
+  // the wall coefficients of a ghost row, loaded before the densities it waits for
+  double kc[N];
+  if (on && solid && geo) {
+    const double *c = coef + (m.n_iter > 0 ? 0 : 2 * m.nx) + (v != 0 ? m.nx : 0);
+#pragma unroll
+    for (int j = 0; j < N; ++j)
+      if (row_warp ? act[j] : j == 0) kc[j] = c[row_warp ? x0 + lane + j * kH : gx];
+  }
+  bool bad = false;
+  V f[9], r = Val<V>::bc((real)0);
+  if (on && (row_warp ? act[0] : true)) {
+    if (!solid) {
+      const real *q = fin + (size_t)y * m.nx + (row_warp ? x0 + lane : gx);
+#pragma unroll
+      for (int a = 0; a < 9; ++a) {
+        f[a] = Val<V>::bc(q[a * n]);
+        if (N == 2 && row_warp && act[N - 1]) Val<V>::set(f[a], 1, q[a * n + kH]);
+      }
+      r = f[0];
+#pragma unroll
+      for (int a = 1; a < 9; ++a) r = r + f[a];
+      V psi, U;
+      psi_U(m, r, psi, U);
+#pragma unroll
+      for (int j = 0; j < N; ++j) {
+        if (row_warp ? act[j] : j == 0) {
+          const int c = row_warp ? lane + j * kH : hc;
+          const real rj = Val<V>::lane(r, j);
+          bad |= !(rj > (real)0) || rj > m.rho_max;
+          wrho[w][c + 2] = rj;
+          win.put(w, c, Val<V>::lane(psi, j), Val<V>::lane(U, j));
+        }
+      }
+    } else if (!geo) {  // Martys-Chen: psi = U = 0 on the solid rows
+#pragma unroll
+      for (int j = 0; j < N; ++j)
+        if (row_warp ? act[j] : j == 0) win.put(w, row_warp ? lane + j * kH : hc, (real)0, (real)0);
+    }
+  }
+  __syncthreads();
+  if (low || high) {  // uniform in the CTA
+    if (on && solid) {
+      // v == 0 from window rows 1, 2; v == ny - 1 from the two rows below it
+      const real *q1 = wrho[v != 0 ? w - 1 : 1], *q2 = wrho[v != 0 ? w - 2 : 2];
+#pragma unroll
+      for (int j = 0; j < N; ++j) {
+        if (row_warp ? act[j] : j == 0) {
+          const int c = row_warp ? lane + j * kH : hc;
+          real psi, U;
+          ghost(m, q1[c + 1], q1[c + 2], q1[c + 3], q2[c + 2], (real)kc[j], psi, U);
+          win.put(w, c, psi, U);
+        }
+      }
+    }
+    __syncthreads();
+  }
+  if (__any_sync(0xffffffffu, bad) && lane == 0 && *(volatile int *)flag == 0) atomicOr(flag, 1);
+  if (warp < 1 || warp > nr || !act[0]) return;
+
+  const bool dn = m.walls && y == 1, up = m.walls && y == m.ny - 2;
+  V fs[9];
+  collide(m, win, w, lane + 2, f, r, dn ? m.ss_dn : (up ? m.ss_up : (real)0), fs);
+  // streaming with half-way bounce-back
+  const size_t ry = (size_t)y * m.nx, rd = (size_t)(y == 0 ? m.ny - 1 : y - 1) * m.nx,
+               ru = (size_t)(y == m.ny - 1 ? 0 : y + 1) * m.nx;
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    if (!act[j]) break;
+    const int x = x0 + lane + j * kH, xm = x == 0 ? m.nx - 1 : x - 1, xp = x == m.nx - 1 ? 0 : x + 1;
+    auto g = [&](int a) { return Val<V>::lane(fs[a], j); };
+    real *o = fout;
+    o[ry + x] = g(0);
+    o[n + ry + xp] = g(1);
+    o[3 * n + ry + xm] = g(3);
+    o[(up ? 4 * n + ry : 2 * n + ru) + x] = g(2);
+    o[up ? 7 * n + ry + x : 5 * n + ru + xp] = g(5);
+    o[up ? 8 * n + ry + x : 6 * n + ru + xm] = g(6);
+    o[(dn ? 2 * n + ry : 4 * n + rd) + x] = g(4);
+    o[dn ? 5 * n + ry + x : 7 * n + rd + xm] = g(7);
+    o[dn ? 6 * n + ry + x : 8 * n + rd + xp] = g(8);
+  }
+}
+
+template <class V, int R>
+cudaError_t launch(const lbm_ctx *C, const void *src, void *dst) {
+  typedef typename Val<V>::R real;
+  Canon<real> m(C);
+  const int W = Val<V>::N * kH;
+  m.strips = (C->nx + W - 1) / W;
+  m.sw = Val<V>::N == 1 ? (C->nx + m.strips - 1) / m.strips : W;
+  const int nrows = C->walls ? C->ny - 2 : C->ny;
+  const unsigned grid = (unsigned)m.strips * (unsigned)((nrows + R - 1) / R);
+  k_canon<V, R><<<grid, (R + 3) * 32, 0, C->stream>>>(m, (const real *)src, (real *)dst, C->d_coef, C->d_flag);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+// Rows per tile.  FP32: 4 (2047 x 1025: 56 us per step, with 2 rows 63, with 6
+// rows 62).  FP64: the FP64 pipe of an SM quarter takes 64 cycles for an
+// operation of a warp, so small domains take as long as one warp's chain (100 x
+// 60: 16.7 us) and want few rows per CTA; larger ones are bound by the pipe and
+// want few repeated rows: 2 / 8 rows, 200 x 100 27.7 / 30.3, 400 x 200 79.8 /
+// 79.1, 800 x 400 253 / 230 us.
+cudaError_t lbm_canon_step(const lbm_ctx *C, const void *src, void *dst, unsigned long long *launches) {
+  ++*launches;
+  if (C->precision == 32) return launch<F2, 4>(C, src, dst);
+  return (long long)C->nx * C->ny < 80000 ? launch<double, 2>(C, src, dst) : launch<double, 8>(C, src, dst);
+}

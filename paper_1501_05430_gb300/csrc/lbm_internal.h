@@ -63,7 +63,7 @@ struct lbm_ctx {
   double *d_rho64;       // nx*ny, measurement density
   cudaStream_t xfer;     // lbm_get_rho: copy stream and its chunk events (lazy; NULL until first needed)
   cudaEvent_t xfer_ev[8];
-  void *d_fields;        // 3*nx*ny reals: rho, psi, U (reference kernels)
+  void *d_fields;        // 3*nx*ny reals: rho, psi, U (getters, adjoint; lazy)
   double *d_aux;         // 7*nx*ny doubles for lbm_get_u / lbm_get_fields (lazy)
   double *d_red;         // reduction partials
   double *d_res;         // small results
@@ -85,12 +85,10 @@ struct lbm_ctx {
   cudaGraphExec_t step_graph[2][kMaxGraphs];
 };
 
-// ---- lbm_ref.cu: unfused kernels in the canonical evaluation order --------
+// ---- lbm_ref.cu: fields and initial states in the canonical order -----------
 // All launchers return the cudaError_t of the launch and add the number of
 // kernels launched to *launches.
 cudaError_t lbm_ref_fields(const lbm_ctx *C, const void *f, void *fields, unsigned long long *launches);
-cudaError_t lbm_ref_collide(const lbm_ctx *C, const void *fin, void *fout, const void *fields,
-                            unsigned long long *launches);
 cudaError_t lbm_ref_macro(const lbm_ctx *C, const void *f, const void *fields, double *out7,
                           unsigned long long *launches);
 // f := f_eq(rho, 0) from device or mapped host densities; with bad != NULL,
@@ -99,6 +97,9 @@ cudaError_t lbm_ref_macro(const lbm_ctx *C, const void *f, const void *fields, d
 cudaError_t lbm_ref_set_rho(const lbm_ctx *C, const double *rho, void *f, int *bad, unsigned long long *launches);
 cudaError_t lbm_ref_droplets(const lbm_ctx *C, int n, const double *drop, double width, double *rho,
                              unsigned long long *launches);
+
+// ---- lbm_canon.cu: one step in the canonical evaluation order ---------------
+cudaError_t lbm_canon_step(const lbm_ctx *C, const void *src, void *dst, unsigned long long *launches);
 
 // ---- lbm_fused.cu: single-pass FP32 step ------------------------------------
 int lbm_fused_plan(lbm_ctx *C);  // sets fused_ok, tile_*, tensor maps

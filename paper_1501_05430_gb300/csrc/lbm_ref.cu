@@ -1,14 +1,11 @@
-// lbm_ref.cu -- unfused reference kernels of the pseudo-potential D2Q9 step,
-// written in the canonical evaluation order (sums left to right in index
-// order, integer moment coefficients applied as multiplications) and compiled
-// with -fmad=false, so that the double instantiation is bit-identical to any
-// IEEE FP64 evaluation of the step in the same order.
-//
-// One step = lbm_ref_fields (rho, psi, U; Eqs. 1, 10, 11 -- and on the solid
-// rows the ghost values of Eqs. 19-21 or the Martys-Chen zero potential) ->
-// lbm_ref_collide (Eq. 9 [+ Eq. 14], Eqs. 16-17, collision Eqs. 4-6 and 15,
-// streaming of Eq. 1 with half-way bounce-back).  The fused FP32 kernel (lbm_fused.cu) computes the
-// same step in one pass; these kernels also serve the macroscopic getters.
+// lbm_ref.cu -- kernels of the pseudo-potential D2Q9 model in the canonical
+// evaluation order (sums left to right in index order, integer moment
+// coefficients applied as multiplications), compiled with -fmad=false, so that
+// the double instantiation is bit-identical to any IEEE FP64 evaluation in the
+// same order: the fields of a state (rho, psi, U; Eqs. 1, 10, 11, with the
+// ghost values of Eqs. 19-21 or the Martys-Chen zero potential on the solid
+// rows), the macroscopic getters and the initial states.  The step in this
+// order is lbm_canon.cu.
 #include <math.h>
 #include <stdint.h>
 
@@ -78,31 +75,6 @@ __global__ void k_fields(Mdl<R> m, const R *__restrict__ f, const double *__rest
   fields[n + i] = psi;
   fields[2 * n + i] = U;
   if (!(r > (R)0) || r > m.rho_max) atomicOr(flag, 1);
-}
-
-template <typename R>
-__global__ void k_collide(Mdl<R> m, const R *__restrict__ fin, R *__restrict__ fout,
-                          const R *__restrict__ fields) {
-  size_t n = (size_t)m.nx * m.ny;
-  size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  int y = (int)(i / m.nx), x = (int)(i - (size_t)y * m.nx);
-  if (m.solid_row(y)) return;
-  R Fx, Fy, Qxx, Qyy, Qxy;
-  force_Q(m, fields, y, x, Fx, Fy, Qxx, Qyy, Qxy);
-  R fl[9], fs[9];
-#pragma unroll
-  for (int a = 0; a < 9; ++a) fl[a] = fin[a * n + i];
-  collide(m, fl, fields[i], Fx, Fy, Qxx, Qyy, Qxy, fs);
-#pragma unroll
-  for (int a = 0; a < 9; ++a) {
-    int yt = m.wy(y + EY(a));
-    if (m.solid_row(yt)) {
-      fout[OPP(a) * n + i] = fs[a];
-    } else {
-      fout[a * n + (size_t)yt * m.nx + m.wx(x + EX(a))] = fs[a];
-    }
-  }
 }
 
 // Macroscopic outputs at every node: out7 = {ux, uy, Fx, Fy, Qxx, Qyy, Qxy}
@@ -243,19 +215,6 @@ cudaError_t lbm_ref_fields(const lbm_ctx *C, const void *f, void *fields, unsign
   else
     k_fields<float><<<nblk(n, 256), 256, 0, C->stream>>>(Mdl<float>(C->dp), (const float *)f, C->d_coef, (float *)fields,
                                                          C->d_flag);
-  ++*launches;
-  return cudaGetLastError();
-}
-
-cudaError_t lbm_ref_collide(const lbm_ctx *C, const void *fin, void *fout, const void *fields,
-                            unsigned long long *launches) {
-  size_t n = (size_t)C->nx * C->ny;
-  if (C->precision == 64)
-    k_collide<double><<<nblk(n, 128), 128, 0, C->stream>>>(Mdl<double>(C->dp), (const double *)fin, (double *)fout,
-                                                           (const double *)fields);
-  else
-    k_collide<float><<<nblk(n, 128), 128, 0, C->stream>>>(Mdl<float>(C->dp), (const float *)fin, (float *)fout,
-                                                          (const float *)fields);
   ++*launches;
   return cudaGetLastError();
 }

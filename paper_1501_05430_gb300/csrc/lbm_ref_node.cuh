@@ -1,8 +1,8 @@
-// lbm_ref_node.cuh -- per-node arithmetic of the canonical-order reference
-// step (model constants, EOS, Eq. 9 / Eq. 17 stencil, MRT collision), shared
-// by the reference kernels (lbm_ref.cu) and the adjoint kernels
-// (lbm_adjoint.cu), which recompute the forward quantities of a step.  Both
-// translation units are compiled with -fmad=false.
+// lbm_ref_node.cuh -- per-node arithmetic in the canonical order (model
+// constants, EOS, Eq. 9 / Eq. 17 stencil), shared by the field kernels
+// (lbm_ref.cu) and the adjoint kernels (lbm_adjoint.cu), which recompute the
+// forward quantities of a step.  Both translation units are compiled with
+// -fmad=false.
 #pragma once
 
 #include <math.h>
@@ -134,62 +134,6 @@ __device__ void force_Q(const Mdl<R> &m, const R *__restrict__ fields, int y, in
   Qxx = pre * ((c1 * qxx1) + (c2 * qxx2));
   Qyy = pre * ((c1 * qyy1) + (c2 * qyy2));
   Qxy = pre * ((c1 * qxy1) + (c2 * qxy2));
-}
-
-// MRT collision with forcing (Eqs. 4, 6, 15 with the Eq. 16 source).
-template <typename R>
-__device__ void collide(const Mdl<R> &m, const R *f, R rho, R Fx, R Fy, R Qxx, R Qyy, R Qxy, R *fs) {
-  R mm[9];
-#pragma unroll
-  for (int k = 0; k < 9; ++k) {
-    R acc = (R)0;
-#pragma unroll
-    for (int a = 0; a < 9; ++a)
-      if (MC(k, a) != 0.0) acc = acc + (R)MC(k, a) * f[a];
-    mm[k] = acc;
-  }
-  R vx = (mm[3] + (R)0.5 * Fx) / rho;
-  R vy = (mm[5] + (R)0.5 * Fy) / rho;
-  R v2 = vx * vx + vy * vy;
-  R meq[9], S[9], C[9];
-  meq[0] = rho;
-  meq[1] = rho * ((R)-2 + (R)3 * v2);
-  meq[2] = rho * ((R)1 - (R)3 * v2);
-  meq[3] = rho * vx;
-  meq[4] = -(rho * vx);
-  meq[5] = rho * vy;
-  meq[6] = -(rho * vy);
-  meq[7] = rho * (vx * vx - vy * vy);
-  meq[8] = rho * (vx * vy);
-  R vF = vx * Fx + vy * Fy;
-  S[0] = 0;
-  S[1] = (R)6 * vF;
-  S[2] = -((R)6 * vF);
-  S[3] = Fx;
-  S[4] = -Fx;
-  S[5] = Fy;
-  S[6] = -Fy;
-  S[7] = (R)2 * (vx * Fx - vy * Fy);
-  S[8] = vx * Fy + vy * Fx;
-#pragma unroll
-  for (int k = 0; k < 9; ++k) C[k] = 0;
-  C[1] = ((R)1.5 * m.s[1]) * (Qxx + Qyy);
-  C[7] = -(m.s[7] * (Qxx - Qyy));
-  C[8] = -(m.s[8] * Qxy);
-  R r[9];
-#pragma unroll
-  for (int k = 0; k < 9; ++k) {
-    R ms = ((mm[k] - m.s[k] * (mm[k] - meq[k])) + ((R)1 - (R)0.5 * m.s[k]) * S[k]) + C[k];
-    r[k] = ms / (R)NRM(k);
-  }
-#pragma unroll
-  for (int a = 0; a < 9; ++a) {
-    R acc = (R)0;
-#pragma unroll
-    for (int k = 0; k < 9; ++k)
-      if (MC(k, a) != 0.0) acc = acc + (R)MC(k, a) * r[k];
-    fs[a] = acc;
-  }
 }
 
 }  // namespace lbm_ref
