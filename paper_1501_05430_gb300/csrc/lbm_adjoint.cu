@@ -7,7 +7,7 @@
 // bounce-back.  Given lam = dL/df^{n+1}, one reverse step computes
 // dL/df^n and adds this step's part of dL/dtheta (per wall node, through
 // c = sin(pi/2 - theta) of Eq. 21 or cot of Eq. 19) and dL/dT (through the
-// EOS), in four kernels:
+// EOS), in FP32 in one kernel (k_adj_step), in FP64 in four (after the fields):
 //
 //   k_adj_collide  per fluid node: pull lam back through the streaming
 //                  (bounce-back included), recompute F, Q and the collision,
@@ -51,10 +51,10 @@ struct lbm_tape {
   std::vector<void *> ckpt;      // state at the start of each segment
   void *seg;                     // (every + 1) states of the segment being reversed
   void *lam[2];                  // adjoint fields
-  void *aux;                     // 5 planes: dL/dFx, dL/dFy, dL/dQxx, dL/dQyy, dL/dQxy
-  void *rhob;                    // dL/drho per node (ghost rows: of the ghost density)
+  void *aux;                     // FP64: 5 planes: dL/dFx, dL/dFy, dL/dQxx, dL/dQyy, dL/dQxy
+  void *rhob;                    // FP64: dL/drho per node (ghost rows: of the ghost density)
   double *tacc;                  // per-node dL/dT, accumulated over the steps
-  double *gpart;                 // [2 walls][4][nx]: ghost-rule partials
+  double *gpart;                 // FP64: [2 walls][4][nx]: ghost-rule partials
   double *dtheta;                // [2][nx]
   double *red;                   // reduction output
   // captured graphs (contexts with a non-NULL stream): the recorded forward of
@@ -88,31 +88,19 @@ __device__ void eos_derivs(const Mdl<R> &m, R rho, R &dp_drho, R &dp_dT) {
   }
 }
 
+// Transpose of the collision at one fluid node: from ls = dL/df* (pulled back
+// through the streaming), the populations f, rho and F to the part of dL/df that
+// passes through the moments (cl), and aux = dL/d(Fx, Fy, Qxx, Qyy, Qxy).
 template <typename R>
-__global__ void k_adj_collide(Mdl<R> m, const R *__restrict__ f, const R *__restrict__ fields,
-                              const R *__restrict__ lam_in, R *__restrict__ lam_out, R *__restrict__ aux) {
-  size_t n = (size_t)m.nx * m.ny;
-  size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  int y = (int)(i / m.nx), x = (int)(i - (size_t)y * m.nx);
-  if (m.solid_row(y)) return;
-  // adjoint of the post-collision populations (transpose of the push streaming)
-  R ls[9];
-#pragma unroll
-  for (int a = 0; a < 9; ++a) {
-    int yt = m.wy(y + EY(a));
-    ls[a] = m.solid_row(yt) ? lam_in[OPP(a) * n + i] : lam_in[a * n + (size_t)yt * m.nx + m.wx(x + EX(a))];
-  }
-  R Fx, Fy, Qxx, Qyy, Qxy;
-  force_Q(m, fields, y, x, Fx, Fy, Qxx, Qyy, Qxy);
-  const R rho = fields[i];
+__device__ __forceinline__ void adj_collide(const Mdl<R> &m, const R (&f)[9], const R (&ls)[9], R rho, R Fx, R Fy,
+                                            R (&cl)[9], R (&aux)[5]) {
   R mm[9];
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
     R acc = (R)0;
 #pragma unroll
     for (int a = 0; a < 9; ++a)
-      if (MC(k, a) != 0.0) acc = acc + (R)MC(k, a) * f[a * n + i];
+      if (MC(k, a) != 0.0) acc = acc + (R)MC(k, a) * f[a];
     mm[k] = acc;
   }
   const R vx = (mm[3] + (R)0.5 * Fx) / rho, vy = (mm[5] + (R)0.5 * Fy) / rho;
@@ -164,27 +152,25 @@ __global__ void k_adj_collide(Mdl<R> m, const R *__restrict__ f, const R *__rest
 #pragma unroll
     for (int k = 0; k < 9; ++k)
       if (MC(k, a) != 0.0) acc = acc + (R)MC(k, a) * mb[k];
-    lam_out[a * n + i] = acc;
+    cl[a] = acc;
   }
-  aux[i] = Fxb;
-  aux[n + i] = Fyb;
-  aux[2 * n + i] = Qxxb;
-  aux[3 * n + i] = Qyyb;
-  aux[4 * n + i] = Qxyb;
+  aux[0] = Fxb;
+  aux[1] = Fyb;
+  aux[2] = Qxxb;
+  aux[3] = Qyyb;
+  aux[4] = Qxyb;
 }
 
-template <typename R>
-__global__ void k_adj_psi(Mdl<R> m, const R *__restrict__ fields, const R *__restrict__ aux,
-                          R *__restrict__ rhob_out, double *__restrict__ tacc) {
-  size_t n = (size_t)m.nx * m.ny;
-  size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  int y = (int)(i / m.nx), x = (int)(i - (size_t)y * m.nx);
-  const R *psi = fields + n, *U = fields + 2 * n;
+// dL/drho and dL/dT of node (row y) through psi and U, gathered from the aux of
+// the fluid nodes whose stencils hold it; ax(ex, ey) is the index of a neighbour
+// in the planes aux + k * an, nb(ex, ey) its index in psi.  rho: its density.
+template <typename R, typename Nb, typename Ax>
+__device__ __forceinline__ void adj_psi(const Mdl<R> &m, const R *__restrict__ psi, const R *__restrict__ aux,
+                                        size_t an, int y, R rho, Nb nb, Ax ax, R &rb, double &tb) {
   const R G = (R)-1;
   const R pre = m.kappa * (G * (R)0.5);
   const R omA = (R)1 - m.A;
-  const R psi_p = psi[i];
+  const R psi_p = psi[nb(0, 0)];
   R pb = (R)0, ub = (R)0;
   // fluid nodes q = p - e_a hold p in their stencil in direction a:
   //   dF(q)/dpsi_p = (1-A) psi_q w_a e_a,  dF(q)/dU_p = -A w_a e_a,
@@ -193,14 +179,12 @@ __global__ void k_adj_psi(Mdl<R> m, const R *__restrict__ fields, const R *__res
   for (int a = 1; a < 9; ++a) {
     int yq = y - EY(a);
     if (m.walls && (yq < 0 || yq >= m.ny)) continue;
-    yq = m.wy(yq);
-    if (m.solid_row(yq)) continue;
-    size_t j = (size_t)yq * m.nx + m.wx(x - EX(a));
+    if (m.solid_row(m.wy(yq))) continue;
+    const R *q = aux + ax(-EX(a), -EY(a));
     const R w = wgt<R>(a);
-    const R eF = aux[j] * (R)EX(a) + aux[n + j] * (R)EY(a);
-    const R eQ = aux[2 * n + j] * (R)(EX(a) * EX(a)) + aux[3 * n + j] * (R)(EY(a) * EY(a)) +
-                 aux[4 * n + j] * (R)(EX(a) * EY(a));
-    const R psi_q = psi[j];
+    const R eF = q[0] * (R)EX(a) + q[an] * (R)EY(a);
+    const R eQ = q[2 * an] * (R)(EX(a) * EX(a)) + q[3 * an] * (R)(EY(a) * EY(a)) + q[4 * an] * (R)(EX(a) * EY(a));
+    const R psi_q = psi[nb(-EX(a), -EY(a))];
     pb = pb + (omA * psi_q) * w * eF + pre * w * eQ * (omA * psi_q + m.A * psi_p);
     ub = ub - m.A * w * eF;
   }
@@ -211,11 +195,9 @@ __global__ void k_adj_psi(Mdl<R> m, const R *__restrict__ fields, const R *__res
     R spx = 0, spy = 0, ssx = 0, ssy = 0, qxx1 = 0, qyy1 = 0, qxy1 = 0;
 #pragma unroll
     for (int a = 1; a < 9; ++a) {
-      int yn = m.wy(y + EY(a)), xn = m.wx(x + EX(a));
-      size_t j = (size_t)yn * m.nx + xn;
       const R w = wgt<R>(a);
-      const R pn = psi[j];
-      const R sol = m.solid_row(yn) ? (R)1 : (R)0;
+      const R pn = psi[nb(EX(a), EY(a))];
+      const R sol = m.solid_row(m.wy(y + EY(a))) ? (R)1 : (R)0;
       spx = spx + w * pn * (R)EX(a);
       spy = spy + w * pn * (R)EY(a);
       ssx = ssx + w * sol * (R)EX(a);
@@ -225,16 +207,15 @@ __global__ void k_adj_psi(Mdl<R> m, const R *__restrict__ fields, const R *__res
       qyy1 = qyy1 + t1 * (R)(EY(a) * EY(a));
       qxy1 = qxy1 + t1 * (R)(EX(a) * EY(a));
     }
-    const R Fxb = aux[i], Fyb = aux[n + i];
+    const R *o = aux + ax(0, 0);
+    const R Fxb = o[0], Fyb = o[an];
     pb = pb + omA * (Fxb * spx + Fyb * spy);
     if (m.wetting == LBM_WET_MARTYS_CHEN) pb = pb - m.Gw * (Fxb * ssx + Fyb * ssy);
-    pb = pb + pre * (omA * (aux[2 * n + i] * qxx1 + aux[3 * n + i] * qyy1 + aux[4 * n + i] * qxy1) -
-                     psi_p * (aux[2 * n + i] + aux[3 * n + i]));
+    pb = pb + pre * (omA * (o[2 * an] * qxx1 + o[3 * an] * qyy1 + o[4 * an] * qxy1) - psi_p * (o[2 * an] + o[3 * an]));
   }
   // to dL/drho (and dL/dT) through U = p(rho) - rho/3 and psi = sqrt(-2U)
-  R rb = (R)0;
-  double tb = 0.0;
-  const R rho = fields[i];
+  rb = (R)0;
+  tb = 0.0;
   const bool ghost = !fluid && m.wetting == LBM_WET_GEOMETRIC;
   if (fluid || (ghost && rho < m.rho_max)) {
     R dp, dpT;
@@ -243,26 +224,14 @@ __global__ void k_adj_psi(Mdl<R> m, const R *__restrict__ fields, const R *__res
     rb = ut * (dp - (R)1 / (R)3);
     tb = (double)(ut * dpT);
   }
-  rhob_out[i] = rb;
-  tacc[i] += tb;
 }
 
+// Transpose of the ghost rule at one wall node, from gb = dL/d(its density):
+// part = dL/d(rho(x-1), rho(x+1), rho(x) of the boundary row, rho(x) of the
+// second row); returns dL/dtheta.  dc, dcot: derivatives of c and cot in theta.
 template <typename R>
-__global__ void k_adj_ghost(Mdl<R> m, const R *__restrict__ fields, const double *__restrict__ coef,
-                            const double *__restrict__ dcoef, const R *__restrict__ rhob,
-                            double *__restrict__ gpart, double *__restrict__ dtheta) {
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= 2 * m.nx) return;
-  int w = t / m.nx, x = t - w * m.nx;
-  int yg = w == 0 ? 0 : m.ny - 1, y1 = w == 0 ? 1 : m.ny - 2, y2 = w == 0 ? 2 : m.ny - 3;
-  double *gp = gpart + (size_t)w * 4 * m.nx;
-  const R *rho = fields;
-  R rim1 = rho[(size_t)y1 * m.nx + m.wx(x - 1)];
-  R rip1 = rho[(size_t)y1 * m.nx + m.wx(x + 1)];
-  R ri1 = rho[(size_t)y1 * m.nx + x];
-  R ri2 = rho[(size_t)y2 * m.nx + x];
-  R c = (R)coef[w * m.nx + x];
-  R cot = (R)coef[2 * m.nx + w * m.nx + x];
+__device__ __forceinline__ double adj_ghost(const Mdl<R> &m, R rim1, R ri1, R rip1, R ri2, R c, R cot, double dc,
+                                            double dcot, R gb, double (&part)[4]) {
   R a = rip1 - rim1;
   // forward again, keeping the iterates
   R d[kMaxIter];
@@ -279,7 +248,6 @@ __global__ void k_adj_ghost(Mdl<R> m, const R *__restrict__ fields, const double
       if (k + 1 < nit) d[k + 1] = ri2 - g;
     }
   }
-  R gb = rhob[(size_t)yg * m.nx + x];
   if (!(g > (R)0 && g < m.ghost_max)) gb = (R)0;  // clamped: no gradient
   R ab = 0, ri1b = 0, ri2b = 0, cb = 0, cotb = 0;
   if (nit <= 0) {
@@ -306,11 +274,199 @@ __global__ void k_adj_ghost(Mdl<R> m, const R *__restrict__ fields, const double
       }
     }
   }
-  gp[x] = -(double)ab;                // to rho(x-1, boundary row)
-  gp[m.nx + x] = (double)ab;          // to rho(x+1, boundary row)
-  gp[2 * m.nx + x] = (double)ri1b;    // to rho(x, boundary row)
-  gp[3 * m.nx + x] = (double)ri2b;    // to rho(x, second row)
-  dtheta[w * m.nx + x] += (double)cb * dcoef[w * m.nx + x] + (double)cotb * dcoef[2 * m.nx + w * m.nx + x];
+  part[0] = -(double)ab;
+  part[1] = (double)ab;
+  part[2] = (double)ri1b;
+  part[3] = (double)ri2b;
+  return (double)cb * dc + (double)cotb * dcot;
+}
+
+// ---- one reverse step in one kernel -----------------------------------------------
+
+constexpr int kTW = 32, kTH = 8;                 // largest tile
+constexpr int kAW = kTW + 4, kAH = kTH + 2;      // nodes with aux: 2 columns and 1 row around the tile
+constexpr int kFW = kTW + 6, kFH = kTH + 4;      // nodes with fields: 3 columns and 2 rows around it
+constexpr int kStepThreads = 480;                // one node per thread in every phase
+
+// lam_out = the reverse step of lam_in at the state f, for the tile of kTW
+// columns x at most kTH rows of this CTA.  Phases, a barrier after each:
+// fields (the values of k_fields) of every node in reach; the transposed
+// collision of every node whose aux the tile reads (threads of the tile keep
+// the part that passes through the moments in registers); dL/drho through psi
+// and U, and at the ghost nodes the transpose of the ghost rule; the sums.
+// Small domains are bound by the latency of a kernel, and five kernels with
+// four global round trips of fields, aux and dL/drho took 19 us (captured; 28
+// launched directly) where this one takes 9; its repeated work at the tiles'
+// edges (1.8 times the fields, 1.4 times the collisions) is paid for at any size
+// by the 170 bytes a node that are not moved: reverse step with its replay, us,
+// five kernels -> one, 256 x 128 21.9 -> 12.0, 800 x 400 61 -> 55, 1600 x 800
+// 245 -> 238.  In FP64 the repeated work costs more than it saves (800 x 400
+// 816 -> 1040; the FP64 pipe is the limit), so FP64 keeps the kernels below.
+template <typename R>
+__global__ void __launch_bounds__(kStepThreads)
+    k_adj_step(Mdl<R> m, int strips, int bands, const R *__restrict__ f, const R *__restrict__ lam_in,
+               R *__restrict__ lam_out, const double *__restrict__ coef, const double *__restrict__ dcoef,
+               double *__restrict__ tacc, double *__restrict__ dtheta, int *flag) {
+  __shared__ R srho[kFH * kFW], spsi[kFH * kFW], sU[kFH * kFW];
+  __shared__ R saux[5 * kAH * kAW];
+  __shared__ double sgp[2][4][kAW];  // ghost-rule parts by wall, part, column (as in aux)
+  const int band = (int)(blockIdx.x / (unsigned)strips);
+  const int x0 = ((int)blockIdx.x - band * strips) * kTW, wr = min(kTW, m.nx - x0);
+  const int first = m.walls ? 1 : 0, rows = m.walls ? m.ny - 2 : m.ny;
+  // equal bands: with walls the outer ones hold both rows that a ghost node reads
+  const int ya = first + (int)((long long)band * rows / bands), yb = first + (int)((long long)(band + 1) * rows / bands);
+  const int hr = yb - ya;
+  const size_t n = (size_t)m.nx * m.ny;
+  const bool geo = m.walls && m.wetting == LBM_WET_GEOMETRIC;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+
+  // this thread's node: rows ya - 1 .. yb, columns x0 - 2 .. x0 + wr + 1
+  const int cy = threadIdx.x / kAW, cx = threadIdx.x - cy * kAW, v = ya - 1 + cy;
+  const bool on = cy < hr + 2 && cx < wr + 4;  // (in a walled domain all these rows exist)
+  const int y = m.wy(v), x = m.wx(x0 - 2 + cx);
+  const bool solid = m.solid_row(y), own = on && cx >= 2 && cx < wr + 2 && (solid || (cy >= 1 && cy <= hr));
+  const size_t i = (size_t)y * m.nx + x;
+  const int jf = (cy + 1) * kFW + cx + 1, ja = cy * kAW + cx;  // its place among the fields and aux
+  auto nb = [&](int ex, int ey) { return jf + ey * kFW + ex; };
+  auto ax = [&](int ex, int ey) { return ja + ey * kAW + ex; };
+  R ls[9], fl[9], cl[9];
+  if (on && !solid) {
+#pragma unroll
+    for (int a = 0; a < 9; ++a) {
+      const int yt = m.wy(y + EY(a));
+      ls[a] = m.solid_row(yt) ? lam_in[OPP(a) * n + i] : lam_in[a * n + (size_t)yt * m.nx + m.wx(x + EX(a))];
+      fl[a] = f[a * n + i];
+    }
+  }
+  // fields: rows ya - 2 .. yb + 1, columns x0 - 3 .. x0 + wr + 2
+  bool bad = false;
+  const int t = threadIdx.x, fy = t / kFW, fx = t - fy * kFW, fv = ya - 2 + fy;
+  if (fy < hr + 4 && fx < wr + 6 && !(m.walls && (fv < 0 || fv >= m.ny))) {
+    const int y = m.wy(fv), x = m.wx(x0 - 3 + fx);
+    R r, psi = (R)0, U = (R)0;
+    if (!m.solid_row(y)) {
+      r = node_rho(f, n, (size_t)y * m.nx + x);
+      psi_U(m, r, psi, U);
+      bad |= !(r > (R)0) || r > m.rho_max;
+    } else if (geo) {
+      const int w = y == 0 ? 0 : 1;
+      const size_t b1 = (size_t)(w == 0 ? 1 : m.ny - 2) * m.nx, b2 = (size_t)(w == 0 ? 2 : m.ny - 3) * m.nx;
+      r = ghost_rho(m, node_rho(f, n, b1 + m.wx(x - 1)), node_rho(f, n, b1 + x), node_rho(f, n, b1 + m.wx(x + 1)),
+                    node_rho(f, n, b2 + x), (R)coef[w * m.nx + x], (R)coef[2 * m.nx + w * m.nx + x]);
+      if (r < m.rho_max) psi_U(m, r, psi, U);
+    } else {
+      r = (R)0;
+    }
+    srho[t] = r;
+    spsi[t] = psi;
+    sU[t] = U;
+  }
+  if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(flag, 1);
+  if (on && !solid) {
+    R Fx, Fy, Qxx, Qyy, Qxy, a5[5];
+    force_Q(m, spsi, sU, y, nb, Fx, Fy, Qxx, Qyy, Qxy);
+    adj_collide(m, fl, ls, srho[jf], Fx, Fy, cl, a5);
+#pragma unroll
+    for (int k = 0; k < 5; ++k) saux[k * kAH * kAW + ja] = a5[k];
+  }
+  __syncthreads();
+  // dL/drho: the tile's nodes, and the ghost nodes of one more column each side
+  R rb = (R)0;
+  if (own || (on && solid && geo && cx >= 1 && cx < wr + 3)) {
+    double tb;
+    adj_psi(m, spsi, saux, kAH * kAW, y, srho[jf], nb, ax, rb, tb);
+    if (own) tacc[i] += tb;
+    if (solid && geo) {
+      const int w = y == 0 ? 0 : 1, s = w == 0 ? kFW : -kFW;
+      double part[4];
+      const double dth = adj_ghost(m, srho[jf + s - 1], srho[jf + s], srho[jf + s + 1], srho[jf + 2 * s],
+                                   (R)coef[w * m.nx + x], (R)coef[2 * m.nx + w * m.nx + x], dcoef[w * m.nx + x],
+                                   dcoef[2 * m.nx + w * m.nx + x], rb, part);
+      if (own) dtheta[w * m.nx + x] += dth;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) sgp[w][k][cx] = part[k];
+    }
+  }
+  if (geo && (ya == 1 || yb == m.ny - 1)) __syncthreads();
+  if (!own) return;
+  if (solid) {
+#pragma unroll
+    for (int a = 0; a < 9; ++a) lam_out[a * n + i] = (R)0;
+    return;
+  }
+  if (geo && (y <= 2 || y >= m.ny - 3)) {
+    double r = (double)rb;
+#pragma unroll
+    for (int w = 0; w < 2; ++w) {
+      const int y1 = w == 0 ? 1 : m.ny - 2, y2 = w == 0 ? 2 : m.ny - 3;
+      // boundary row: this node is x-1 of wall node x+1, x+1 of wall node x-1, and x of wall node x
+      if (y == y1) r += sgp[w][0][cx + 1] + sgp[w][1][cx - 1] + sgp[w][2][cx];
+      if (y == y2) r += sgp[w][3][cx];
+    }
+    rb = (R)r;
+  }
+#pragma unroll
+  for (int a = 0; a < 9; ++a) lam_out[a * n + i] = cl[a] + rb;
+}
+
+// ---- the four kernels of a reverse step on whole fields (FP64, see reverse_step) --
+
+template <typename R>
+__global__ void k_adj_collide(Mdl<R> m, const R *__restrict__ f, const R *__restrict__ fields,
+                              const R *__restrict__ lam_in, R *__restrict__ lam_out, R *__restrict__ aux) {
+  size_t n = (size_t)m.nx * m.ny;
+  size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  int y = (int)(i / m.nx), x = (int)(i - (size_t)y * m.nx);
+  if (m.solid_row(y)) return;
+  // adjoint of the post-collision populations (transpose of the push streaming)
+  R ls[9], fl[9], cl[9], ax[5];
+#pragma unroll
+  for (int a = 0; a < 9; ++a) {
+    int yt = m.wy(y + EY(a));
+    ls[a] = m.solid_row(yt) ? lam_in[OPP(a) * n + i] : lam_in[a * n + (size_t)yt * m.nx + m.wx(x + EX(a))];
+    fl[a] = f[a * n + i];
+  }
+  R Fx, Fy, Qxx, Qyy, Qxy;
+  force_Q(m, fields + n, fields + 2 * n, y, FieldNb<R>{m, y, x}, Fx, Fy, Qxx, Qyy, Qxy);
+  adj_collide(m, fl, ls, fields[i], Fx, Fy, cl, ax);
+#pragma unroll
+  for (int a = 0; a < 9; ++a) lam_out[a * n + i] = cl[a];
+#pragma unroll
+  for (int k = 0; k < 5; ++k) aux[k * n + i] = ax[k];
+}
+
+template <typename R>
+__global__ void k_adj_psi(Mdl<R> m, const R *__restrict__ fields, const R *__restrict__ aux,
+                          R *__restrict__ rhob_out, double *__restrict__ tacc) {
+  size_t n = (size_t)m.nx * m.ny;
+  size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  int y = (int)(i / m.nx), x = (int)(i - (size_t)y * m.nx);
+  const FieldNb<R> nb{m, y, x};
+  R rb;
+  double tb;
+  adj_psi(m, fields + n, aux, n, y, fields[i], nb, nb, rb, tb);
+  rhob_out[i] = rb;
+  tacc[i] += tb;
+}
+
+template <typename R>
+__global__ void k_adj_ghost(Mdl<R> m, const R *__restrict__ fields, const double *__restrict__ coef,
+                            const double *__restrict__ dcoef, const R *__restrict__ rhob,
+                            double *__restrict__ gpart, double *__restrict__ dtheta) {
+  int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= 2 * m.nx) return;
+  int w = t / m.nx, x = t - w * m.nx;
+  int yg = w == 0 ? 0 : m.ny - 1, y1 = w == 0 ? 1 : m.ny - 2, y2 = w == 0 ? 2 : m.ny - 3;
+  const R *r1 = fields + (size_t)y1 * m.nx, *r2 = fields + (size_t)y2 * m.nx;
+  double part[4];
+  dtheta[w * m.nx + x] += adj_ghost(m, r1[m.wx(x - 1)], r1[x], r1[m.wx(x + 1)], r2[x], (R)coef[w * m.nx + x],
+                                    (R)coef[2 * m.nx + w * m.nx + x], dcoef[w * m.nx + x],
+                                    dcoef[2 * m.nx + w * m.nx + x], rhob[(size_t)yg * m.nx + x], part);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) gpart[((size_t)w * 4 + k) * m.nx + x] = part[k];
 }
 
 template <typename R>
@@ -353,20 +509,6 @@ __global__ void k_adj_init(lbm_dev_params P, const double *__restrict__ dl_drho,
   for (int a = 0; a < 9; ++a) lam[a * n + i] = v;
 }
 
-// Deterministic sum of n doubles by one block.
-__global__ void k_sum(const double *__restrict__ v, size_t n, double *__restrict__ out) {
-  __shared__ double sh[1024];
-  double s = 0.0;
-  for (size_t i = threadIdx.x; i < n; i += blockDim.x) s += v[i];
-  sh[threadIdx.x] = s;
-  __syncthreads();
-  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-    if ((int)threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) out[0] = sh[0];
-}
-
 template <typename R>
 __global__ void k_to_double(const R *__restrict__ in, double *__restrict__ out, size_t n) {
   size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -398,26 +540,44 @@ int fwd_step(lbm_ctx *C, const void *src, void *dst) {
 
 template <typename R>
 int reverse_step(lbm_ctx *C, lbm_tape *T, const void *f, int lin) {
-  const size_t n = (size_t)C->nx * C->ny;
-  const int B = 256;
-  const unsigned g = (unsigned)((n + B - 1) / B), gw = (unsigned)((2 * C->nx + B - 1) / B);
   const Mdl<R> m(C->dp);
-  const R *fields = (const R *)C->d_fields;
-  ACK(lbm_ref_fields(C, f, C->d_fields, &C->launches));
   R *lam_in = (R *)T->lam[lin], *lam_out = (R *)T->lam[lin ^ 1];
-  k_adj_collide<R><<<g, B, 0, C->stream>>>(m, (const R *)f, fields, lam_in, lam_out, (R *)T->aux);
-  k_adj_psi<R><<<g, B, 0, C->stream>>>(m, fields, (const R *)T->aux, (R *)T->rhob, T->tacc);
-  C->launches += 2;
-  const int geo = C->walls && m.wetting == LBM_WET_GEOMETRIC;
-  if (geo) {
-    k_adj_ghost<R><<<gw, B, 0, C->stream>>>(m, fields, C->d_coef, C->d_dcoef, (const R *)T->rhob, T->gpart,
-                                            T->dtheta);
+  if constexpr (sizeof(R) == sizeof(float)) {
+    const int rows = C->walls ? C->ny - 2 : C->ny, strips = (C->nx + kTW - 1) / kTW, bands = (rows + kTH - 1) / kTH;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)strips * (unsigned)bands);
+    cfg.blockDim = dim3(kStepThreads);
+    cfg.stream = C->stream;
+    // direct launches overlap their set-up with the kernel before (as k_tile's); captured ones keep plain edges
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = C->capturing ? 0 : 1;
+    ACK(cudaLaunchKernelEx(&cfg, k_adj_step<R>, m, strips, bands, (const R *)f, (const R *)lam_in, lam_out,
+                           (const double *)C->d_coef, (const double *)C->d_dcoef, T->tacc, T->dtheta, C->d_flag));
     ++C->launches;
+    return LBM_OK;
+  } else {
+    const int B = 256;
+    const size_t n = (size_t)C->nx * C->ny;
+    const unsigned g = (unsigned)((n + B - 1) / B), gw = (unsigned)((2 * C->nx + B - 1) / B);
+    const R *fields = (const R *)C->d_fields;
+    ACK(lbm_ref_fields(C, f, C->d_fields, &C->launches));
+    k_adj_collide<R><<<g, B, 0, C->stream>>>(m, (const R *)f, fields, lam_in, lam_out, (R *)T->aux);
+    k_adj_psi<R><<<g, B, 0, C->stream>>>(m, fields, (const R *)T->aux, (R *)T->rhob, T->tacc);
+    C->launches += 2;
+    const int geo = C->walls && m.wetting == LBM_WET_GEOMETRIC;
+    if (geo) {
+      k_adj_ghost<R><<<gw, B, 0, C->stream>>>(m, fields, C->d_coef, C->d_dcoef, (const R *)T->rhob, T->gpart,
+                                              T->dtheta);
+      ++C->launches;
+    }
+    k_adj_finish<R><<<g, B, 0, C->stream>>>(m, lam_out, (const R *)T->rhob, T->gpart, geo);
+    ++C->launches;
+    ACK(cudaGetLastError());
+    return LBM_OK;
   }
-  k_adj_finish<R><<<g, B, 0, C->stream>>>(m, lam_out, (const R *)T->rhob, T->gpart, geo);
-  ++C->launches;
-  ACK(cudaGetLastError());
-  return LBM_OK;
 }
 
 // Capture the work that fn() enqueues on the context stream into *out; the
@@ -475,7 +635,7 @@ int backward(lbm_ctx *C, lbm_tape *T, const double *dl_drho, double *dl_dtheta, 
   }
   if (e == cudaSuccess) e = cudaMemsetAsync(T->tacc, 0, n * sizeof(double), C->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(T->dtheta, 0, 2 * (size_t)C->nx * sizeof(double), C->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(T->gpart, 0, 8 * (size_t)C->nx * sizeof(double), C->stream);
+  if (e == cudaSuccess && T->gpart) e = cudaMemsetAsync(T->gpart, 0, 8 * (size_t)C->nx * sizeof(double), C->stream);
   if (e != cudaSuccess) {
     cudaGetLastError();
     cudaFree(h);
@@ -511,10 +671,8 @@ int backward(lbm_ctx *C, lbm_tape *T, const double *dl_drho, double *dl_dtheta, 
     }
   }
   if (st == LBM_OK) {
-    // dL/dT: deterministic sum of the per-node parts; dL/dtheta; dL/df0
-    k_sum<<<1, 1024, 0, C->stream>>>(T->tacc, n, T->red);
-    ++C->launches;
-    e = cudaGetLastError();
+    // dL/dT: sum of the per-node parts in a fixed order; dL/dtheta; dL/df0
+    e = lbm_reduce_rows(C, T->tacc, 0, C->ny, C->d_red, C->red_len, T->red, &C->launches);
     if (e == cudaSuccess && dl_dT)
       e = cudaMemcpyAsync(dl_dT, T->red, sizeof(double), cudaMemcpyDeviceToHost, C->stream);
     if (e == cudaSuccess && dl_dtheta)
@@ -590,9 +748,7 @@ int lbm_adjoint_record(lbm_ctx *C, int nsteps, int checkpoint_every) {
   for (int k = 0; k < T->nseg && ok; ++k) ok = cudaMalloc(&T->ckpt[k], T->state_bytes) == cudaSuccess;
   ok = ok && cudaMalloc(&T->seg, (size_t)T->every * T->state_bytes) == cudaSuccess &&
        cudaMalloc(&T->lam[0], T->state_bytes) == cudaSuccess && cudaMalloc(&T->lam[1], T->state_bytes) == cudaSuccess &&
-       cudaMalloc(&T->aux, 5 * n * rs) == cudaSuccess && cudaMalloc(&T->rhob, n * rs) == cudaSuccess &&
        cudaMalloc(&T->tacc, n * sizeof(double)) == cudaSuccess &&
-       cudaMalloc(&T->gpart, 8 * (size_t)C->nx * sizeof(double)) == cudaSuccess &&
        cudaMalloc(&T->dtheta, 2 * (size_t)C->nx * sizeof(double)) == cudaSuccess &&
        cudaMalloc(&T->red, sizeof(double)) == cudaSuccess;
   if (!ok) {
@@ -600,7 +756,11 @@ int lbm_adjoint_record(lbm_ctx *C, int nsteps, int checkpoint_every) {
     lbm_adjoint_free_tape(C);
     return LBM_ENOMEM;
   }
-  if (!C->d_fields && cudaMalloc(&C->d_fields, 3 * n * rs) != cudaSuccess) {
+  // scratch of the FP64 reverse step's separate kernels
+  if (C->precision == 64 &&
+      (cudaMalloc(&T->aux, 5 * n * rs) != cudaSuccess || cudaMalloc(&T->rhob, n * rs) != cudaSuccess ||
+       cudaMalloc(&T->gpart, 8 * (size_t)C->nx * sizeof(double)) != cudaSuccess ||
+       (!C->d_fields && cudaMalloc(&C->d_fields, 3 * n * rs) != cudaSuccess))) {
     cudaGetLastError();
     lbm_adjoint_free_tape(C);
     return LBM_ENOMEM;

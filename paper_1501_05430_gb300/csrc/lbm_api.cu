@@ -783,7 +783,8 @@ int lbm_mass(lbm_ctx *C, double *mass) {
   if (!C || !mass) return LBM_EINVAL;
   if (C->status == LBM_ECUDA) return C->status;
   CK(lbm_rho64(C, C->f[C->cur], C->d_rho64, &C->launches));
-  CK(lbm_reduce_mass(C, C->d_rho64, C->d_red, C->red_len, C->d_res, &C->launches));
+  CK(lbm_reduce_rows(C, C->d_rho64, C->walls ? 1 : 0, C->walls ? C->ny - 1 : C->ny, C->d_red, C->red_len, C->d_res,
+                     &C->launches));
   CK(cudaMemcpyAsync(mass, C->d_res, sizeof(double), cudaMemcpyDeviceToHost, C->stream));
   CK(cudaStreamSynchronize(C->stream));
   return LBM_OK;

@@ -120,8 +120,9 @@ cudaError_t lbm_rho64(const lbm_ctx *C, const void *f, double *rho, unsigned lon
 // the same for rows [row0, row1) only (rho indexed like the whole field)
 cudaError_t lbm_rho64_rows(const lbm_ctx *C, const void *f, double *rho, int row0, int row1,
                            unsigned long long *launches);
-cudaError_t lbm_reduce_mass(const lbm_ctx *C, const double *rho, double *partial, int npart, double *res,
-                            unsigned long long *launches);
+// sum of rows [row0, row1) of a node field, in a fixed order
+cudaError_t lbm_reduce_rows(const lbm_ctx *C, const double *v, int row0, int row1, double *partial, int npart,
+                            double *res, unsigned long long *launches);
 cudaError_t lbm_reduce_max_speed(const lbm_ctx *C, const double *ux, const double *uy, double *partial,
                                  int npart, double *res, unsigned long long *launches);
 cudaError_t lbm_angle(const lbm_ctx *C, const double *rho, int wall, int x0, int x1, double rho_mid, double *res,

@@ -311,10 +311,9 @@ cudaError_t lbm_rho64(const lbm_ctx *C, const void *f, double *rho, unsigned lon
   return lbm_rho64_rows(C, f, rho, 0, C->ny, launches);
 }
 
-cudaError_t lbm_reduce_mass(const lbm_ctx *C, const double *rho, double *partial, int npart, double *res,
-                            unsigned long long *launches) {
-  size_t y0 = C->walls ? 1 : 0, y1 = C->walls ? C->ny - 1 : C->ny;
-  k_sum_partial<<<npart, 256, 0, C->stream>>>(rho, (size_t)C->nx * C->ny, y0, y1, C->nx, partial);
+cudaError_t lbm_reduce_rows(const lbm_ctx *C, const double *v, int row0, int row1, double *partial, int npart,
+                            double *res, unsigned long long *launches) {
+  k_sum_partial<<<npart, 256, 0, C->stream>>>(v, (size_t)C->nx * C->ny, row0, row1, C->nx, partial);
   k_sum_final<<<1, 1024, 0, C->stream>>>(partial, npart, res);
   *launches += 2;
   return cudaGetLastError();

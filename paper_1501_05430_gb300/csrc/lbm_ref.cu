@@ -16,15 +16,6 @@ namespace {
 
 using namespace lbm_ref;
 
-// rho at node i: f_0 + f_1 + ... + f_8, left to right.
-template <typename R>
-__device__ __forceinline__ R node_rho(const R *__restrict__ f, size_t n, size_t i) {
-  R r = (R)0;
-#pragma unroll
-  for (int a = 0; a < 9; ++a) r = r + f[a * n + i];
-  return r;
-}
-
 // rho, psi, U at every node.  A solid-row node carries its wall's ghost
 // values: Eqs. 19-21 (geometric) from the densities of rows 1-2 (ny-2, ny-3),
 // which the thread sums itself in the same order as their own threads do, or
@@ -47,19 +38,7 @@ __global__ void k_fields(Mdl<R> m, const R *__restrict__ f, const double *__rest
       const R ri2 = node_rho(f, n, (size_t)y2 * m.nx + x);
       const R c = (R)coef[w * m.nx + x];
       const R cot = (R)coef[2 * m.nx + w * m.nx + x];
-      const R a = rip1 - rim1;
-      if (m.n_iter <= 0) {
-        g = ri2 + cot * fabs(a);
-      } else {
-        R d = (R)2 * (ri2 - ri1);
-        g = ri2;
-        for (int k = 0; k < m.n_iter; ++k) {
-          R s = a * a + d * d;
-          g = ri2 + c * sqrt(s);
-          d = ri2 - g;
-        }
-      }
-      g = fmin(fmax(g, (R)0), m.ghost_max);
+      g = ghost_rho(m, rim1, ri1, rip1, ri2, c, cot);
       // at rho_max (the root of U, Eq. 10) psi and U take their exact value 0
       if (g < m.rho_max) psi_U(m, g, psi, U);
     }
@@ -91,7 +70,7 @@ __global__ void k_macro(Mdl<R> m, const R *__restrict__ f, const R *__restrict__
     return;
   }
   R Fx, Fy, Qxx, Qyy, Qxy;
-  force_Q(m, fields, y, x, Fx, Fy, Qxx, Qyy, Qxy);
+  force_Q(m, fields + n, fields + 2 * n, y, FieldNb<R>{m, y, x}, Fx, Fy, Qxx, Qyy, Qxy);
   R jx = 0, jy = 0;
 #pragma unroll
   for (int a = 0; a < 9; ++a) {

@@ -81,25 +81,62 @@ __device__ void psi_U(const Mdl<R> &m, R rho, R &psi, R &U) {
   psi = sqrt(fmax((R)0, (R)-2 * u));
 }
 
+// rho at node i: f_0 + f_1 + ... + f_8, left to right.
+template <typename R>
+__device__ __forceinline__ R node_rho(const R *__restrict__ f, size_t n, size_t i) {
+  R r = (R)0;
+#pragma unroll
+  for (int a = 0; a < 9; ++a) r = r + f[a * n + i];
+  return r;
+}
+
+// Ghost density of Eqs. 19-21 at column x of a wall, clamped: from the boundary
+// row at x - 1, x, x + 1, the second row at x, c = sin(pi/2 - theta) and
+// cot = tan(pi/2 - theta).
+template <typename R>
+__device__ __forceinline__ R ghost_rho(const Mdl<R> &m, R rim1, R ri1, R rip1, R ri2, R c, R cot) {
+  const R a = rip1 - rim1;
+  R g = ri2;
+  if (m.n_iter <= 0) {
+    g = ri2 + cot * fabs(a);
+  } else {
+    R d = (R)2 * (ri2 - ri1);
+    for (int k = 0; k < m.n_iter; ++k) {
+      R s = a * a + d * d;
+      g = ri2 + c * sqrt(s);
+      d = ri2 - g;
+    }
+  }
+  return fmin(fmax(g, (R)0), m.ghost_max);
+}
+
 template <typename R>
 __device__ __forceinline__ R wgt(int a) { return a <= 4 ? (R)1 / (R)3 : (R)1 / (R)12; }
 
-// Eq. 9 force (+ Eq. 14) and Eq. 17 tensor at fluid node (x, y).
+// Neighbour indices of node (x, y) of a whole field [ny][nx].
 template <typename R>
-__device__ void force_Q(const Mdl<R> &m, const R *__restrict__ fields, int y, int x, R &Fx, R &Fy, R &Qxx,
-                        R &Qyy, R &Qxy) {
-  size_t n = (size_t)m.nx * m.ny;
-  const R *psi = fields + n, *U = fields + 2 * n;
-  R psi0 = psi[(size_t)y * m.nx + x];
+struct FieldNb {
+  const Mdl<R> &m;
+  int y, x;
+  __device__ __forceinline__ size_t operator()(int ex, int ey) const {
+    return (size_t)m.wy(y + ey) * m.nx + m.wx(x + ex);
+  }
+};
+
+// Eq. 9 force (+ Eq. 14) and Eq. 17 tensor at a fluid node of row y; nb(ex, ey)
+// is the index of a neighbour in psi and U.
+template <typename R, typename Nb>
+__device__ __forceinline__ void force_Q(const Mdl<R> &m, const R *__restrict__ psi, const R *__restrict__ U, int y,
+                                        Nb nb, R &Fx, R &Fy, R &Qxx, R &Qyy, R &Qxy) {
+  R psi0 = psi[nb(0, 0)];
   R spx = 0, spy = 0, sUx = 0, sUy = 0, ssx = 0, ssy = 0;
   R qxx1 = 0, qyy1 = 0, qxy1 = 0, qxx2 = 0, qyy2 = 0, qxy2 = 0;
 #pragma unroll
   for (int a = 1; a < 9; ++a) {
-    int yn = m.wy(y + EY(a)), xn = m.wx(x + EX(a));
-    size_t j = (size_t)yn * m.nx + xn;
+    const auto j = nb(EX(a), EY(a));
     R pn = psi[j], un = U[j];
     R w = wgt<R>(a);
-    R solid = m.solid_row(yn) ? (R)1 : (R)0;
+    R solid = m.solid_row(m.wy(y + EY(a))) ? (R)1 : (R)0;
     if (EX(a) != 0) {
       R tp = w * pn, tu = w * un, ts = w * solid;
       if (EX(a) > 0) { spx = spx + tp; sUx = sUx + tu; ssx = ssx + ts; }
