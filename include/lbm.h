@@ -362,7 +362,10 @@ typedef struct {
   lbm_params params;     /* precision must be 32; kernel is ignored */
 } lbm_instance_desc;
 
-/* Launch shape.  Zero fields take the defaults in brackets. */
+/* Launch shape.  Zero fields take the defaults in brackets.  With every field
+ * at its default (or no config) the library may run a small batch with one
+ * launch per step instead (tiles of 64 columns x 4 rows, no waits); results
+ * are the same. */
 typedef struct {
   int threads;           /* 256 [default]: every instance in one launch of 256-thread
                             CTAs; 128: the instances up to 256 wide in a launch of their
@@ -424,14 +427,16 @@ int lbm_batch_contact_angles(lbm_batch *b, int wall, double *theta, double *H, d
 /* Pick the launch shape by timing trial_steps steps of candidate
  * configurations on a copy of the current state (threads x stages, then the
  * band height of each size class present, then steps_per_launch), install the
- * fastest and put the state back.  best (may be NULL) receives it.
+ * fastest and put the state back.  best (may be NULL) receives the fastest
+ * shape; when one launch per step is faster still, that is what is installed.
  * Needs one extra state-sized device allocation while it runs. */
 int lbm_batch_autotune(lbm_batch *b, int trial_steps, lbm_batch_config *best);
 
 int lbm_batch_get_config(const lbm_batch *b, lbm_batch_config *cfg);
 /* Install a launch shape (validated as in lbm_batch_create). */
 int lbm_batch_set_config(lbm_batch *b, const lbm_batch_config *cfg);
-/* Plan of the current shape: CTAs per launch, work items, dynamic shared
+/* Plan of the current shape (one launch per step: CTAs and items are its tiles,
+ * no dynamic shared memory): CTAs per launch, work items, dynamic shared
  * memory per CTA, resident CTAs per SM.  With threads = 128 and instances on
  * both sides of 256 columns, CTAs and items are summed over the two launches,
  * the shared memory is the larger one and the CTAs per SM are the 256-thread

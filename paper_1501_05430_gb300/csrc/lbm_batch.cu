@@ -41,7 +41,7 @@
 #include <vector>
 
 #include "lbm_internal.h"
-#include "lbm_node.cuh"
+#include "lbm_tile.cuh"
 
 namespace {
 
@@ -529,6 +529,59 @@ __global__ void __launch_bounds__(NT, 768 / NT) k_batch(BatchArgs A) {
   }
 }
 
+// ---- small batches: one launch per step, one tile per CTA -------------------------
+
+constexpr int kTileRows = 4;
+constexpr int kTileThreads = (kTileRows + 3) * 32;
+
+struct BTile {
+  int inst, x0, y0, pad;
+};
+
+struct TileArgs {
+  const BInst *inst;
+  const BTile *tiles;
+  int *iflag;
+  unsigned long long *work;
+  const int *cur;
+  int phase;  // parity of the step
+  int pdl;    // launched as a programmatic dependent of the step before
+};
+
+template <int KIND, int MCW>
+__global__ void __launch_bounds__(kTileThreads) k_batch_tile(TileArgs A) {
+  __shared__ BInst P;
+  __shared__ lbm_tile::Smem<kTileRows> M;
+  if (A.pdl) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const BTile t = A.tiles[blockIdx.x];
+  const int *src = (const int *)(A.inst + t.inst);
+  for (int k = threadIdx.x; k < (int)(sizeof(BInst) / sizeof(int)); k += kTileThreads) ((int *)&P)[k] = src[k];
+  const int par = A.cur[t.inst] ^ A.phase;
+  __syncthreads();
+  if (A.pdl) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (*(volatile const int *)(A.iflag + t.inst) & 1) return;  // a blown-up instance is frozen
+  auto ready = [] {};
+  auto unstable = [&] {
+    atomicOr(A.iflag + t.inst, 1);
+    atomicOr(P.flag, 1);
+  };
+  const float *fin = P.f[par];
+  float *fout = P.f[par ^ 1];
+  if (P.unit)
+    lbm_tile::step<true, MCW, KIND, kTileRows>(P, t.x0, t.y0, fin, fout, M, ready, unstable);
+  else
+    lbm_tile::step<false, MCW, KIND, kTileRows>(P, t.x0, t.y0, fin, fout, M, ready, unstable);
+  if (threadIdx.x == 0)
+    atomicAdd(A.work + t.inst, (unsigned long long)(min(kTileRows, P.ny - 1 - t.y0) * min(lbm_tile::kW, P.nx - t.x0)));
+}
+
+typedef void (*TileKernel)(TileArgs);
+TileKernel tile_kernel(int kind) {
+  if (kind == LBM_EOS_CARNAHAN_STARLING) return k_batch_tile<LBM_EOS_CARNAHAN_STARLING, 0>;
+  if (kind == LBM_EOS_PIECEWISE) return k_batch_tile<LBM_EOS_PIECEWISE, 0>;
+  return k_batch_tile<-1, -1>;
+}
+
 typedef void (*BatchKernel)(BatchArgs);
 template <int NT>
 BatchKernel pick_batch(int kind) {
@@ -581,6 +634,11 @@ struct lbm_batch {
   unsigned long long *d_work;  // [n] fluid-node updates computed per instance
   int *d_cur;
   int nsm;
+  // small batches with the default shape: one launch of tile CTAs per step
+  bool tile;
+  int tile_kind, tile_occ;
+  std::vector<BTile> tiles;
+  BTile *d_tiles;
   cudaGraphExec_t graph[2];   // per starting phase
   int graph_steps;
   unsigned long long graph_kernels;  // kernels one graph replay launches
@@ -628,6 +686,39 @@ int resolve_config(const lbm_batch *B, const lbm_batch_config *in, lbm_batch_con
   if (!(c.wait_seconds > 0.0) || c.wait_seconds > 60.0) return LBM_EINVAL;
   if (c.hold_instance < -1 || c.hold_instance >= B->n) return LBM_EINVAL;
   *out = c;
+  return LBM_OK;
+}
+
+bool default_shape(const lbm_batch_config &c) {
+  return !c.threads && !c.ctas_per_sm && !c.stages && !c.band_rows[0] && !c.band_rows[1] && !c.band_rows[2] &&
+         !c.band_rows[3] && !c.steps_per_launch && !c.graph_launches && c.wait_seconds == 0.0 &&
+         c.hold_instance == -1;
+}
+
+// Tile list of the whole batch, made once.
+int plan_tiles(lbm_batch *B) {
+  if (!B->tiles.empty()) return LBM_OK;
+  B->tile_kind = -2;
+  for (int i = 0; i < B->n; ++i) {
+    const lbm_ctx *C = B->ctx[i];
+    const int k = C->dp.wetting == LBM_WET_GEOMETRIC ? C->dp.eos_kind : -1;
+    B->tile_kind = B->tile_kind == -2 || B->tile_kind == k ? k : -1;
+    for (int y = 1; y < C->ny - 1; y += kTileRows)
+      for (int x = 0; x < C->nx; x += lbm_tile::kW) B->tiles.push_back(BTile{i, x, y, 0});
+  }
+  cudaError_t e = cudaMalloc(&B->d_tiles, B->tiles.size() * sizeof(BTile));
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(B->d_tiles, B->tiles.data(), B->tiles.size() * sizeof(BTile), cudaMemcpyHostToDevice,
+                        B->stream);
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&B->tile_occ, tile_kernel(B->tile_kind), kTileThreads, 0);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    cudaFree(B->d_tiles);
+    B->d_tiles = nullptr;
+    B->tiles.clear();
+    return e == cudaErrorMemoryAllocation ? LBM_ENOMEM : LBM_ECUDA;
+  }
   return LBM_OK;
 }
 
@@ -799,9 +890,35 @@ void fill_inst(BInst &I, const lbm_ctx *C, int *flag) {
   I.flag = flag;
 }
 
+// One step of every instance (tile form) at parity `phase`.
+int launch_tiles(lbm_batch *B, int phase, bool capturing) {
+  TileArgs A{B->d_inst, B->d_tiles, B->d_iflag, B->d_work, B->d_cur, phase, capturing ? 0 : 1};
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = dim3((unsigned)B->tiles.size());
+  lc.blockDim = dim3(kTileThreads);
+  lc.stream = B->stream;
+  cudaLaunchAttribute at[1];  // direct launches only; captured ones keep plain edges (see lbm_tile.cu)
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  lc.attrs = at;
+  lc.numAttrs = A.pdl;
+  BCK(cudaLaunchKernelEx(&lc, tile_kernel(B->tile_kind), A));
+  ++B->launches;
+  return LBM_OK;
+}
+
+// `launches` launches of `steps` steps each from parity `phase`.
+int launch_many(lbm_batch *B, int launches, int steps, int phase, bool capturing) {
+  for (int l = 0; l < launches; ++l) {
+    const int st = B->tile ? launch_tiles(B, (phase + l) & 1, capturing) : launch(B, steps, phase ^ (l * steps & 1));
+    if (st != LBM_OK) return st;
+  }
+  return LBM_OK;
+}
+
 int run_steps(lbm_batch *B, int nsteps) {
-  const int k = B->cfg.steps_per_launch;
-  const int G = B->cfg.graph_launches;
+  const int k = B->tile ? 1 : B->cfg.steps_per_launch;
+  const int G = B->tile ? 32 : B->cfg.graph_launches;  // tiles: steps captured per graph
   int done = 0;
   // whole graphs (an even number of steps each, so a replay ends on the phase it started from)
   if (G > 0 && B->stream && (long long)G * k % 2 == 0 && nsteps >= G * k) {
@@ -809,9 +926,8 @@ int run_steps(lbm_batch *B, int nsteps) {
     if (!B->graph[p]) {
       cudaGraph_t g = nullptr;
       BCK(cudaStreamBeginCapture(B->stream, cudaStreamCaptureModeThreadLocal));
-      int st = LBM_OK;
       const unsigned long long l0 = B->launches;
-      for (int l = 0; l < G && st == LBM_OK; ++l) st = launch(B, k, p ^ (l * k & 1));
+      const int st = launch_many(B, G, k, p, true);
       cudaError_t e = cudaStreamEndCapture(B->stream, &g);
       B->graph_kernels = B->launches - l0;
       B->launches = l0;  // counted when replayed
@@ -833,11 +949,27 @@ int run_steps(lbm_batch *B, int nsteps) {
   }
   while (done < nsteps) {
     const int m = std::min(k, nsteps - done);
-    int st = launch(B, m, (B->phase + done) & 1);
+    int st = launch_many(B, 1, m, (B->phase + done) & 1, false);
     if (st) return st;
     done += m;
   }
   return LBM_OK;
+}
+
+// Whether the batch steps in tiles; only an all-default shape leaves it to the
+// library.  The persistent kernel's step lasts at least as long as a band of 32
+// rows sweeps (45 us) and advances 34 nodes per ns in instances up to 128 wide
+// (three quarters of a CTA idle), about 68 in wider ones; the tile kernel
+// advances 50 whatever the width.  Measured, us per step, persistent / tile:
+// 6 of 300 x 100 47 / 6.4, 32 of 256 x 128 45 / 20, 64 of them 53 / 44, 128 of
+// them 69 / 83, 16 of 512 x 256 49 / 42, 32 of them 64 / 80, 1024 of 128 x 64
+// 236 / 162, 100 of the four sizes 102 / 122.
+int choose_tiles(lbm_batch *B, const lbm_batch_config &asked) {
+  double narrow = 0.0, wide = 0.0;
+  for (int i = 0; i < B->n; ++i)
+    (B->ctx[i]->nx <= 128 ? narrow : wide) += (double)B->ctx[i]->nx * (B->ctx[i]->ny - 2);
+  B->tile = default_shape(asked) && (narrow + wide) / 50e3 < std::max(45.0, narrow / 34e3 + wide / 68e3);
+  return B->tile ? plan_tiles(B) : LBM_OK;
 }
 
 }  // namespace
@@ -915,7 +1047,8 @@ int lbm_batch_create(int n, const lbm_instance_desc *inst, const lbm_batch_confi
   lbm_batch_config c;
   lbm_batch_config_default(&c);
   if (cfg) c = *cfg;
-  if ((st = resolve_config(B, &c, &B->cfg)) != LBM_OK || (st = plan(B)) != LBM_OK) {
+  if ((st = resolve_config(B, &c, &B->cfg)) != LBM_OK || (st = plan(B)) != LBM_OK ||
+      (st = choose_tiles(B, c)) != LBM_OK) {
     lbm_batch_destroy(B);
     return st;
   }
@@ -948,7 +1081,7 @@ int lbm_batch_set_config(lbm_batch *B, const lbm_batch_config *cfg) {
     plan(B);
     return st;
   }
-  return LBM_OK;
+  return choose_tiles(B, *cfg);
 }
 
 int lbm_batch_step(lbm_batch *B, int nsteps) {
@@ -1021,8 +1154,11 @@ int lbm_batch_autotune(lbm_batch *B, int trial_steps, lbm_batch_config *best) {
   lbm_batch_config cur = start;
   cur.graph_launches = 0;
   cur.hold_instance = -1;
+  const bool tile0 = B->tile;
+  B->tile = false;
   double best_ms = INFINITY;
   lbm_batch_config best_cfg = cur;
+  bool best_tile = false;
   auto trial = [&](const lbm_batch_config &c) -> int {
     lbm_batch_config r;
     if (resolve_config(B, &c, &r) != LBM_OK) return LBM_OK;  // not applicable to this batch
@@ -1030,7 +1166,7 @@ int lbm_batch_autotune(lbm_batch *B, int trial_steps, lbm_batch_config *best) {
     int s = plan(B);
     if (s == LBM_EUNSUPPORTED) return LBM_OK;
     if (s) return s;
-    s = run_steps(B, 2);  // warm-up
+    s = run_steps(B, B->tile ? trial_steps : 2);  // warm-up (tiles: with the graphs)
     if (s) return s;
     BCK(cudaEventRecord(t0, B->stream));
     s = run_steps(B, trial_steps);
@@ -1045,6 +1181,7 @@ int lbm_batch_autotune(lbm_batch *B, int trial_steps, lbm_batch_config *best) {
     if (ms < best_ms) {
       best_ms = ms;
       best_cfg = r;
+      best_tile = B->tile;
     }
     return LBM_OK;
   };
@@ -1079,10 +1216,16 @@ int lbm_batch_autotune(lbm_batch *B, int trial_steps, lbm_batch_config *best) {
       st = trial(c);
     }
     cur = best_cfg;
+    // the tile form last: *best stays the best persistent shape
+    if (st == LBM_OK && (st = plan_tiles(B)) == LBM_OK) {
+      B->tile = true;
+      st = trial(cur);
+    }
   } else {
     cudaGetLastError();
     st = LBM_ECUDA;
   }
+  B->tile = st == LBM_OK ? best_tile : tile0;
   // restore the state and install the winner (with the caller's graph and wait settings)
   if (st == LBM_OK) {
     cur.graph_launches = start.graph_launches;
@@ -1129,6 +1272,13 @@ int lbm_batch_node_updates(lbm_batch *B, unsigned long long *updates) {
 
 int lbm_batch_get_plan(const lbm_batch *B, int *grid, int *items, int *smem_bytes, int *ctas_per_sm) {
   if (!B) return LBM_EINVAL;
+  if (B->tile) {
+    if (grid) *grid = (int)B->tiles.size();
+    if (items) *items = (int)B->tiles.size();
+    if (smem_bytes) *smem_bytes = 0;
+    if (ctas_per_sm) *ctas_per_sm = B->tile_occ;
+    return LBM_OK;
+  }
   const lbm_batch::Part &P0 = B->part[0], &P1 = B->part[1];
   if (grid) *grid = P0.grid + P1.grid;
   if (items) *items = (int)(P0.items.size() + P1.items.size());
@@ -1147,6 +1297,7 @@ void lbm_batch_destroy(lbm_batch *B) {
   cudaFree(B->pool);
   cudaFree(B->d_inst);
   for (int s = 0; s < 2; ++s) cudaFree(B->part[s].d_items);
+  cudaFree(B->d_tiles);
   cudaFree(B->d_bar);
   cudaFree(B->d_abort);
   cudaFree(B->d_iflag);

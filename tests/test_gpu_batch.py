@@ -299,3 +299,56 @@ def test_invalid_batches_rejected():
     with pytest.raises(L.LbmError):
         L.LbmBatch([d], L.lbm_batch_config_default(stages=9))
     c.orc.close()
+
+
+@pytest.mark.parametrize("specs", [SPECS, SPECS_CS, [(68, 7, dict(tau=0.8)), (64, 6, dict()), (60, 8, dict(n_iter=0)),
+                                                     (132, 9, dict(wetting=1, G_w=-0.2))]])
+@pytest.mark.parametrize("on_stream", [False, True])
+def test_tile_form_gives_the_persistent_kernels_bits(specs, on_stream):
+    """An all-default shape steps a small batch with one launch per step (direct
+    or from graphs of 32): same bits, counts and statuses as the persistent
+    kernel, whatever the step counts and switches between the two."""
+    import torch
+
+    stream = torch.cuda.Stream() if on_stream else None
+    cases = _cases(specs, seed=21)
+    with _batch(cases, stream=stream) as a, _batch(cases, stream=stream, stages=3) as b:
+        for n in (1, 33, 2):
+            a.step(n)
+            b.step(n)
+        assert a.launches() == 36 and a.plan()["items"] == sum(-(-c.nx // 64) * -(-(c.ny - 2) // 4) for c in cases)
+        a.set_config(L.lbm_batch_config_default(stages=4))
+        a.step(3)
+        a.set_config(L.lbm_batch_config_default())
+        a.step(2)
+        b.step(5)
+        st = a.status()[1]
+        assert np.array_equal(st, b.status()[1])
+        ua, ub = a.node_updates(), b.node_updates()
+        for k, (x, y) in enumerate(zip(a.instances, b.instances)):
+            if st[k] == 0:  # (an unstable one is frozen somewhere within its step)
+                assert np.array_equal(x.f(), y.f())
+                assert ua[k] == ub[k]
+    _close(cases)
+
+
+def test_tile_form_freezes_an_unstable_instance():
+    cases = _cases()[:3]
+    bad = cases[1].f0.copy()
+    bad[:, 5, 7] = np.nan
+    with _batch(cases) as b, _batch(cases, stages=3) as ok:
+        b[1].set_f(bad)
+        b.step(9)
+        ok.step(9)
+        inst = b.status()[1]
+        assert inst[1] == L.LBM_EUNSTABLE and inst[0] == inst[2] == 0
+        upd = b.node_updates()
+        for k in (0, 2):
+            assert np.array_equal(b[k].f(), ok[k].f())
+            assert upd[k] == cases[k].nx * (cases[k].ny - 2) * 9
+        assert 0 < upd[1] <= cases[1].nx * (cases[1].ny - 2)
+        f = b[1].f()
+        b.step(4)
+        assert np.array_equal(b[1].f(), f, equal_nan=True)
+        assert b.node_updates()[1] == upd[1]
+    _close(cases)
