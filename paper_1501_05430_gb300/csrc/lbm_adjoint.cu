@@ -563,7 +563,7 @@ int reverse_step(lbm_ctx *C, lbm_tape *T, const void *f, int lin) {
     const size_t n = (size_t)C->nx * C->ny;
     const unsigned g = (unsigned)((n + B - 1) / B), gw = (unsigned)((2 * C->nx + B - 1) / B);
     const R *fields = (const R *)C->d_fields;
-    ACK(lbm_ref_fields(C, f, C->d_fields, &C->launches));
+    ACK(lbm_ref_fields(C, (const double *)f, (double *)C->d_fields, &C->launches));
     k_adj_collide<R><<<g, B, 0, C->stream>>>(m, (const R *)f, fields, lam_in, lam_out, (R *)T->aux);
     k_adj_psi<R><<<g, B, 0, C->stream>>>(m, fields, (const R *)T->aux, (R *)T->rhob, T->tacc);
     C->launches += 2;
@@ -672,7 +672,7 @@ int backward(lbm_ctx *C, lbm_tape *T, const double *dl_drho, double *dl_dtheta, 
   }
   if (st == LBM_OK) {
     // dL/dT: sum of the per-node parts in a fixed order; dL/dtheta; dL/df0
-    e = lbm_reduce_rows(C, T->tacc, 0, C->ny, C->d_red, C->red_len, T->red, &C->launches);
+    e = lbm_reduce_rows(C, T->tacc, 0, C->ny, T->red, &C->launches);
     if (e == cudaSuccess && dl_dT)
       e = cudaMemcpyAsync(dl_dT, T->red, sizeof(double), cudaMemcpyDeviceToHost, C->stream);
     if (e == cudaSuccess && dl_dtheta)

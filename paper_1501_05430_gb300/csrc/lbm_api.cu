@@ -220,31 +220,13 @@ void *mapped_host(const void *p) {
   return a.devicePointer;
 }
 
-int ensure_fields(lbm_ctx *C) {
-  if (C->d_fields) return LBM_OK;
-  if (cudaMalloc(&C->d_fields, 3 * n_nodes(C) * real_size(C->precision)) != cudaSuccess) {
-    C->d_fields = nullptr;
-    cudaGetLastError();
-    return LBM_ENOMEM;
-  }
-  return LBM_OK;
-}
-
 int ensure_aux(lbm_ctx *C) {
   if (C->d_aux) return LBM_OK;
-  if (cudaMalloc(&C->d_aux, 7 * n_nodes(C) * sizeof(double)) != cudaSuccess) {
+  if (cudaMalloc(&C->d_aux, 8 * n_nodes(C) * sizeof(double)) != cudaSuccess) {
     C->d_aux = nullptr;
     cudaGetLastError();
     return LBM_ENOMEM;
   }
-  return LBM_OK;
-}
-
-// Reference-path fields (rho, psi, U incl. ghost rows) of the current state.
-int compute_fields(lbm_ctx *C) {
-  int st = ensure_fields(C);
-  if (st) return st;
-  CK(lbm_ref_fields(C, C->f[C->cur], C->d_fields, &C->launches));
   return LBM_OK;
 }
 
@@ -679,49 +661,32 @@ int lbm_get_rho(lbm_ctx *C, double *rho) {
   return LBM_OK;
 }
 
-int lbm_get_fields(lbm_ctx *C, double *rho, double *psi, double *U, double *Fx, double *Fy, double *Qxx,
-                   double *Qyy, double *Qxy) {
-  if (!C) return LBM_EINVAL;
+// Fields of the current state (order of lbm_canon_fields) into the host arrays
+// that are not NULL, at most 8 of them.
+static int get_fields(lbm_ctx *C, double *const (&host)[10]) {
   if (C->status == LBM_ECUDA) return C->status;
-  int st = compute_fields(C);
+  int st = ensure_aux(C);
   if (st) return st;
-  if ((st = ensure_aux(C)) != LBM_OK) return st;
-  CK(lbm_ref_macro(C, C->f[C->cur], C->d_fields, C->d_aux, &C->launches));
-  size_t n = n_nodes(C), rs = real_size(C->precision);
-  double *outs[3] = {rho, psi, U};
-  void *host = nullptr;
-  if (rho || psi || U) {
-    host = malloc(3 * n * rs);
-    if (!host) return LBM_ENOMEM;
-    cudaError_t e = cudaMemcpyAsync(host, C->d_fields, 3 * n * rs, cudaMemcpyDeviceToHost, C->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(C->stream);
-    if (e != cudaSuccess) { free(host); C->status = LBM_ECUDA; return LBM_ECUDA; }
-    for (int k = 0; k < 3; ++k) {
-      if (!outs[k]) continue;
-      for (size_t i = 0; i < n; ++i)
-        outs[k][i] = rs == 8 ? ((double *)host)[k * n + i] : (double)((float *)host)[k * n + i];
-    }
-    free(host);
-  }
-  double *o7[5] = {Fx, Fy, Qxx, Qyy, Qxy};
-  for (int k = 0; k < 5; ++k)
-    if (o7[k]) CK(cudaMemcpyAsync(o7[k], C->d_aux + (2 + k) * n, n * sizeof(double), cudaMemcpyDeviceToHost, C->stream));
+  const size_t n = n_nodes(C);
+  double *dev[10];
+  int used = 0;
+  for (int k = 0; k < 10; ++k) dev[k] = host[k] ? C->d_aux + (size_t)used++ * n : nullptr;
+  CK(lbm_canon_fields(C, C->f[C->cur], dev, &C->launches));
+  for (int k = 0; k < 10; ++k)
+    if (host[k]) CK(cudaMemcpyAsync(host[k], dev[k], n * sizeof(double), cudaMemcpyDeviceToHost, C->stream));
   CK(cudaStreamSynchronize(C->stream));
   return LBM_OK;
 }
 
+int lbm_get_fields(lbm_ctx *C, double *rho, double *psi, double *U, double *Fx, double *Fy, double *Qxx,
+                   double *Qyy, double *Qxy) {
+  if (!C) return LBM_EINVAL;
+  return get_fields(C, {rho, psi, U, nullptr, nullptr, Fx, Fy, Qxx, Qyy, Qxy});
+}
+
 int lbm_get_u(lbm_ctx *C, double *ux, double *uy) {
   if (!C) return LBM_EINVAL;
-  if (C->status == LBM_ECUDA) return C->status;
-  int st = compute_fields(C);
-  if (st) return st;
-  if ((st = ensure_aux(C)) != LBM_OK) return st;
-  CK(lbm_ref_macro(C, C->f[C->cur], C->d_fields, C->d_aux, &C->launches));
-  size_t n = n_nodes(C);
-  if (ux) CK(cudaMemcpyAsync(ux, C->d_aux, n * sizeof(double), cudaMemcpyDeviceToHost, C->stream));
-  if (uy) CK(cudaMemcpyAsync(uy, C->d_aux + n, n * sizeof(double), cudaMemcpyDeviceToHost, C->stream));
-  CK(cudaStreamSynchronize(C->stream));
-  return LBM_OK;
+  return get_fields(C, {nullptr, nullptr, nullptr, ux, uy, nullptr, nullptr, nullptr, nullptr, nullptr});
 }
 
 int lbm_get_f(lbm_ctx *C, double *f) {
@@ -767,24 +732,23 @@ int lbm_contact_angle(lbm_ctx *C, int wall, int x0, int x1, double *theta, doubl
   if (!C || (wall != 0 && wall != 1) || x0 < 0 || x1 > C->nx || x0 >= x1) return LBM_EINVAL;
   if (!C->walls) return LBM_EINVAL;
   if (C->status == LBM_ECUDA) return C->status;
-  CK(lbm_rho64(C, C->f[C->cur], C->d_rho64, &C->launches));
-  CK(lbm_angle(C, C->d_rho64, wall, x0, x1, C->rho_mid, C->d_res, &C->launches));
-  double r[5];
-  CK(cudaMemcpyAsync(r, C->d_res, sizeof(r), cudaMemcpyDeviceToHost, C->stream));
+  CK(lbm_angle(C, lbm_make_angle_args(C, wall, x0, x1, C->d_res), &C->launches));
+  lbm_angle_cut r;
+  CK(cudaMemcpyAsync(&r, C->d_res, sizeof(r), cudaMemcpyDeviceToHost, C->stream));
   CK(cudaStreamSynchronize(C->stream));
-  if (r[4] != 0.0) return LBM_ENOCONTACT;
-  if (theta) *theta = r[0];
-  if (H) *H = r[1];
-  if (L) *L = r[2];
+  double t, h, l;
+  const int st = lbm_angle_of(r, C->rho_mid, &t, &h, &l);
+  if (st) return st;
+  if (theta) *theta = t;
+  if (H) *H = h;
+  if (L) *L = l;
   return LBM_OK;
 }
 
 int lbm_mass(lbm_ctx *C, double *mass) {
   if (!C || !mass) return LBM_EINVAL;
   if (C->status == LBM_ECUDA) return C->status;
-  CK(lbm_rho64(C, C->f[C->cur], C->d_rho64, &C->launches));
-  CK(lbm_reduce_rows(C, C->d_rho64, C->walls ? 1 : 0, C->walls ? C->ny - 1 : C->ny, C->d_red, C->red_len, C->d_res,
-                     &C->launches));
+  CK(lbm_mass_of(C, C->f[C->cur], C->d_res, &C->launches));
   CK(cudaMemcpyAsync(mass, C->d_res, sizeof(double), cudaMemcpyDeviceToHost, C->stream));
   CK(cudaStreamSynchronize(C->stream));
   return LBM_OK;
@@ -793,14 +757,11 @@ int lbm_mass(lbm_ctx *C, double *mass) {
 int lbm_max_speed(lbm_ctx *C, double *umax) {
   if (!C || !umax) return LBM_EINVAL;
   if (C->status == LBM_ECUDA) return C->status;
-  int st = compute_fields(C);
-  if (st) return st;
-  if ((st = ensure_aux(C)) != LBM_OK) return st;
-  CK(lbm_ref_macro(C, C->f[C->cur], C->d_fields, C->d_aux, &C->launches));
-  size_t n = n_nodes(C);
-  CK(lbm_reduce_max_speed(C, C->d_aux, C->d_aux + n, C->d_red, C->red_len, C->d_res, &C->launches));
-  CK(cudaMemcpyAsync(umax, C->d_res, sizeof(double), cudaMemcpyDeviceToHost, C->stream));
+  double u2 = 0.0;
+  CK(lbm_canon_max_speed2(C, C->f[C->cur], C->d_res, &C->launches));
+  CK(cudaMemcpyAsync(&u2, C->d_res, sizeof(double), cudaMemcpyDeviceToHost, C->stream));
   CK(cudaStreamSynchronize(C->stream));
+  *umax = sqrt(u2);
   return LBM_OK;
 }
 

@@ -19,6 +19,8 @@
 // instruction issue and the FMA pipe.
 #include <math.h>
 
+#include <type_traits>
+
 #include "lbm_internal.h"
 
 namespace {
@@ -152,11 +154,11 @@ __device__ __forceinline__ void psi_U(const Canon<R> &m, V rho, V &psi, V &U) {
   psi = root0(bc((R)-2) * U);
 }
 
-// Ghost psi and U (Eqs. 19-21) from the densities around column x.
+// Ghost density, psi and U (Eqs. 19-21) from the densities around column x.
 template <class R>
-__device__ __forceinline__ void ghost(const Canon<R> &m, R rim1, R ri1, R rip1, R ri2, R c, R &psi, R &U) {
+__device__ __forceinline__ void ghost(const Canon<R> &m, R rim1, R ri1, R rip1, R ri2, R c, R &g, R &psi, R &U) {
   const R a = rip1 - rim1;
-  R g = ri2;
+  g = ri2;
   if (m.n_iter <= 0) {
     g = ri2 + c * fabs(a);
   } else {
@@ -202,10 +204,12 @@ struct Window<F2, R> {
 };
 template <int R>
 struct Window<double, R> {
-  double p[R + 2][kWP], p2[R + 2][kWP], p1w[R + 2][kWP], p2w[R + 2][kWP], u1w[R + 2][kWP], u2w[R + 2][kWP];
+  double p[R + 2][kWP], u[R + 2][kWP], p2[R + 2][kWP], p1w[R + 2][kWP], p2w[R + 2][kWP], u1w[R + 2][kWP],
+      u2w[R + 2][kWP];
   __device__ __forceinline__ void put(int row, int c, double psi, double U) {
     const int i = c + 2;
     p[row][i] = psi;
+    u[row][i] = U;
     p2[row][i] = psi * psi;
     p1w[row][i] = (1.0 / 3.0) * psi;
     p2w[row][i] = (1.0 / 12.0) * psi;
@@ -218,62 +222,75 @@ struct Window<double, R> {
   }
 };
 
-// Force (Eq. 9, + Eq. 14 with ss = sum_a w_a S e_ay), Eq. 17 tensor and MRT
-// collision of the node(s) at window row `row`, entry i; f: populations, rho:
-// density, fs: post-collision populations.
+// Force (Eq. 9, + Eq. 14 with ss = sum_a w_a S e_ay) and Eq. 17 tensor of the
+// node(s) at window row `row`, entry i.
+template <class V, class R, class W>
+__device__ __forceinline__ void force(const Canon<R> &m, const W &win, int row, int i, R ss, V &Fx, V &Fy, V &Qxx,
+                                      V &Qyy, V &Qxy) {
+  auto bc = [](R c) { return Val<V>::bc(c); };
+  const V w1 = bc((R)1 / (R)3), w2 = bc((R)1 / (R)12);
+  const Nb<V> n0 = win.template at<false>(row, i);
+  V spx, spy, sUx, sUy, xx1, yy1, xy1, xx2, yy2, xy2;
+  auto t1 = [&](const Nb<V> &n, V w) { return w * (n.p - n0.p); };
+  auto t2 = [&](const Nb<V> &n, V w) { return w * (n.p2 - n0.p2); };
+  Nb<V> n = win.template at<false>(row, i + 1);  // e1
+  spx = n.tp, sUx = n.tu, xx1 = t1(n, w1), xx2 = t2(n, w1);
+  n = win.template at<false>(row + 1, i);  // e2
+  spy = n.tp, sUy = n.tu, yy1 = t1(n, w1), yy2 = t2(n, w1);
+  n = win.template at<false>(row, i - 1);  // e3
+  spx = spx - n.tp, sUx = sUx - n.tu, xx1 = xx1 + t1(n, w1), xx2 = xx2 + t2(n, w1);
+  n = win.template at<false>(row - 1, i);  // e4
+  spy = spy - n.tp, sUy = sUy - n.tu, yy1 = yy1 + t1(n, w1), yy2 = yy2 + t2(n, w1);
+  n = win.template at<true>(row + 1, i + 1);  // e5
+  V a = t1(n, w2), b = t2(n, w2);
+  spx = spx + n.tp, sUx = sUx + n.tu, spy = spy + n.tp, sUy = sUy + n.tu;
+  xx1 = xx1 + a, xx2 = xx2 + b, yy1 = yy1 + a, yy2 = yy2 + b, xy1 = a, xy2 = b;
+  n = win.template at<true>(row + 1, i - 1);  // e6
+  a = t1(n, w2), b = t2(n, w2);
+  spx = spx - n.tp, sUx = sUx - n.tu, spy = spy + n.tp, sUy = sUy + n.tu;
+  xx1 = xx1 + a, xx2 = xx2 + b, yy1 = yy1 + a, yy2 = yy2 + b, xy1 = xy1 - a, xy2 = xy2 - b;
+  n = win.template at<true>(row - 1, i - 1);  // e7
+  a = t1(n, w2), b = t2(n, w2);
+  spx = spx - n.tp, sUx = sUx - n.tu, spy = spy - n.tp, sUy = sUy - n.tu;
+  xx1 = xx1 + a, xx2 = xx2 + b, yy1 = yy1 + a, yy2 = yy2 + b, xy1 = xy1 + a, xy2 = xy2 + b;
+  n = win.template at<true>(row - 1, i + 1);  // e8
+  a = t1(n, w2), b = t2(n, w2);
+  spx = spx + n.tp, sUx = sUx + n.tu, spy = spy - n.tp, sUy = sUy - n.tu;
+  xx1 = xx1 + a, xx2 = xx2 + b, yy1 = yy1 + a, yy2 = yy2 + b, xy1 = xy1 - a, xy2 = xy2 - b;
+  const V c1 = bc(m.omA) * n0.p, c2 = bc(m.c2), pre = bc(m.pre);
+  Fx = c1 * spx - bc(m.A) * sUx;
+  Fy = c1 * spy - bc(m.A) * sUy;
+  if (m.wetting == LBM_WET_MARTYS_CHEN) Fy = Fy - (bc(m.Gw) * n0.p) * bc(ss);
+  Qxx = pre * (c1 * xx1 + c2 * xx2);
+  Qyy = pre * (c1 * yy1 + c2 * yy2);
+  Qxy = pre * (c1 * xy1 + c2 * xy2);
+}
+
+// Momenta j_x, j_y, left to right in f_0 .. f_8 (also the first terms of q_x, q_y).
+template <class V>
+__device__ __forceinline__ void momentum(const V (&f)[9], V &d13, V &d24, V &jx, V &jy) {
+  d13 = f[1] - f[3];
+  d24 = f[2] - f[4];
+  jx = (((d13 + f[5]) - f[6]) - f[7]) + f[8];
+  jy = (((d24 + f[5]) + f[6]) - f[7]) - f[8];
+}
+
+// MRT collision of the node(s) at window row `row`, entry i; f: populations,
+// rho: density, fs: post-collision populations.
 template <class V, class R, class W>
 __device__ __forceinline__ void collide(const Canon<R> &m, const W &win, int row, int i, const V (&f)[9], V rho,
                                         R ss, V (&fs)[9]) {
   auto bc = [](R c) { return Val<V>::bc(c); };
-  const V w1 = bc((R)1 / (R)3), w2 = bc((R)1 / (R)12);
-  V Fx, Fy, Qxx, Qyy, Qxy;
-  {
-    const Nb<V> n0 = win.template at<false>(row, i);
-    V spx, spy, sUx, sUy, xx1, yy1, xy1, xx2, yy2, xy2;
-    auto t1 = [&](const Nb<V> &n, V w) { return w * (n.p - n0.p); };
-    auto t2 = [&](const Nb<V> &n, V w) { return w * (n.p2 - n0.p2); };
-    Nb<V> n = win.template at<false>(row, i + 1);  // e1
-    spx = n.tp, sUx = n.tu, xx1 = t1(n, w1), xx2 = t2(n, w1);
-    n = win.template at<false>(row + 1, i);  // e2
-    spy = n.tp, sUy = n.tu, yy1 = t1(n, w1), yy2 = t2(n, w1);
-    n = win.template at<false>(row, i - 1);  // e3
-    spx = spx - n.tp, sUx = sUx - n.tu, xx1 = xx1 + t1(n, w1), xx2 = xx2 + t2(n, w1);
-    n = win.template at<false>(row - 1, i);  // e4
-    spy = spy - n.tp, sUy = sUy - n.tu, yy1 = yy1 + t1(n, w1), yy2 = yy2 + t2(n, w1);
-    n = win.template at<true>(row + 1, i + 1);  // e5
-    V a = t1(n, w2), b = t2(n, w2);
-    spx = spx + n.tp, sUx = sUx + n.tu, spy = spy + n.tp, sUy = sUy + n.tu;
-    xx1 = xx1 + a, xx2 = xx2 + b, yy1 = yy1 + a, yy2 = yy2 + b, xy1 = a, xy2 = b;
-    n = win.template at<true>(row + 1, i - 1);  // e6
-    a = t1(n, w2), b = t2(n, w2);
-    spx = spx - n.tp, sUx = sUx - n.tu, spy = spy + n.tp, sUy = sUy + n.tu;
-    xx1 = xx1 + a, xx2 = xx2 + b, yy1 = yy1 + a, yy2 = yy2 + b, xy1 = xy1 - a, xy2 = xy2 - b;
-    n = win.template at<true>(row - 1, i - 1);  // e7
-    a = t1(n, w2), b = t2(n, w2);
-    spx = spx - n.tp, sUx = sUx - n.tu, spy = spy - n.tp, sUy = sUy - n.tu;
-    xx1 = xx1 + a, xx2 = xx2 + b, yy1 = yy1 + a, yy2 = yy2 + b, xy1 = xy1 + a, xy2 = xy2 + b;
-    n = win.template at<true>(row - 1, i + 1);  // e8
-    a = t1(n, w2), b = t2(n, w2);
-    spx = spx + n.tp, sUx = sUx + n.tu, spy = spy - n.tp, sUy = sUy - n.tu;
-    xx1 = xx1 + a, xx2 = xx2 + b, yy1 = yy1 + a, yy2 = yy2 + b, xy1 = xy1 - a, xy2 = xy2 - b;
-    const V c1 = bc(m.omA) * n0.p, c2 = bc(m.c2), pre = bc(m.pre);
-    Fx = c1 * spx - bc(m.A) * sUx;
-    Fy = c1 * spy - bc(m.A) * sUy;
-    if (m.wetting == LBM_WET_MARTYS_CHEN) Fy = Fy - (bc(m.Gw) * n0.p) * bc(ss);
-    Qxx = pre * (c1 * xx1 + c2 * xx2);
-    Qyy = pre * (c1 * yy1 + c2 * yy2);
-    Qxy = pre * (c1 * xy1 + c2 * xy2);
-  }
+  V Fx, Fy, Qxx, Qyy, Qxy, d13, d24, jx, jy;
+  force(m, win, row, i, ss, Fx, Fy, Qxx, Qyy, Qxy);
+  momentum(f, d13, d24, jx, jy);
   const V half = bc((R)0.5), two = bc((R)2), m2 = bc((R)-2), four = bc((R)4), m4 = bc((R)-4), quarter = bc((R)0.25);
   // moments (rho is the first), left to right in f_0 .. f_8
-  const V d13 = f[1] - f[3], d24 = f[2] - f[4];
   V me = vfma(m4, f[0], -f[1]);
   me = ((me - f[2]) - f[3]) - f[4];
   me = vfma(two, f[8], vfma(two, f[7], vfma(two, f[6], vfma(two, f[5], me))));
   V mp = ((vfma(two, f[0], -f[1]) - f[2]) - f[3]) - f[4];  // half of 4 f_0 - 2 f_1 - ...
   mp = ((vfma(two, mp, f[5]) + f[6]) + f[7]) + f[8];
-  const V jx = (((d13 + f[5]) - f[6]) - f[7]) + f[8];
-  const V jy = (((d24 + f[5]) + f[6]) - f[7]) - f[8];
   const V qx = ((vfma(m2, d13, f[5]) - f[6]) - f[7]) + f[8];
   const V qy = ((vfma(m2, d24, f[5]) + f[6]) - f[7]) - f[8];
   const V nn = ((f[1] - f[2]) + f[3]) - f[4];
@@ -313,13 +330,128 @@ __device__ __forceinline__ void collide(const Canon<R> &m, const W &win, int row
   fs[8] = vfma(mq, r8, (dp - r5) - r6);
 }
 
+// Outputs of the kernel below: Step writes the state after the step, Speed the largest |u|^2 (as the bits
+// of a non-negative double, which order like the number), Fields the fields.
+template <class R>
+struct Step {
+  R *f;
+};
+struct Speed {
+  unsigned long long *max2;
+};
+struct Fields {
+  double *o[10];  // rho, psi, U, ux, uy, Fx, Fy, Qxx, Qyy, Qxy; NULL where not wanted
+};
+
+// What a CTA does with its window, per output.
+template <class V, int R, class real>
+__device__ __forceinline__ void emit(const Canon<real> &m, const Step<real> &out, const Window<V, R> &win,
+                                     const real (&)[R + 2][Val<V>::N * kH + 4], int w, int lane, int, int y, int x0,
+                                     const bool (&act)[Val<V>::N], bool node, bool, real ss, const V (&f)[9], V r) {
+  constexpr int N = Val<V>::N;
+  if (!node) return;
+  const size_t n = (size_t)m.nx * m.ny;
+  const bool dn = m.walls && y == 1, up = m.walls && y == m.ny - 2;
+  V fs[9];
+  collide(m, win, w, lane + 2, f, r, ss, fs);
+  // streaming with half-way bounce-back
+  const size_t ry = (size_t)y * m.nx, rd = (size_t)(y == 0 ? m.ny - 1 : y - 1) * m.nx,
+               ru = (size_t)(y == m.ny - 1 ? 0 : y + 1) * m.nx;
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    if (!act[j]) break;
+    const int x = x0 + lane + j * kH, xm = x == 0 ? m.nx - 1 : x - 1, xp = x == m.nx - 1 ? 0 : x + 1;
+    auto g = [&](int a) { return Val<V>::lane(fs[a], j); };
+    real *const o = out.f;
+    o[ry + x] = g(0);
+    o[n + ry + xp] = g(1);
+    o[3 * n + ry + xm] = g(3);
+    o[(up ? 4 * n + ry : 2 * n + ru) + x] = g(2);
+    o[up ? 7 * n + ry + x : 5 * n + ru + xp] = g(5);
+    o[up ? 8 * n + ry + x : 6 * n + ru + xm] = g(6);
+    o[(dn ? 2 * n + ry : 4 * n + rd) + x] = g(4);
+    o[dn ? 5 * n + ry + x : 7 * n + rd + xm] = g(7);
+    o[dn ? 6 * n + ry + x : 8 * n + rd + xp] = g(8);
+  }
+}
+
+// |u|^2 in double of the velocity in the kernel's precision, as lbm_get_u gives
+// it; its largest value, the square root of which is the largest |u| (both are
+// monotone).  FP32: only nodes near the largest of their warp in single
+// precision go through the FP64 pipe.
+template <class V, int R, class real>
+__device__ __forceinline__ void emit(const Canon<real> &m, const Speed &out, const Window<V, R> &win,
+                                     const real (&)[R + 2][Val<V>::N * kH + 4], int w, int lane, int, int, int,
+                                     const bool (&act)[Val<V>::N], bool node, bool, real ss, const V (&f)[9], V r) {
+  constexpr int N = Val<V>::N;
+  V Fx, Fy, Qxx, Qyy, Qxy, d13, d24, jx, jy;
+  if (node) {
+    force(m, win, w, lane + 2, ss, Fx, Fy, Qxx, Qyy, Qxy);
+    momentum(f, d13, d24, jx, jy);
+    const V half = Val<V>::bc((real)0.5);
+    Fx = vfma(half, Fx, jx) / r;
+    Fy = vfma(half, Fy, jy) / r;
+  }
+  float near[N], top = 0.0f;
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    const float ux = node && act[j] ? (float)Val<V>::lane(Fx, j) : 0.0f;
+    const float uy = node && act[j] ? (float)Val<V>::lane(Fy, j) : 0.0f;
+    near[j] = ux * ux + uy * uy;
+    top = fmaxf(top, near[j]);  // (NaN counts for nothing)
+  }
+  for (int o = 16; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+  const float lim = top > 1e-30f ? top * 0.99999f : 0.0f;  // (below, squares lose their precision)
+#pragma unroll
+  for (int j = 0; j < N; ++j)
+    if (node && act[j] && near[j] >= lim) {
+      const double ux = (double)Val<V>::lane(Fx, j), uy = (double)Val<V>::lane(Fy, j);
+      const unsigned long long s = (unsigned long long)__double_as_longlong(ux * ux + uy * uy);
+      if (s > *(volatile unsigned long long *)out.max2) atomicMax(out.max2, s);
+    }
+}
+
+// The fields as doubles; solid rows (written by the tile beside them) carry their
+// ghost rho, psi, U and zeros.
+template <class V, int R, class real>
+__device__ __forceinline__ void emit(const Canon<real> &m, const Fields &out, const Window<V, R> &win,
+                                     const real (&wrho)[R + 2][Val<V>::N * kH + 4], int w, int lane, int, int y,
+                                     int x0, const bool (&act)[Val<V>::N], bool node, bool solid, real ss,
+                                     const V (&f)[9], V r) {
+  constexpr int N = Val<V>::N;
+  if (!node && !solid) return;
+  V v[7];
+#pragma unroll
+  for (int k = 0; k < 7; ++k) v[k] = Val<V>::bc((real)0);
+  if (node) {
+    V d13, d24, jx, jy;
+    force(m, win, w, lane + 2, ss, v[2], v[3], v[4], v[5], v[6]);
+    momentum(f, d13, d24, jx, jy);
+    const V half = Val<V>::bc((real)0.5);
+    v[0] = vfma(half, v[2], jx) / r;
+    v[1] = vfma(half, v[3], jy) / r;
+  }
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    if (!act[j]) break;
+    const size_t i = (size_t)y * m.nx + x0 + lane + j * kH;
+    const bool ghost = solid && m.wetting != LBM_WET_MARTYS_CHEN;
+    if (out.o[0]) out.o[0][i] = (double)(node || ghost ? wrho[w][lane + j * kH + 2] : (real)0);
+    if (out.o[1]) out.o[1][i] = (double)Val<V>::lane(win.p[w][lane + 2], j);
+    if (out.o[2]) out.o[2][i] = (double)Val<V>::lane(win.u[w][lane + 2], j);
+#pragma unroll
+    for (int k = 0; k < 7; ++k)
+      if (out.o[3 + k]) out.o[3 + k][i] = (double)Val<V>::lane(v[k], j);
+  }
+}
+
 // Tile of m.sw columns x R rows per CTA of R + 3 warps: warps 0 .. R + 1 each
 // load one row (the tile's, the one above, the one below), the last one the
 // columns beside the tile.  Window row w holds row y0 - 1 + w.
-template <class V, int R>
+template <class V, int R, class OUT>
 __global__ void __launch_bounds__((R + 3) * 32)
-    k_canon(Canon<typename Val<V>::R> m, const typename Val<V>::R *__restrict__ fin,
-            typename Val<V>::R *__restrict__ fout, const double *__restrict__ coef, int *flag) {
+    k_canon(Canon<typename Val<V>::R> m, const typename Val<V>::R *__restrict__ fin, OUT out,
+            const double *__restrict__ coef, int *flag) {
   typedef typename Val<V>::R real;
   constexpr int N = Val<V>::N;
   static_assert(2 * (R + 2) + 4 <= 32, "one warp loads the columns beside the tile");
@@ -406,43 +538,24 @@ __global__ void __launch_bounds__((R + 3) * 32)
       for (int j = 0; j < N; ++j) {
         if (row_warp ? act[j] : j == 0) {
           const int c = row_warp ? lane + j * kH : hc;
-          real psi, U;
-          ghost(m, q1[c + 1], q1[c + 2], q1[c + 3], q2[c + 2], (real)kc[j], psi, U);
+          real g, psi, U;
+          ghost(m, q1[c + 1], q1[c + 2], q1[c + 3], q2[c + 2], (real)kc[j], g, psi, U);
           win.put(w, c, psi, U);
+          if (std::is_same<OUT, Fields>::value) wrho[w][c + 2] = g;
         }
       }
     }
     __syncthreads();
   }
   if (__any_sync(0xffffffffu, bad) && lane == 0 && *(volatile int *)flag == 0) atomicOr(flag, 1);
-  if (warp < 1 || warp > nr || !act[0]) return;
-
   const bool dn = m.walls && y == 1, up = m.walls && y == m.ny - 2;
-  V fs[9];
-  collide(m, win, w, lane + 2, f, r, dn ? m.ss_dn : (up ? m.ss_up : (real)0), fs);
-  // streaming with half-way bounce-back
-  const size_t ry = (size_t)y * m.nx, rd = (size_t)(y == 0 ? m.ny - 1 : y - 1) * m.nx,
-               ru = (size_t)(y == m.ny - 1 ? 0 : y + 1) * m.nx;
-#pragma unroll
-  for (int j = 0; j < N; ++j) {
-    if (!act[j]) break;
-    const int x = x0 + lane + j * kH, xm = x == 0 ? m.nx - 1 : x - 1, xp = x == m.nx - 1 ? 0 : x + 1;
-    auto g = [&](int a) { return Val<V>::lane(fs[a], j); };
-    real *o = fout;
-    o[ry + x] = g(0);
-    o[n + ry + xp] = g(1);
-    o[3 * n + ry + xm] = g(3);
-    o[(up ? 4 * n + ry : 2 * n + ru) + x] = g(2);
-    o[up ? 7 * n + ry + x : 5 * n + ru + xp] = g(5);
-    o[up ? 8 * n + ry + x : 6 * n + ru + xm] = g(6);
-    o[(dn ? 2 * n + ry : 4 * n + rd) + x] = g(4);
-    o[dn ? 5 * n + ry + x : 7 * n + rd + xm] = g(7);
-    o[dn ? 6 * n + ry + x : 8 * n + rd + xp] = g(8);
-  }
+  const real ss = dn ? m.ss_dn : (up ? m.ss_up : (real)0);
+  const bool node = warp >= 1 && warp <= nr && act[0];
+  emit(m, out, win, wrho, w, lane, warp, y, x0, act, node, solid && row_warp && on, ss, f, r);
 }
 
-template <class V, int R>
-cudaError_t launch(const lbm_ctx *C, const void *src, void *dst) {
+template <class V, int R, class OUT>
+cudaError_t launch(const lbm_ctx *C, const void *src, OUT out) {
   typedef typename Val<V>::R real;
   Canon<real> m(C);
   const int W = Val<V>::N * kH;
@@ -450,7 +563,7 @@ cudaError_t launch(const lbm_ctx *C, const void *src, void *dst) {
   m.sw = Val<V>::N == 1 ? (C->nx + m.strips - 1) / m.strips : W;
   const int nrows = C->walls ? C->ny - 2 : C->ny;
   const unsigned grid = (unsigned)m.strips * (unsigned)((nrows + R - 1) / R);
-  k_canon<V, R><<<grid, (R + 3) * 32, 0, C->stream>>>(m, (const real *)src, (real *)dst, C->d_coef, C->d_flag);
+  k_canon<V, R, OUT><<<grid, (R + 3) * 32, 0, C->stream>>>(m, (const real *)src, out, C->d_coef, C->d_flag);
   return cudaGetLastError();
 }
 
@@ -464,6 +577,25 @@ cudaError_t launch(const lbm_ctx *C, const void *src, void *dst) {
 // 79.1, 800 x 400 253 / 230 us.
 cudaError_t lbm_canon_step(const lbm_ctx *C, const void *src, void *dst, unsigned long long *launches) {
   ++*launches;
-  if (C->precision == 32) return launch<F2, 4>(C, src, dst);
-  return (long long)C->nx * C->ny < 80000 ? launch<double, 2>(C, src, dst) : launch<double, 8>(C, src, dst);
+  if (C->precision == 32) return launch<F2, 4>(C, src, Step<float>{(float *)dst});
+  const Step<double> out{(double *)dst};
+  return (long long)C->nx * C->ny < 80000 ? launch<double, 2>(C, src, out) : launch<double, 8>(C, src, out);
+}
+
+// The getters' fields and the largest speed, in one pass over the populations
+// (before: fields, then seven planes of doubles, then the reduction of two of
+// them).  4096 x 2048: largest speed 590 -> 200 us.
+cudaError_t lbm_canon_fields(const lbm_ctx *C, const void *f, double *const (&o)[10], unsigned long long *launches) {
+  ++*launches;
+  Fields out;
+  for (int k = 0; k < 10; ++k) out.o[k] = o[k];
+  return C->precision == 32 ? launch<F2, 4>(C, f, out) : launch<double, 4>(C, f, out);
+}
+
+cudaError_t lbm_canon_max_speed2(const lbm_ctx *C, const void *f, double *max2, unsigned long long *launches) {
+  ++*launches;
+  const cudaError_t e = cudaMemsetAsync(max2, 0, sizeof(double), C->stream);
+  if (e != cudaSuccess) return e;
+  const Speed out{(unsigned long long *)max2};
+  return C->precision == 32 ? launch<F2, 4>(C, f, out) : launch<double, 4>(C, f, out);
 }

@@ -59,13 +59,13 @@ struct lbm_ctx {
   double *d_coef;        // 4*nx: c_bot, c_top, cot_bot, cot_top
   double *d_dcoef;       // 4*nx: their derivatives in theta (adjoint)
   struct lbm_tape *tape; // adjoint record (lbm_adjoint.cu); NULL when none
-  int *d_flag;           // [0]: instability, [1]: timeout, [2]: lbm_set_rho input check
+  int *d_flag;           // [0]: instability, [1]: timeout, [2]: lbm_set_rho input check, [3]: arrivals of a reduction
   double *d_rho64;       // nx*ny, measurement density
   cudaStream_t xfer;     // lbm_get_rho: copy stream and its chunk events (lazy; NULL until first needed)
   cudaEvent_t xfer_ev[8];
-  void *d_fields;        // 3*nx*ny reals: rho, psi, U (getters, adjoint; lazy)
-  double *d_aux;         // 7*nx*ny doubles for lbm_get_u / lbm_get_fields (lazy)
-  double *d_red;         // reduction partials
+  void *d_fields;        // 3*nx*ny reals: rho, psi, U (FP64 adjoint; lazy)
+  double *d_aux;         // 8*nx*ny doubles for lbm_get_u / lbm_get_fields (lazy)
+  double *d_red;         // reduction partials (red_len)
   double *d_res;         // small results
   int red_len;
   // fused kernel plan
@@ -88,9 +88,8 @@ struct lbm_ctx {
 // ---- lbm_ref.cu: fields and initial states in the canonical order -----------
 // All launchers return the cudaError_t of the launch and add the number of
 // kernels launched to *launches.
-cudaError_t lbm_ref_fields(const lbm_ctx *C, const void *f, void *fields, unsigned long long *launches);
-cudaError_t lbm_ref_macro(const lbm_ctx *C, const void *f, const void *fields, double *out7,
-                          unsigned long long *launches);
+// rho, psi, U of an FP64 state, ghost values included (the adjoint's reverse step)
+cudaError_t lbm_ref_fields(const lbm_ctx *C, const double *f, double *fields, unsigned long long *launches);
 // f := f_eq(rho, 0) from device or mapped host densities; with bad != NULL,
 // *bad |= 1 if a fluid-node density is not finite or not > 0 (bad zeroed by
 // the caller; f is written all the same)
@@ -100,6 +99,11 @@ cudaError_t lbm_ref_droplets(const lbm_ctx *C, int n, const double *drop, double
 
 // ---- lbm_canon.cu: one step in the canonical evaluation order ---------------
 cudaError_t lbm_canon_step(const lbm_ctx *C, const void *src, void *dst, unsigned long long *launches);
+// Fields of the state f as doubles, [ny][nx] each: rho, psi, U (ghost values on
+// the solid rows), ux, uy, Fx, Fy, Qxx, Qyy, Qxy (0 there); NULL: not wanted.
+cudaError_t lbm_canon_fields(const lbm_ctx *C, const void *f, double *const (&o)[10], unsigned long long *launches);
+// Largest |u|^2 over the fluid nodes.
+cudaError_t lbm_canon_max_speed2(const lbm_ctx *C, const void *f, double *max2, unsigned long long *launches);
 
 // ---- lbm_fused.cu: single-pass FP32 step ------------------------------------
 int lbm_fused_plan(lbm_ctx *C);  // sets fused_ok, tile_*, tensor maps
@@ -121,9 +125,30 @@ cudaError_t lbm_rho64(const lbm_ctx *C, const void *f, double *rho, unsigned lon
 cudaError_t lbm_rho64_rows(const lbm_ctx *C, const void *f, double *rho, int row0, int row1,
                            unsigned long long *launches);
 // sum of rows [row0, row1) of a node field, in a fixed order
-cudaError_t lbm_reduce_rows(const lbm_ctx *C, const double *v, int row0, int row1, double *partial, int npart,
-                            double *res, unsigned long long *launches);
-cudaError_t lbm_reduce_max_speed(const lbm_ctx *C, const double *ux, const double *uy, double *partial,
-                                 int npart, double *res, unsigned long long *launches);
-cudaError_t lbm_angle(const lbm_ctx *C, const double *rho, int wall, int x0, int x1, double rho_mid, double *res,
-                      unsigned long long *launches);
+cudaError_t lbm_reduce_rows(const lbm_ctx *C, const double *v, int row0, int row1, double *res,
+                            unsigned long long *launches);
+// sum of rho over the fluid nodes of a state
+cudaError_t lbm_mass_of(const lbm_ctx *C, const void *f, double *res, unsigned long long *launches);
+// Apparent contact angle of the droplet on `wall` in columns [x0, x1) of the
+// state f: the kernel finds where the contour cuts the boundary row and the
+// centre column, lbm_angle_of interpolates there.
+struct lbm_angle_cut {
+  int contact, xl, xr, steps;  // cuts right of xl and of xr, and above row `steps` from the boundary row
+  double rho[6];               // at xl, xl + 1; xr, xr + 1; the last liquid node up the centre column, the next
+};
+struct lbm_angle_args {
+  const void *f;
+  int nx, ny, wall, x0, x1;
+  double rho_mid;
+  double *partial;    // scratch: a row of x1 - x0 doubles per 64 rows
+  unsigned *counter;  // 0 before and after
+  lbm_angle_cut *res;
+};
+lbm_angle_args lbm_make_angle_args(const lbm_ctx *C, int wall, int x0, int x1, void *res);
+// LBM_OK with the angle, height and base width, or LBM_ENOCONTACT
+int lbm_angle_of(const lbm_angle_cut &r, double rho_mid, double *theta, double *H, double *L);
+int lbm_angle_blocks(const lbm_angle_args &A);
+cudaError_t lbm_angle(const lbm_ctx *C, const lbm_angle_args &A, unsigned long long *launches);
+// the same for entries [first, first + count) (at most 65535) of a device table
+// of FP32 domains; blocks: the largest lbm_angle_blocks among them
+cudaError_t lbm_angle_many(const lbm_angle_args *tab, int first, int count, int blocks, cudaStream_t stream);

@@ -8,6 +8,8 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "lbm_internal.h"
 
 namespace {
@@ -117,79 +119,112 @@ __device__ __forceinline__ double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
   return v;
 }
-__device__ __forceinline__ double warp_max(double v) {
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_down_sync(0xffffffffu, v, o));
-  return v;
-}
 
-// Stage 1: block b sums the fluid part of a fixed contiguous chunk; stage 2:
-// one block sums the partials.  Both stages use a fixed tree, so the result
-// does not depend on scheduling.
-__global__ void k_sum_partial(const double *__restrict__ v, size_t n, size_t y0, size_t y1, int nx,
-                              double *__restrict__ partial) {
-  __shared__ double sh[32];
-  size_t lo = y0 * nx, hi = y1 * nx;
-  size_t len = hi - lo, chunk = (len + gridDim.x - 1) / gridDim.x;
-  size_t b0 = lo + blockIdx.x * chunk, b1 = min(hi, b0 + chunk);
-  double s = 0.0;
-  for (size_t i = b0 + threadIdx.x; i < b1; i += blockDim.x) s += v[i];
+// Sum over the block (<= 1024 threads), valid in thread 0; a fixed tree.
+__device__ __forceinline__ double block_sum(double s, double *sh) {
   s = warp_sum(s);
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
   __syncthreads();
-  if (threadIdx.x < 32) {
-    double t = threadIdx.x < (blockDim.x >> 5) ? sh[threadIdx.x] : 0.0;
-    t = warp_sum(t);
-    if (threadIdx.x == 0) partial[blockIdx.x] = t;
-  }
+  double t = 0.0;
+  if (threadIdx.x < 32) t = warp_sum(threadIdx.x < (blockDim.x >> 5) ? sh[threadIdx.x] : 0.0);
+  __syncthreads();
+  return t;
 }
 
-__global__ void k_sum_final(const double *__restrict__ partial, int np, double *__restrict__ out) {
+// True in every thread of the block that arrives last of nb at *counter (which
+// it leaves at 0): it then sees what the others wrote before arriving.
+__device__ __forceinline__ bool arrives_last(unsigned *counter, unsigned nb) {
+  __shared__ bool last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    last = atomicAdd(counter, 1u) == nb - 1u;
+    if (last) *counter = 0u;
+  }
+  __syncthreads();
+  if (last) __threadfence();
+  return last;
+}
+
+// Sum of val(i), i in [i0, i1), in a fixed order: block b sums a contiguous
+// chunk, the last block to arrive the chunks' sums.
+template <class Val>
+__device__ __forceinline__ void sum_range(size_t i0, size_t i1, double *partial, unsigned *counter, double *out,
+                                          Val val) {
   __shared__ double sh[32];
+  const size_t len = i1 - i0, chunk = (len + gridDim.x - 1) / gridDim.x;
+  const size_t b0 = i0 + blockIdx.x * chunk, b1 = min(i1, b0 + chunk);
   double s = 0.0;
-  for (int i = threadIdx.x; i < np; i += blockDim.x) s += partial[i];
-  s = warp_sum(s);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double t = threadIdx.x < (blockDim.x >> 5) ? sh[threadIdx.x] : 0.0;
-    t = warp_sum(t);
-    if (threadIdx.x == 0) out[0] = t;
-  }
+  for (size_t i = b0 + threadIdx.x; i < b1; i += blockDim.x) s += val(i);
+  s = block_sum(s, sh);
+  if (threadIdx.x == 0) partial[blockIdx.x] = s;
+  if (!arrives_last(counter, gridDim.x)) return;
+  s = 0.0;
+  for (unsigned i = threadIdx.x; i < gridDim.x; i += blockDim.x) s += __ldcg(partial + i);
+  s = block_sum(s, sh);
+  if (threadIdx.x == 0) out[0] = s;
 }
 
-__global__ void k_speed_partial(const double *__restrict__ ux, const double *__restrict__ uy, size_t y0, size_t y1,
-                                int nx, double *__restrict__ partial) {
-  __shared__ double sh[32];
-  size_t lo = y0 * nx, hi = y1 * nx;
-  size_t len = hi - lo, chunk = (len + gridDim.x - 1) / gridDim.x;
-  size_t b0 = lo + blockIdx.x * chunk, b1 = min(hi, b0 + chunk);
-  double m = 0.0;
-  for (size_t i = b0 + threadIdx.x; i < b1; i += blockDim.x) m = fmax(m, sqrt(ux[i] * ux[i] + uy[i] * uy[i]));
-  m = warp_max(m);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double t = threadIdx.x < (blockDim.x >> 5) ? sh[threadIdx.x] : 0.0;
-    t = warp_max(t);
-    if (threadIdx.x == 0) partial[blockIdx.x] = t;
-  }
+__global__ void k_sum(const double *__restrict__ v, size_t i0, size_t i1, double *partial, unsigned *counter,
+                      double *out) {
+  sum_range(i0, i1, partial, counter, out, [&](size_t i) { return v[i]; });
 }
 
-__global__ void k_max_final(const double *__restrict__ partial, int np, double *__restrict__ out) {
-  __shared__ double sh[32];
-  double m = 0.0;
-  for (int i = threadIdx.x; i < np; i += blockDim.x) m = fmax(m, partial[i]);
-  m = warp_max(m);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double t = threadIdx.x < (blockDim.x >> 5) ? sh[threadIdx.x] : 0.0;
-    t = warp_max(t);
-    if (threadIdx.x == 0) out[0] = t;
-  }
+// rho = sum_a f_a in double, left to right, at node i.
+__device__ __forceinline__ double node_rho64(const float *__restrict__ f, size_t n, size_t i) {
+  float v[9];
+#pragma unroll
+  for (int a = 0; a < 9; ++a) v[a] = f[a * n + i];
+  return sum9(v);
+}
+__device__ __forceinline__ double node_rho64(const double *__restrict__ f, size_t n, size_t i) {
+  double r = 0.0;
+#pragma unroll
+  for (int a = 0; a < 9; ++a) r = r + f[a * n + i];
+  return r;
 }
 
-// Block-wide reductions of one int / one (value, index) pair.
+// Total mass of the nodes [i0, i1) straight from the populations (the density
+// field does not go through memory: 36 bytes a node instead of 52).
+template <typename R>
+__global__ void k_mass(const R *__restrict__ f, size_t n, size_t i0, size_t i1, double *partial, unsigned *counter,
+                       double *out) {
+  sum_range(i0, i1, partial, counter, out, [&](size_t i) { return node_rho64(f, n, i); });
+}
+
+// s + e += v for lane pairs, without loss: e takes the rounding error of the sum
+// (Knuth's two-sum).
+__device__ __forceinline__ void two_sum(float2 &s, float2 &e, float2 v) {
+  const float2 m1 = make_float2(-1.0f, -1.0f);
+  const float2 t = __fadd2_rn(s, v), b = __ffma2_rn(s, m1, t);
+  e = __fadd2_rn(e, __fadd2_rn(__ffma2_rn(__ffma2_rn(b, m1, t), m1, s), __ffma2_rn(b, m1, v)));
+  s = t;
+}
+
+// The same for four nodes at once (nx % 4 == 0; groups [q0, q1)): 16-byte loads,
+// and per group a sum in single precision with its rounding errors beside it (48
+// bits), which takes a fifth of the instructions of nine exact sums: 4096 x 2048
+// 134 us (density field and sum) -> 60 us; the populations alone take 45.
+__global__ void k_mass_x4(const float4 *__restrict__ f, size_t n4, size_t q0, size_t q1, double *partial,
+                          unsigned *counter, double *out) {
+  sum_range(q0, q1, partial, counter, out, [&](size_t i) {
+    float4 v[9];
+#pragma unroll
+    for (int a = 0; a < 9; ++a) v[a] = f[a * n4 + i];
+    float2 s = make_float2(v[0].x, v[0].y), e = make_float2(0.0f, 0.0f);
+#pragma unroll
+    for (int a = 1; a < 9; ++a) two_sum(s, e, make_float2(v[a].x, v[a].y));
+#pragma unroll
+    for (int a = 0; a < 9; ++a) two_sum(s, e, make_float2(v[a].z, v[a].w));
+    // (an infinite or NaN sum stands by itself)
+    float2 lo = make_float2(s.y, 0.0f), le = make_float2(0.0f, 0.0f);
+    two_sum(lo, le, make_float2(s.x, 0.0f));
+    const float err = (e.x + e.y) + le.x;
+    return (double)lo.x + (fabsf(err) <= FLT_MAX ? (double)err : 0.0);
+  });
+}
+
+// Block-wide minimum or maximum of one int, in every thread.
 __device__ int block_reduce_int(int v, bool is_max, int *sh) {
   for (int o = 16; o > 0; o >>= 1) {
     int u = __shfl_down_sync(0xffffffffu, v, o);
@@ -211,80 +246,214 @@ __device__ int block_reduce_int(int v, bool is_max, int *sh) {
   return sh[32];
 }
 
-// One block per call.  res = {theta, H, L, xc, status}.
-__global__ void k_angle(const double *__restrict__ rho, int nx, int ny, int wall, int x0, int x1, double rho_mid,
-                        double *__restrict__ res) {
-  __shared__ double shv[33];
-  __shared__ int shi[33];
-  int ylo = wall == 0 ? 1 : ny / 2, yhi = wall == 0 ? ny / 2 : ny - 1;
-  int base = wall == 0 ? 1 : ny - 2, dir = wall == 0 ? 1 : -1;
-  // column sums over the wall's half, each summed bottom to top
-  double best = -DBL_MAX;
-  int bx = INT_MAX;
-  for (int x = x0 + threadIdx.x; x < x1; x += blockDim.x) {
+// ---- apparent contact angle ---------------------------------------------------
+// The centre column is the one with the largest sum over the wall's half, each
+// sum taken bottom to top, one addition after the other: a chain that no single
+// block shortens (1023 rows: 198 us, after 110 us for the densities of the
+// whole field).  Here all blocks sum chunks of rows in parallel, which places
+// every column's sum within a proven distance of the sequential one; only
+// columns within twice that distance of the largest (nearly always one) still
+// need the sequential sum to tell them apart, and the last block takes it.
+// Everything else (the boundary row's liquid run, the walk up the centre column)
+// reads its densities straight from the populations.  The last block's phases
+// follow one another, so they are kept short: comparisons of positive doubles
+// are made on their bits (an FP64 instruction of a warp takes 64 cycles), and
+// the few divisions and the arc tangent are left to the host.
+
+constexpr int kACols = 32, kALanes = 8, kARows = 64;  // columns, row lanes, rows of a block
+constexpr int kAThreads = kACols * kALanes;
+constexpr int kAFew = 16;  // candidates evaluated one after the other by the whole block
+
+__device__ __forceinline__ long long bits(double v) { return __double_as_longlong(v); }
+constexpr long long kInfBits = 0x7ff0000000000000ll;
+// v >= lim for lim > 0 (false for NaN): numbers order like their bits, negative
+// ones below, NaNs above infinity
+__device__ __forceinline__ bool at_least(double v, long long lim) { return bits(v) >= lim && bits(v) <= kInfBits; }
+
+// One copy of the density's code for the last block, which runs through its
+// phases once: inlined in each, the instructions had to be fetched anew every
+// time (400 x 200: 23 us more).
+template <typename R>
+__device__ __noinline__ double rho_at(const R *f, size_t n, size_t i) {
+  return node_rho64(f, n, i);
+}
+
+__device__ __forceinline__ long long block_max_key(long long k, long long *sh) {
+  for (int o = 16; o > 0; o >>= 1) k = max(k, __shfl_xor_sync(0xffffffffu, k, o));
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = k;
+  __syncthreads();
+  for (int j = 0; j < kAThreads / 32; ++j) k = max(k, sh[j]);
+  return k;
+}
+
+// Blocks (kACols columns x kARows rows) of one domain along x, domains of a
+// table along y (tab == NULL: the one in A).
+template <typename R>
+__global__ void __launch_bounds__(kAThreads) k_angle(lbm_angle_args A, const lbm_angle_args *__restrict__ tab) {
+  if (tab) A = tab[blockIdx.y];
+  const int nx = A.nx, ny = A.ny, wall = A.wall, x0 = A.x0, x1 = A.x1, cols = x1 - x0;
+  const long long mid = bits(A.rho_mid);
+  const R *f = (const R *)A.f;
+  const size_t n = (size_t)nx * ny;
+  const int ylo = wall == 0 ? 1 : ny / 2, yhi = wall == 0 ? ny / 2 : ny - 1, half = yhi - ylo;
+  const int groups = (cols + kACols - 1) / kACols, chunks = (half + kARows - 1) / kARows;
+  if ((int)blockIdx.x >= groups * chunks) return;
+
+  // the block's part of its columns' sums; NaN where a density is negative or
+  // not finite (the bound below is for positive terms)
+  __shared__ double sh[kALanes][kACols];
+  {
+    const int g = (int)blockIdx.x % groups, k = (int)blockIdx.x / groups;
+    const int tx = threadIdx.x % kACols, ty = threadIdx.x / kACols, c = g * kACols + tx;
     double s = 0.0;
-    for (int y = ylo; y < yhi; ++y) s = s + rho[(size_t)y * nx + x];
-    if (s > best || (s == best && x < bx)) { best = s; bx = x; }
-  }
-  // argmax, ties to the lowest column
-  for (int o = 16; o > 0; o >>= 1) {
-    double ov = __shfl_down_sync(0xffffffffu, best, o);
-    int ox = __shfl_down_sync(0xffffffffu, bx, o);
-    if (ov > best || (ov == best && ox < bx)) { best = ov; bx = ox; }
-  }
-  if ((threadIdx.x & 31) == 0) { shv[threadIdx.x >> 5] = best; shi[threadIdx.x >> 5] = bx; }
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    int nw = blockDim.x >> 5;
-    double v = threadIdx.x < nw ? shv[threadIdx.x] : -DBL_MAX;
-    int xx = threadIdx.x < nw ? shi[threadIdx.x] : INT_MAX;
-    for (int o = 16; o > 0; o >>= 1) {
-      double ov = __shfl_down_sync(0xffffffffu, v, o);
-      int ox = __shfl_down_sync(0xffffffffu, xx, o);
-      if (ov > v || (ov == v && ox < xx)) { v = ov; xx = ox; }
+    if (c < cols) {
+      const int ya = ylo + k * kARows, yb = min(yhi, ya + kARows);
+      bool odd = false;
+#pragma unroll 2
+      for (int y = ya + ty; y < yb; y += kALanes) {
+        const double r = node_rho64(f, n, (size_t)y * nx + x0 + c);
+        odd |= (unsigned long long)bits(r) >= (unsigned long long)kInfBits;
+        s += r;
+      }
+      if (odd) s = (double)NAN;
     }
-    if (threadIdx.x == 0) shi[32] = xx;
+    sh[ty][tx] = s;
+    __syncthreads();
+    if (ty == 0 && c < cols) {
+      for (int j = 1; j < kALanes; ++j) s += sh[j][tx];
+      A.partial[(size_t)k * cols + c] = s;
+    }
   }
+  if (!arrives_last(A.counter, (unsigned)(groups * chunks))) return;
+
+  // ---- the last block ----
+  auto rho = [&](int y, int x) { return rho_at(f, n, (size_t)y * nx + x); };
+  __shared__ int shi[33];
+  __shared__ long long shk[kAThreads / 32];
+  // bits of a column's sum (NaN: above kInfBits)
+  auto total = [&](int c) {
+    double s = __ldcg(A.partial + c);
+    for (int k = 1; k < chunks; ++k) s += __ldcg(A.partial + (size_t)k * cols + c);
+    return bits(s);
+  };
+  long long top = -1;
+  for (int c = threadIdx.x; c < cols; c += kAThreads) {
+    const long long t = total(c);
+    if (t <= kInfBits) top = max(top, t);
+  }
+  top = block_max_key(top, shk);
+  // A sum of m positive terms, in any order, is within m 2^-53 of the true one
+  // (relative, to first order), so two sums of a column differ by at most
+  // m 2^-52 or m units in the last place; the largest sequential sum is among
+  // the columns within twice that of the largest of these (here eight times, as
+  // the units halve below a power of two).
+  const long long near = top - (8LL * half + 64LL);
+  // candidates: their first column and their number
+  int first = INT_MAX, count = 0;
+  for (int c = threadIdx.x; c < cols; c += kAThreads)
+    if (total(c) >= near) {
+      first = min(first, c);
+      ++count;
+    }
+  first = block_reduce_int(first, false, shi);
+  __shared__ int found;
+  if (threadIdx.x == 0) found = 0;
   __syncthreads();
-  int xc = shi[32];
-  const double *row = rho + (size_t)base * nx;
-  // liquid run of the boundary row containing xc
-  int jl = INT_MIN, jr = INT_MAX;
-  for (int x = x0 + threadIdx.x; x < x1; x += blockDim.x) {
-    bool vap = !(row[x] >= rho_mid);
-    if (vap && x < xc) jl = max(jl, x);
-    if (vap && x > xc) jr = min(jr, x);
+  if (count) atomicAdd(&found, count);
+  __syncthreads();
+  int xc = INT_MAX;
+  if (found == 1) {
+    xc = x0 + first;
+  } else if (found <= kAFew) {
+    __shared__ int cand[kAFew];
+    __shared__ double line[kAThreads];
+    for (int j = 0, c = first; j < found; ++j) {
+      if (threadIdx.x == 0) cand[j] = c;
+      int next = INT_MAX;
+      for (int q = threadIdx.x; q < cols; q += kAThreads)
+        if (q > c && total(q) >= near) next = min(next, q);
+      c = block_reduce_int(next, false, shi);
+    }
+    double best = -DBL_MAX;
+    for (int j = 0; j < found; ++j) {
+      // sequential sum: densities of 256 rows at a time in parallel, added by one thread
+      double s = 0.0;
+      for (int y = ylo; y < yhi; y += kAThreads) {
+        if (y + (int)threadIdx.x < yhi) line[threadIdx.x] = rho(y + threadIdx.x, x0 + cand[j]);
+        __syncthreads();
+        if (threadIdx.x == 0)
+          for (int k = 0; k < min(kAThreads, yhi - y); ++k) s = s + line[k];
+        __syncthreads();
+      }
+      if (threadIdx.x == 0 && s > best) best = s, xc = x0 + cand[j];  // (ties: the lower column came first)
+    }
+    if (threadIdx.x == 0) shi[0] = xc;
+    __syncthreads();
+    xc = shi[0];
+    __syncthreads();
+  } else {  // many equal columns: a sequential sum per thread
+    __shared__ double shv[kAThreads / 32];
+    double best = -DBL_MAX;
+    for (int c = threadIdx.x; c < cols; c += kAThreads) {
+      if (total(c) < near) continue;
+      double s = 0.0;
+      for (int y = ylo; y < yhi; ++y) s = s + rho(y, x0 + c);
+      if (s > best || (s == best && x0 + c < xc)) best = s, xc = x0 + c;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      const double ov = __shfl_down_sync(0xffffffffu, best, o);
+      const int ox = __shfl_down_sync(0xffffffffu, xc, o);
+      if (ov > best || (ov == best && ox < xc)) best = ov, xc = ox;
+    }
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) shv[threadIdx.x >> 5] = best, shi[threadIdx.x >> 5] = xc;
+    __syncthreads();
+    best = shv[0], xc = shi[0];
+    for (int j = 1; j < kAThreads / 32; ++j)
+      if (shv[j] > best || (shv[j] == best && shi[j] < xc)) best = shv[j], xc = shi[j];
+    __syncthreads();
   }
-  __shared__ int shr[33];
-  jl = block_reduce_int(jl, true, shr);
-  jr = block_reduce_int(jr, false, shr);
-  // first vapour node walking away from the wall along xc
-  int ymax = wall == 0 ? yhi : ylo - 1;
-  int kmin = INT_MAX;
-  int nwalk = wall == 0 ? (ymax - base - 1) : (base - ymax - 1);
-  for (int k = 1 + threadIdx.x; k <= nwalk; k += blockDim.x) {
-    int y = base + k * dir;
-    if (!(rho[(size_t)y * nx + xc] >= rho_mid)) kmin = min(kmin, k);
-  }
-  kmin = block_reduce_int(kmin, false, shr);
-  if (threadIdx.x != 0) return;
-  res[3] = (double)xc;
-  if (!(row[xc] >= rho_mid) || jl == INT_MIN || jr == INT_MAX || kmin == INT_MAX) {
-    res[4] = (double)LBM_ENOCONTACT;
+  lbm_angle_cut *res = A.res;
+  if (xc < x0 || xc >= x1) {  // no column has a sum at all (NaN everywhere)
+    if (threadIdx.x == 0) res->contact = 0;
     return;
   }
-  int xl = jl + 1, xr = jr - 1;
-  double xleft = (double)(xl - 1) + (rho_mid - row[xl - 1]) / (row[xl] - row[xl - 1]);
-  double xright = (double)xr + (row[xr] - rho_mid) / (row[xr] - row[xr + 1]);
-  int steps = kmin - 1;
-  int y = base + steps * dir;
-  double ra = rho[(size_t)y * nx + xc], rb = rho[(size_t)(y + dir) * nx + xc];
-  double h = (double)steps + (ra - rho_mid) / (ra - rb);
-  double L = xright - xleft;
-  res[0] = 2.0 * atan2(2.0 * h, L);
-  res[1] = h;
-  res[2] = L;
-  res[4] = 0.0;
+
+  const int base = wall == 0 ? 1 : ny - 2, dir = wall == 0 ? 1 : -1;
+  // liquid run of the boundary row containing xc
+  int jl = INT_MIN, jr = INT_MAX;
+  bool dry = false;
+  for (int x = x0 + threadIdx.x; x < x1; x += kAThreads) {
+    const bool vap = !at_least(rho(base, x), mid);
+    if (vap && x < xc) jl = max(jl, x);
+    if (vap && x > xc) jr = min(jr, x);
+    dry |= vap && x == xc;
+  }
+  // first vapour node walking away from the wall along xc
+  const int ymax = wall == 0 ? yhi : ylo - 1;
+  const int nwalk = wall == 0 ? (ymax - base - 1) : (base - ymax - 1);
+  int kmin = INT_MAX;
+  for (int k = 1 + threadIdx.x; k <= nwalk; k += kAThreads)
+    if (!at_least(rho(base + k * dir, xc), mid)) {
+      kmin = k;
+      break;
+    }
+  jl = block_reduce_int(jl, true, shi);
+  jr = block_reduce_int(jr, false, shi);
+  kmin = block_reduce_int(kmin, false, shi);
+  if (__syncthreads_or(dry) || jl == INT_MIN || jr == INT_MAX || kmin == INT_MAX) {
+    if (threadIdx.x == 0) res->contact = 0;
+    return;
+  }
+  // the six densities around the three crossings
+  const int t = threadIdx.x, y = base + (kmin - 1) * dir;
+  if (t < 6) res->rho[t] = t < 4 ? rho(base, t < 2 ? jl + t : jr - 3 + t) : rho(y + (t - 4) * dir, xc);
+  if (t == 0) {
+    res->xl = jl;
+    res->xr = jr - 1;
+    res->steps = kmin - 1;
+    res->contact = 1;
+  }
 }
 
 inline unsigned nblk(size_t n, int t) { return (unsigned)((n + t - 1) / t); }
@@ -311,26 +480,61 @@ cudaError_t lbm_rho64(const lbm_ctx *C, const void *f, double *rho, unsigned lon
   return lbm_rho64_rows(C, f, rho, 0, C->ny, launches);
 }
 
-cudaError_t lbm_reduce_rows(const lbm_ctx *C, const double *v, int row0, int row1, double *partial, int npart,
-                            double *res, unsigned long long *launches) {
-  k_sum_partial<<<npart, 256, 0, C->stream>>>(v, (size_t)C->nx * C->ny, row0, row1, C->nx, partial);
-  k_sum_final<<<1, 1024, 0, C->stream>>>(partial, npart, res);
-  *launches += 2;
-  return cudaGetLastError();
-}
-
-cudaError_t lbm_reduce_max_speed(const lbm_ctx *C, const double *ux, const double *uy, double *partial, int npart,
-                                 double *res, unsigned long long *launches) {
-  size_t y0 = C->walls ? 1 : 0, y1 = C->walls ? C->ny - 1 : C->ny;
-  k_speed_partial<<<npart, 256, 0, C->stream>>>(ux, uy, y0, y1, C->nx, partial);
-  k_max_final<<<1, 1024, 0, C->stream>>>(partial, npart, res);
-  *launches += 2;
-  return cudaGetLastError();
-}
-
-cudaError_t lbm_angle(const lbm_ctx *C, const double *rho, int wall, int x0, int x1, double rho_mid, double *res,
-                      unsigned long long *launches) {
-  k_angle<<<1, 1024, 0, C->stream>>>(rho, C->nx, C->ny, wall, x0, x1, rho_mid, res);
+cudaError_t lbm_reduce_rows(const lbm_ctx *C, const double *v, int row0, int row1, double *res,
+                            unsigned long long *launches) {
+  k_sum<<<C->red_len, 256, 0, C->stream>>>(v, (size_t)row0 * C->nx, (size_t)row1 * C->nx, C->d_red,
+                                           (unsigned *)C->d_flag + 3, res);
   ++*launches;
+  return cudaGetLastError();
+}
+
+cudaError_t lbm_mass_of(const lbm_ctx *C, const void *f, double *res, unsigned long long *launches) {
+  const size_t n = (size_t)C->nx * C->ny, i0 = C->walls ? C->nx : 0, i1 = n - i0;
+  unsigned *counter = (unsigned *)C->d_flag + 3;
+  const bool x4 = C->precision == 32 && C->nx % 4 == 0 && ((uintptr_t)f & 15) == 0;
+  const unsigned g = std::min((unsigned)C->red_len, nblk((i1 - i0) / (x4 ? 4 : 1), 256));
+  if (C->precision == 64)
+    k_mass<double><<<g, 256, 0, C->stream>>>((const double *)f, n, i0, i1, C->d_red, counter, res);
+  else if (x4)
+    k_mass_x4<<<g, 256, 0, C->stream>>>((const float4 *)f, n / 4, i0 / 4, i1 / 4, C->d_red, counter, res);
+  else
+    k_mass<float><<<g, 256, 0, C->stream>>>((const float *)f, n, i0, i1, C->d_red, counter, res);
+  ++*launches;
+  return cudaGetLastError();
+}
+
+lbm_angle_args lbm_make_angle_args(const lbm_ctx *C, int wall, int x0, int x1, void *res) {
+  return lbm_angle_args{C->f[C->cur], C->nx, C->ny, wall, x0, x1, C->rho_mid, C->d_rho64, (unsigned *)C->d_flag + 3,
+                        (lbm_angle_cut *)res};
+}
+
+int lbm_angle_of(const lbm_angle_cut &r, double rho_mid, double *theta, double *H, double *L) {
+  if (!r.contact) return LBM_ENOCONTACT;
+  const double *q = r.rho;
+  const double left = (double)r.xl + (rho_mid - q[0]) / (q[1] - q[0]);
+  const double right = (double)r.xr + (q[2] - rho_mid) / (q[2] - q[3]);
+  *H = (double)r.steps + (q[4] - rho_mid) / (q[4] - q[5]);
+  *L = right - left;
+  *theta = 2.0 * atan2(2.0 * *H, *L);
+  return LBM_OK;
+}
+
+int lbm_angle_blocks(const lbm_angle_args &A) {
+  const int half = A.wall == 0 ? A.ny / 2 - 1 : A.ny - 1 - A.ny / 2;
+  return ((A.x1 - A.x0 + kACols - 1) / kACols) * ((half + kARows - 1) / kARows);
+}
+
+cudaError_t lbm_angle(const lbm_ctx *C, const lbm_angle_args &A, unsigned long long *launches) {
+  const dim3 g(lbm_angle_blocks(A));
+  if (C->precision == 64)
+    k_angle<double><<<g, kAThreads, 0, C->stream>>>(A, nullptr);
+  else
+    k_angle<float><<<g, kAThreads, 0, C->stream>>>(A, nullptr);
+  ++*launches;
+  return cudaGetLastError();
+}
+
+cudaError_t lbm_angle_many(const lbm_angle_args *tab, int first, int count, int blocks, cudaStream_t stream) {
+  k_angle<float><<<dim3(blocks, count), kAThreads, 0, stream>>>(lbm_angle_args{}, tab + first);
   return cudaGetLastError();
 }

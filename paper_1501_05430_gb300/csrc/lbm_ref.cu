@@ -56,37 +56,6 @@ __global__ void k_fields(Mdl<R> m, const R *__restrict__ f, const double *__rest
   if (!(r > (R)0) || r > m.rho_max) atomicOr(flag, 1);
 }
 
-// Macroscopic outputs at every node: out7 = {ux, uy, Fx, Fy, Qxx, Qyy, Qxy}
-// (zero on the solid rows).
-template <typename R>
-__global__ void k_macro(Mdl<R> m, const R *__restrict__ f, const R *__restrict__ fields,
-                        double *__restrict__ out7) {
-  size_t n = (size_t)m.nx * m.ny;
-  size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  int y = (int)(i / m.nx), x = (int)(i - (size_t)y * m.nx);
-  if (m.solid_row(y)) {
-    for (int k = 0; k < 7; ++k) out7[k * n + i] = 0.0;
-    return;
-  }
-  R Fx, Fy, Qxx, Qyy, Qxy;
-  force_Q(m, fields + n, fields + 2 * n, y, FieldNb<R>{m, y, x}, Fx, Fy, Qxx, Qyy, Qxy);
-  R jx = 0, jy = 0;
-#pragma unroll
-  for (int a = 0; a < 9; ++a) {
-    if (MC(3, a) != 0.0) jx = jx + (R)MC(3, a) * f[a * n + i];
-    if (MC(5, a) != 0.0) jy = jy + (R)MC(5, a) * f[a * n + i];
-  }
-  R r = fields[i];
-  out7[i] = (double)((jx + (R)0.5 * Fx) / r);
-  out7[n + i] = (double)((jy + (R)0.5 * Fy) / r);
-  out7[2 * n + i] = (double)Fx;
-  out7[3 * n + i] = (double)Fy;
-  out7[4 * n + i] = (double)Qxx;
-  out7[5 * n + i] = (double)Qyy;
-  out7[6 * n + i] = (double)Qxy;
-}
-
 // A density a state may start from: finite and > 0.  Tested on the bits
 // (0 < bits < the bits of +infinity), without FP64 instructions.
 __device__ __forceinline__ bool rho_ok(double r) {
@@ -186,25 +155,9 @@ inline unsigned nblk(size_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
 }  // namespace
 
-cudaError_t lbm_ref_fields(const lbm_ctx *C, const void *f, void *fields, unsigned long long *launches) {
+cudaError_t lbm_ref_fields(const lbm_ctx *C, const double *f, double *fields, unsigned long long *launches) {
   size_t n = (size_t)C->nx * C->ny;
-  if (C->precision == 64)
-    k_fields<double><<<nblk(n, 256), 256, 0, C->stream>>>(Mdl<double>(C->dp), (const double *)f, C->d_coef, (double *)fields,
-                                                          C->d_flag);
-  else
-    k_fields<float><<<nblk(n, 256), 256, 0, C->stream>>>(Mdl<float>(C->dp), (const float *)f, C->d_coef, (float *)fields,
-                                                         C->d_flag);
-  ++*launches;
-  return cudaGetLastError();
-}
-
-cudaError_t lbm_ref_macro(const lbm_ctx *C, const void *f, const void *fields, double *out7,
-                          unsigned long long *launches) {
-  size_t n = (size_t)C->nx * C->ny;
-  if (C->precision == 64)
-    k_macro<double><<<nblk(n, 128), 128, 0, C->stream>>>(Mdl<double>(C->dp), (const double *)f, (const double *)fields, out7);
-  else
-    k_macro<float><<<nblk(n, 128), 128, 0, C->stream>>>(Mdl<float>(C->dp), (const float *)f, (const float *)fields, out7);
+  k_fields<double><<<nblk(n, 256), 256, 0, C->stream>>>(Mdl<double>(C->dp), f, C->d_coef, fields, C->d_flag);
   ++*launches;
   return cudaGetLastError();
 }

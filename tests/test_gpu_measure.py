@@ -1,0 +1,105 @@
+"""The contact-angle measurement (parallel column sums that narrow the centre
+column down, sequential sums where columns tie) and the mass, against the
+oracle's sequential measurement of the library's own density field."""
+import math
+
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_1501_05430_gb300 import inputs as I
+from paper_1501_05430_gb300 import lbm as L
+
+pytestmark = pytest.mark.gpu
+
+
+def _sim(nx, ny, precision):
+    eos = L.carnahan_starling()
+    T = 0.7 * L.lbm_eos_critical(eos)[0]
+    p = L.lbm_params_default(precision=precision, check_every=0)
+    return L.Lbm(nx, ny, eos, T, 1.0, params=p, torch_state=False), L.lbm_coexistence(eos, T)
+
+
+def _block(nx, ny, rv, rl, seed, columns, wall):
+    """A liquid block whose columns hold the same densities in different orders:
+    sums equal up to their rounding, different heights of the first vapour node."""
+    rng = np.random.default_rng(seed)
+    rho = np.full((ny, nx), rv)
+    values = np.concatenate([rng.uniform(0.9, 1.1, 12) * rl, rng.uniform(0.9, 1.1, 8) * rv])
+    x0 = nx // 3
+    for x in range(x0, x0 + columns):
+        col = np.concatenate([[rl], rng.permutation(values)])
+        if wall == 0:
+            rho[1:22, x] = col
+        else:
+            rho[ny - 22:ny - 1, x] = col[::-1]
+    return rho
+
+
+@pytest.mark.parametrize("wall", [0, 1])
+@pytest.mark.parametrize("precision", [32, 64])
+@pytest.mark.parametrize("nx,ny,columns", [(64, 140, 1), (96, 300, 2), (131, 64, 16), (131, 133, 17), (300, 50, 90)])
+def test_ties_are_broken_like_the_sequential_measurement(nx, ny, columns, precision, wall):
+    sim, (rv, rl) = _sim(nx, ny, precision)
+    with sim:
+        sim.set_rho(_block(nx, ny, rv, rl, nx + ny, columns, wall))
+        th, H, Lb = sim.contact_angle(wall, 2, nx - 1)
+        mid = sim.info.rho_mid
+        ot, oH, oL, _ = O.contact_angle_field(sim.rho(), wall, 2, nx - 1, mid)
+        assert H == oH and Lb == oL and th == pytest.approx(ot, rel=1e-15)
+
+
+@pytest.mark.parametrize("precision", [32, 64])
+def test_no_contact_line(precision):
+    sim, (rv, rl) = _sim(40, 30, precision)
+    with sim:
+        for rho in (np.full((30, 40), rv), np.full((30, 40), rl)):
+            sim.set_rho(rho)
+            with pytest.raises(L.LbmError) as e:
+                sim.contact_angle(0, 0, 40)
+            assert e.value.status == L.LBM_ENOCONTACT
+        sim.set_f(np.full((9, 30, 40), np.nan))
+        with pytest.raises(L.LbmError) as e:
+            sim.contact_angle(1, 3, 20)
+        assert e.value.status == L.LBM_ENOCONTACT
+
+
+def test_batch_angles_are_the_instances_own():
+    ws = I.batched(count=9)
+    eos = L.carnahan_starling(0.25, 4.0, 1.0)
+    tc = L.lbm_eos_critical(eos)[0]
+    descs = [dict(nx=w.nx, ny=w.ny, eos=eos, T=w.t_over_tc * tc, tau=w.tau, theta=w.theta) for w in ws]
+    with L.LbmBatch(descs) as b:
+        for w, d, inst in zip(ws, descs, b.instances):
+            rv, rl = L.lbm_coexistence(eos, d["T"])
+            inst.set_rho(I.droplet_field(w.nx, w.ny, w.droplets, rv, rl, w.width))
+        b[4].set_rho(np.full((ws[4].ny, ws[4].nx), rv))
+        th, H, Lb, st = b.contact_angles(0)
+        assert st[4] == L.LBM_ENOCONTACT and (st == 0).any()
+        for k, inst in enumerate(b.instances):
+            try:
+                own = inst.contact_angle(0, 0, inst.nx)
+            except L.LbmError as e:  # (a wide cap may reach the region's edge too)
+                assert st[k] == e.status == L.LBM_ENOCONTACT and math.isnan(th[k])
+            else:
+                assert st[k] == 0 and (th[k], H[k], Lb[k]) == own
+
+
+@pytest.mark.parametrize("nx,ny,walls", [(4, 5, True), (64, 33, True), (30, 17, False), (1024, 300, True)])
+def test_fp32_mass_is_the_exact_sum(nx, ny, walls):
+    """Against the correctly rounded sum of the populations: 48 bits a term and
+    fixed-order FP64 sums of up to 3e5 of them stay within 1e-13."""
+    eos = L.carnahan_starling()
+    T = 0.7 * L.lbm_eos_critical(eos)[0]
+    rng = np.random.default_rng(nx)
+    f = rng.uniform(0.01, 2.0, (9, ny, nx)) * 10.0 ** rng.uniform(-3, 3, (9, ny, nx))
+    if walls:
+        f[:, 0] = f[:, -1] = 0.0
+    p = L.lbm_params_default(precision=32, check_every=0)
+    with L.Lbm(nx, ny, eos, T, 1.0, walls=walls, params=p, torch_state=False) as s:
+        s.set_f(f)
+        want = math.fsum(f.astype(np.float32).astype(float).ravel())
+        assert s.mass() == pytest.approx(want, rel=1e-13)
+        f[3, 2, 1] = np.inf
+        s.set_f(f)
+        assert s.mass() == math.inf
