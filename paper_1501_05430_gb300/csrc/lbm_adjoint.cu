@@ -775,9 +775,8 @@ int lbm_adjoint_record(lbm_ctx *C, int nsteps, int checkpoint_every) {
       st = LBM_ECUDA;
     }
     auto steps = [&](int count, int cur) {
-      int r = LBM_OK;
-      for (int k = 0; k < count && r == LBM_OK; ++k) r = fwd_step(C, C->f[cur ^ (k & 1)], C->f[cur ^ (k & 1) ^ 1]);
-      return r;
+      ACK(lbm_launch_steps(C, cur, count, &C->launches));
+      return LBM_OK;
     };
     if (st == LBM_OK && C->stream && len == T->every) {
       const int p = C->cur;

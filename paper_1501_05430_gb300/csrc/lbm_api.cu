@@ -246,6 +246,8 @@ cudaError_t launch_step(lbm_ctx *C, int src, unsigned long long *launches) {
   return lbm_canon_step(C, C->f[src], C->f[dst], launches);
 }
 
+int launches_of(const lbm_ctx *C, int count) { return C->tile_pairs ? count / 4 * 2 + count % 4 : count; }
+
 // Steps per captured graph (even), or 0 when graphs are off or impossible
 // (the legacy default stream cannot be captured).
 int graph_steps(const lbm_ctx *C) {
@@ -264,7 +266,7 @@ int capture_steps(lbm_ctx *C, int start, int G, cudaGraphExec_t *out) {
   unsigned long long dummy = 0;
   cudaError_t e = cudaSuccess;
   C->capturing = 1;
-  for (int k = 0; k < G && e == cudaSuccess; ++k) e = launch_step(C, start ^ (k & 1), &dummy);
+  e = lbm_launch_steps(C, start, G, &dummy);
   C->capturing = 0;
   cudaError_t e2 = cudaStreamEndCapture(C->stream, &graph);
   if (e == cudaSuccess) e = e2;
@@ -445,6 +447,21 @@ int create_impl(int nx, int ny, const lbm_eos *eos, double T, double tau, const 
 
 }  // namespace
 
+// `count` steps from array `start`, queued one after the other.  Where two steps
+// go into one launch they are taken four at a time, A -> B -> A, so that the
+// state is in array start ^ (count & 1) afterwards as after single steps.
+cudaError_t lbm_launch_steps(lbm_ctx *C, int start, int count, unsigned long long *launches) {
+  int k = 0;
+  cudaError_t e = cudaSuccess;
+  if (C->tile_pairs)
+    for (; k + 4 <= count && e == cudaSuccess; k += 4) {
+      e = lbm_tile_pair(C, C->f[start], C->f[start ^ 1], launches);
+      if (e == cudaSuccess) e = lbm_tile_pair(C, C->f[start ^ 1], C->f[start], launches);
+    }
+  for (; k < count && e == cudaSuccess; ++k) e = launch_step(C, start ^ (k & 1), launches);
+  return e;
+}
+
 // ---------------------------------------------------------------------------
 // Public API
 // ---------------------------------------------------------------------------
@@ -582,7 +599,7 @@ int lbm_step(lbm_ctx *C, int nsteps) {
       const int len = C->graph_len[k];
       while (nsteps - it >= len) {
         CK(cudaGraphLaunch(C->step_graph[C->cur][k], C->stream));
-        C->launches += (unsigned long long)len;
+        C->launches += (unsigned long long)launches_of(C, len);
         const long long before = C->steps;
         C->steps += len;
         it += len;
@@ -594,11 +611,15 @@ int lbm_step(lbm_ctx *C, int nsteps) {
       }
     }
   }
-  for (; it < nsteps; ++it) {
-    CK(launch_step(C, C->cur, &C->launches));
-    C->cur ^= 1;
-    C->steps++;
-    if (C->params.check_every > 0 && C->steps % C->params.check_every == 0) {
+  while (it < nsteps) {
+    // as many at once as no stability check falls between
+    const int ce = C->params.check_every, left = nsteps - it;
+    const int m = ce > 0 ? (int)std::min<long long>(left, ce - C->steps % ce) : left;
+    CK(lbm_launch_steps(C, C->cur, m, &C->launches));
+    C->cur ^= m & 1;
+    C->steps += m;
+    it += m;
+    if (ce > 0 && C->steps % ce == 0) {
       int st = read_flags(C);
       if (st) return st;
     }

@@ -538,6 +538,10 @@ struct BTile {
   int inst, x0, y0, pad;
 };
 
+struct TileInst : BInst {
+  static constexpr bool short_math = true;
+};
+
 struct TileArgs {
   const BInst *inst;
   const BTile *tiles;
@@ -549,8 +553,8 @@ struct TileArgs {
 };
 
 template <int KIND, int MCW>
-__global__ void __launch_bounds__(kTileThreads) k_batch_tile(TileArgs A) {
-  __shared__ BInst P;
+__global__ void __launch_bounds__(kTileThreads, 5) k_batch_tile(TileArgs A) {
+  __shared__ TileInst P;
   __shared__ lbm_tile::Smem<kTileRows> M;
   if (A.pdl) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const BTile t = A.tiles[blockIdx.x];

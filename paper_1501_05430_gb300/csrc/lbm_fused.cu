@@ -39,7 +39,6 @@ using lbm_node::collide_node2;
 using lbm_node::eos_node;
 using lbm_node::eos_node2;
 using lbm_node::ghost_node;
-using lbm_node::sqrt0;
 
 constexpr int NCONS = 128;               // threads per CTA (4 warps)
 constexpr int HB = 4;                    // halo box width (16 bytes of floats)

@@ -13,7 +13,6 @@ struct lbm_fused_args {
   int nstrips, nrows, y0;
   long long total;
   int stages;
-  int pdl;  // tile kernel: launched as a programmatic dependent
   float b4, RT2, a2, r1, r2, pc0, pc1, pc2;    // EOS constants (b/4, -2RT, 2a; Eq. 11 break-
                                                 // points and slopes folded into -2U)
   float A, omA, pre, halfA, rho_max, ghost_max; // force / Q constants, bounds
@@ -24,6 +23,7 @@ struct lbm_fused_args {
   const double *coef;
   float *fout;
   int *flag;
+  int pdl;  // tile kernels: launched as a programmatic dependent
 };
 
 // Launch arguments of a context's step (all but the destination array).

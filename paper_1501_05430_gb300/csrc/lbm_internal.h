@@ -72,6 +72,7 @@ struct lbm_ctx {
   int fused_ok, fused_unit;  // fused kernel usable; unit-rate specialisation
   int fused_cols;            // columns per thread of the fused kernel
   int tile_rows;             // rows per tile of the small-domain kernel, 0: the ring kernel runs
+  int tile_pairs;            // it also has a form that makes two steps per launch
   int tile_w, tile_blocks, tile_stages, fused_smem;
   unsigned char tmaps[4][128];   // CUtensorMap for f[0], f[1]: main box, halo box
   // lbm_step graphs, captured at the first lbm_step for both starting arrays:
@@ -97,6 +98,10 @@ cudaError_t lbm_ref_set_rho(const lbm_ctx *C, const double *rho, void *f, int *b
 cudaError_t lbm_ref_droplets(const lbm_ctx *C, int n, const double *drop, double width, double *rho,
                              unsigned long long *launches);
 
+// ---- lbm_api.cu -------------------------------------------------------------
+// `count` steps of a context from array f[start] with its own kernel
+cudaError_t lbm_launch_steps(lbm_ctx *C, int start, int count, unsigned long long *launches);
+
 // ---- lbm_canon.cu: one step in the canonical evaluation order ---------------
 cudaError_t lbm_canon_step(const lbm_ctx *C, const void *src, void *dst, unsigned long long *launches);
 // Fields of the state f as doubles, [ny][nx] each: rho, psi, U (ghost values on
@@ -115,6 +120,8 @@ cudaError_t lbm_fused_step_between(lbm_ctx *C, const void *src, void *dst, unsig
 // ---- lbm_tile.cu: the FP32 step of small domains ------------------------------
 void lbm_tile_plan(lbm_ctx *C);  // sets tile_rows (0: not for this domain) and the tile_* shape
 cudaError_t lbm_tile_step(const lbm_ctx *C, const void *src, void *dst, unsigned long long *launches);
+// two steps in one launch (tile_pairs)
+cudaError_t lbm_tile_pair(const lbm_ctx *C, const void *src, void *dst, unsigned long long *launches);
 
 // ---- lbm_adjoint.cu: discrete adjoint ---------------------------------------
 void lbm_adjoint_free_tape(lbm_ctx *C);

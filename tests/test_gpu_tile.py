@@ -23,9 +23,10 @@ MODELS = {
     "piecewise_martys_chen_general": dict(eos="pw", pw=PW10, wetting=1, G_w=-0.1, tau=0.8),
     "periodic": dict(walls=False),
 }
-# one and several strips with a ragged last one, bands with every remainder
-# (walled: ny - 2 rows), the smallest grid
-SIZES = [(4, 5), (64, 6), (60, 7), (68, 8), (132, 9), (260, 24), (128, 13)]
+# one and several strips with a ragged last one (64 columns a tile, 58 with two
+# steps per launch, which 4 columns are too few for), bands with every remainder
+# (walled: ny - 2 rows), the smallest grids
+SIZES = [(4, 5), (8, 5), (8, 6), (56, 6), (60, 7), (64, 6), (68, 8), (116, 10), (132, 9), (260, 24), (128, 13)]
 
 
 def _context(c, f, monkeypatch, ring):
@@ -54,7 +55,7 @@ def test_tile_and_ring_kernels_give_the_same_bits(name, nx, ny, monkeypatch):
     out = []
     for ring in (False, True):
         with _context(c, f, monkeypatch, ring) as g:
-            g.step(7)
+            g.step(7)  # two launches of two steps and three of one where both forms exist
             out.append((g.f(), g.status()))
     c.orc.close()
     assert np.array_equal(out[0][0], out[1][0])
@@ -82,4 +83,35 @@ def test_tile_kernel_flags_an_unstable_node(y, x, monkeypatch):
     with _context(c, f, monkeypatch, False) as g:
         g.step(1)
         assert g.status() == L.LBM_EUNSTABLE
+    c.orc.close()
+
+
+def test_state_alternates_between_the_two_arrays():
+    """n steps leave the state in array n % 2, however many a launch makes, and
+    stability checks fall due after every check_every-th step."""
+    torch = pytest.importorskip("torch")
+    c, f = _case(72, 20, 9)
+    c.params.check_every = 6
+    nbytes = L.lbm_required_state_bytes(c.nx, c.ny, 32)
+    for stream in (None, torch.cuda.Stream()):
+        buf = torch.zeros((2, 9, c.ny, c.nx), dtype=torch.float32, device="cuda")
+        ctx = L.lbm_create_with_buffer(c.nx, c.ny, c.geos, c.T, c.tau, buf.data_ptr(), nbytes, c.theta, True, c.params,
+                                       stream)
+        L.lbm_set_f(ctx, f)
+        done = 0
+        for n in (1, 2, 3, 4, 5, 8, 13, 70):
+            L.lbm_step(ctx, n)
+            done += n
+            got = L.lbm_get_f(ctx)
+            assert np.array_equal(buf[done % 2].cpu().numpy(), got.astype(np.float32))
+        assert L.lbm_get_info(ctx).steps_done == done
+        bad = f.copy()
+        bad[:, 9, 9] = np.nan
+        L.lbm_set_f(ctx, bad)
+        with pytest.raises(L.LbmError) as e:
+            L.lbm_step(ctx, 20)
+        assert e.value.status == L.LBM_EUNSTABLE
+        if stream is None:
+            assert L.lbm_get_info(ctx).steps_done == done + 6 - done % 6
+        L.lbm_destroy(ctx)
     c.orc.close()
