@@ -68,8 +68,55 @@ namespace {
 
 constexpr int kMaxIter = 64;
 
+__device__ __forceinline__ float fma_(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_(double a, double b, double c) { return __fma_rn(a, b, c); }
+
+// a / b from y = 1/b rounded to nearest: each correction with the exact remainder
+// brings the quotient to 1 ulp and then to the correctly rounded one (Markstein,
+// IBM J. Res. Dev. 34, 1990), the bits of a division, without its special cases:
+// five instructions where several quotients share a divisor.  (A remainder below
+// the normal range, |a| < 1e-30 in FP32, can leave it an ulp off.)
 template <typename R>
-__device__ void eos_derivs(const Mdl<R> &m, R rho, R &dp_drho, R &dp_dT) {
+__device__ __forceinline__ R quot(R a, R b, R y) {
+  const R q0 = a * y, q1 = fma_(fma_(-b, q0, a), y, q0);
+  return fma_(fma_(-b, q1, a), y, q1);
+}
+// a / N for a small integer N: in FP32 one correction is enough for 3, 9 and
+// their multiples by powers of two (true of every significand)
+template <int N, typename R>
+__device__ __forceinline__ R over(R a) {
+  constexpr R y = (R)1 / (R)N;
+  if constexpr ((N & (N - 1)) == 0) return a * y;
+  if constexpr (sizeof(R) == 8) return quot(a, (R)N, y);
+  const R q = a * y;
+  return fma_(fma_(-(R)N, q, a), y, q);
+}
+
+// Row k of M times v, left to right (the products by 2 and 4 are exact, so the
+// fused ones round as separate ones).
+template <typename R>
+__device__ __forceinline__ R moment(int k, const R (&v)[9]) {
+  R acc = (R)0;
+  bool first = true;
+#pragma unroll
+  for (int a = 0; a < 9; ++a) {
+    const R c = (R)MC(k, a);
+    if (c == (R)0) continue;
+    acc = first ? c * v[a] : (c == (R)1 ? acc + v[a] : (c == (R)-1 ? acc - v[a] : fma_(c, v[a], acc)));
+    first = false;
+  }
+  return acc;
+}
+
+// psi_U with a shorter division by 3.
+template <typename R>
+__device__ __forceinline__ void node_eos(const Mdl<R> &m, R rho, R &psi, R &U) {
+  U = pressure(m, rho) - over<3>(rho);
+  psi = sqrt(fmax((R)0, (R)-2 * U));
+}
+
+template <typename R>
+__device__ __forceinline__ void eos_derivs(const Mdl<R> &m, R rho, R &dp_drho, R &dp_dT) {
   if (m.kind == LBM_EOS_CARNAHAN_STARLING) {
     // p = rho R T Z(eta) - a rho^2, Z = N/D, N = 1 + eta + eta^2 - eta^3, D = (1 - eta)^3, eta = b rho/4:
     // dp/drho = R T (Z + eta dZ/deta) - 2 a rho,  dZ/deta = N'/D + 3 N/(1 - eta)^4
@@ -78,8 +125,9 @@ __device__ void eos_derivs(const Mdl<R> &m, R rho, R &dp_drho, R &dp_dT) {
     R num = (((R)1 + eta) + eta * eta) - (eta * eta) * eta;
     R dnum = ((R)1 + (R)2 * eta) - (R)3 * (eta * eta);
     R den = (om * om) * om;
-    R Z = num / den;
-    R dZ = dnum / den + ((R)3 * num) / (den * om);
+    const R y = (R)1 / den;
+    R Z = quot(num, den, y);
+    R dZ = quot(dnum, den, y) + ((R)3 * num) / (den * om);
     dp_drho = (m.Rg * m.T) * (Z + eta * dZ) - (R)2 * (m.a * rho);
     dp_dT = (rho * m.Rg) * Z;
   } else {
@@ -88,45 +136,87 @@ __device__ void eos_derivs(const Mdl<R> &m, R rho, R &dp_drho, R &dp_dT) {
   }
 }
 
+// Eq. 14's sums over the solid neighbours of a fluid node of row y.
+template <typename R>
+__device__ __forceinline__ void solid_sums(const Mdl<R> &m, int y, R &ssx, R &ssy) {
+  ssx = ssy = (R)0;
+#pragma unroll
+  for (int a = 1; a < 9; ++a) {
+    const R ts = m.solid_row(m.wy(y + EY(a))) ? wgt<R>(a) : (R)0;
+    if (EX(a)) ssx = EX(a) > 0 ? ssx + ts : ssx - ts;
+    if (EY(a)) ssy = EY(a) > 0 ? ssy + ts : ssy - ts;
+  }
+}
+
+// Eq. 9 force (+ Eq. 14) at a fluid node: the F of force_Q.
+template <typename R, typename Nb>
+__device__ __forceinline__ void force(const Mdl<R> &m, const R *__restrict__ psi, const R *__restrict__ U, int y, Nb nb,
+                                      R &Fx, R &Fy) {
+  const R psi0 = psi[nb(0, 0)];
+  R spx = (R)0, spy = (R)0, sUx = (R)0, sUy = (R)0;
+#pragma unroll
+  for (int a = 1; a < 9; ++a) {
+    const auto j = nb(EX(a), EY(a));
+    const R tp = wgt<R>(a) * psi[j], tu = wgt<R>(a) * U[j];
+    if (EX(a)) {
+      spx = EX(a) > 0 ? spx + tp : spx - tp;
+      sUx = EX(a) > 0 ? sUx + tu : sUx - tu;
+    }
+    if (EY(a)) {
+      spy = EY(a) > 0 ? spy + tp : spy - tp;
+      sUy = EY(a) > 0 ? sUy + tu : sUy - tu;
+    }
+  }
+  const R cpsi = -(((R)1 - m.A) * psi0);
+  Fx = -(m.A * sUx) - cpsi * spx;
+  Fy = -(m.A * sUy) - cpsi * spy;
+  if (m.wetting == LBM_WET_MARTYS_CHEN) {
+    R ssx, ssy;
+    solid_sums(m, y, ssx, ssy);
+    const R gp = m.Gw * psi0;
+    Fx = Fx - gp * ssx;
+    Fy = Fy - gp * ssy;
+  }
+}
+
+// Factors of the transposed collision that every node shares.
+template <typename R>
+struct AdjRates {
+  R m[9], S[9];  // 1 - s_k, 1 - s_k/2
+  explicit AdjRates(const lbm_dev_params &P) {
+    for (int k = 0; k < 9; ++k) {
+      m[k] = (R)1 - (R)P.s[k];
+      S[k] = (R)1 - (R)0.5 * (R)P.s[k];
+    }
+  }
+};
+
 // Transpose of the collision at one fluid node: from ls = dL/df* (pulled back
 // through the streaming), the populations f, rho and F to the part of dL/df that
 // passes through the moments (cl), and aux = dL/d(Fx, Fy, Qxx, Qyy, Qxy).
 template <typename R>
-__device__ __forceinline__ void adj_collide(const Mdl<R> &m, const R (&f)[9], const R (&ls)[9], R rho, R Fx, R Fy,
-                                            R (&cl)[9], R (&aux)[5]) {
-  R mm[9];
-#pragma unroll
-  for (int k = 0; k < 9; ++k) {
-    R acc = (R)0;
-#pragma unroll
-    for (int a = 0; a < 9; ++a)
-      if (MC(k, a) != 0.0) acc = acc + (R)MC(k, a) * f[a];
-    mm[k] = acc;
-  }
-  const R vx = (mm[3] + (R)0.5 * Fx) / rho, vy = (mm[5] + (R)0.5 * Fy) / rho;
+__device__ __forceinline__ void adj_collide(const Mdl<R> &m, const AdjRates<R> &K, const R (&f)[9], const R (&ls)[9],
+                                            R rho, R Fx, R Fy, R (&cl)[9], R (&aux)[5]) {
+  const R ir = (R)1 / rho;
+  const R vx = quot(moment(3, f) + (R)0.5 * Fx, rho, ir), vy = quot(moment(5, f) + (R)0.5 * Fy, rho, ir);
   const R v2 = vx * vx + vy * vy;
   // f* = M^T diag(1/N) m*  ->  dL/dm*_k = sum_a M_ka ls_a / N_k
-  R msb[9], mb[9];
-#pragma unroll
-  for (int k = 0; k < 9; ++k) {
-    R acc = (R)0;
-#pragma unroll
-    for (int a = 0; a < 9; ++a)
-      if (MC(k, a) != 0.0) acc = acc + (R)MC(k, a) * ls[a];
-    msb[k] = acc / (R)NRM(k);
-  }
+  const R msb[9] = {over<9>(moment(0, ls)),  over<36>(moment(1, ls)), over<36>(moment(2, ls)),
+                    over<6>(moment(3, ls)),  over<12>(moment(4, ls)), over<6>(moment(5, ls)),
+                    over<12>(moment(6, ls)), over<4>(moment(7, ls)),  over<4>(moment(8, ls))};
+  R mb[9];
   // m*_k = m_k - s_k (m_k - meq_k) + (1 - s_k/2) S_k + C_k
   R meqb[9], Sb[9];
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
-    mb[k] = ((R)1 - m.s[k]) * msb[k];
+    mb[k] = K.m[k] * msb[k];
     meqb[k] = m.s[k] * msb[k];
-    Sb[k] = ((R)1 - (R)0.5 * m.s[k]) * msb[k];
+    Sb[k] = K.S[k] * msb[k];
   }
   // C_1 = 1.5 s_1 (Qxx + Qyy), C_7 = -s_7 (Qxx - Qyy), C_8 = -s_8 Qxy
-  const R Qxxb = ((R)1.5 * m.s[1]) * msb[1] - m.s[7] * msb[7];
-  const R Qyyb = ((R)1.5 * m.s[1]) * msb[1] + m.s[7] * msb[7];
-  const R Qxyb = -(m.s[8] * msb[8]);
+  aux[2] = ((R)1.5 * m.s[1]) * msb[1] - m.s[7] * msb[7];
+  aux[3] = ((R)1.5 * m.s[1]) * msb[1] + m.s[7] * msb[7];
+  aux[4] = -(m.s[8] * msb[8]);
   // S = (0, 6 vF, -6 vF, Fx, -Fx, Fy, -Fy, 2 (vx Fx - vy Fy), vx Fy + vy Fx), vF = v.F
   const R vFb = (R)6 * (Sb[1] - Sb[2]);
   R Fxb = (Sb[3] - Sb[4]) + (R)2 * vx * Sb[7] + vy * Sb[8] + vx * vFb;
@@ -140,131 +230,139 @@ __device__ __forceinline__ void adj_collide(const Mdl<R> &m, const R (&f)[9], co
   vxb = vxb + (R)2 * vx * v2b + rho * (meqb[3] - meqb[4]) + (R)2 * rho * vx * meqb[7] + rho * vy * meqb[8];
   vyb = vyb + (R)2 * vy * v2b + rho * (meqb[5] - meqb[6]) - (R)2 * rho * vy * meqb[7] + rho * vx * meqb[8];
   // v = (j + F/2) / rho
-  mb[3] = mb[3] + vxb / rho;
-  mb[5] = mb[5] + vyb / rho;
-  Fxb = Fxb + (R)0.5 * vxb / rho;
-  Fyb = Fyb + (R)0.5 * vyb / rho;
-  rhob = rhob - (vxb * vx + vyb * vy) / rho;
+  const R wx = quot(vxb, rho, ir), wy = quot(vyb, rho, ir);
+  mb[3] = mb[3] + wx;
+  mb[5] = mb[5] + wy;
+  aux[0] = Fxb + (R)0.5 * wx;
+  aux[1] = Fyb + (R)0.5 * wy;
+  rhob = rhob - quot(vxb * vx + vyb * vy, rho, ir);
   // m = M f and rho = sum_a f_a
 #pragma unroll
   for (int a = 0; a < 9; ++a) {
     R acc = rhob;
 #pragma unroll
-    for (int k = 0; k < 9; ++k)
-      if (MC(k, a) != 0.0) acc = acc + (R)MC(k, a) * mb[k];
+    for (int k = 0; k < 9; ++k) {
+      const R c = (R)MC(k, a);
+      if (c == (R)0) continue;
+      acc = c == (R)1 ? acc + mb[k] : (c == (R)-1 ? acc - mb[k] : fma_(c, mb[k], acc));
+    }
     cl[a] = acc;
   }
-  aux[0] = Fxb;
-  aux[1] = Fyb;
-  aux[2] = Qxxb;
-  aux[3] = Qyyb;
-  aux[4] = Qxyb;
 }
 
 // dL/drho and dL/dT of node (row y) through psi and U, gathered from the aux of
 // the fluid nodes whose stencils hold it; ax(ex, ey) is the index of a neighbour
 // in the planes aux + k * an, nb(ex, ey) its index in psi.  rho: its density.
+// aux is 0 at solid nodes (and psi finite), so that they add nothing.
 template <typename R, typename Nb, typename Ax>
 __device__ __forceinline__ void adj_psi(const Mdl<R> &m, const R *__restrict__ psi, const R *__restrict__ aux,
-                                        size_t an, int y, R rho, Nb nb, Ax ax, R &rb, double &tb) {
-  const R G = (R)-1;
-  const R pre = m.kappa * (G * (R)0.5);
+                                        size_t an, int y, R rho, Nb nb, Ax ax, R &rb, R &tb) {
+  const R pre = m.kappa * (R)-0.5;
   const R omA = (R)1 - m.A;
-  const R psi_p = psi[nb(0, 0)];
+  const R psi_p = psi[nb(0, 0)], Ap = m.A * psi_p;
   R pb = (R)0, ub = (R)0;
   // fluid nodes q = p - e_a hold p in their stencil in direction a:
   //   dF(q)/dpsi_p = (1-A) psi_q w_a e_a,  dF(q)/dU_p = -A w_a e_a,
   //   dQ_ij(q)/dpsi_p = pre w_a e_ai e_aj ((1-A) psi_q + A psi_p)
 #pragma unroll
   for (int a = 1; a < 9; ++a) {
-    int yq = y - EY(a);
-    if (m.walls && (yq < 0 || yq >= m.ny)) continue;
-    if (m.solid_row(m.wy(yq))) continue;
-    const R *q = aux + ax(-EX(a), -EY(a));
-    const R w = wgt<R>(a);
-    const R eF = q[0] * (R)EX(a) + q[an] * (R)EY(a);
-    const R eQ = q[2 * an] * (R)(EX(a) * EX(a)) + q[3 * an] * (R)(EY(a) * EY(a)) + q[4 * an] * (R)(EX(a) * EY(a));
-    const R psi_q = psi[nb(-EX(a), -EY(a))];
-    pb = pb + (omA * psi_q) * w * eF + pre * w * eQ * (omA * psi_q + m.A * psi_p);
+    const int ex = EX(a), ey = EY(a);
+    const R *q = aux + ax(-ex, -ey);
+    const R w = wgt<R>(a), c = omA * psi[nb(-ex, -ey)];
+    R eF, eQ;
+    if (ey == 0) {
+      eF = ex > 0 ? q[0] : -q[0];
+      eQ = q[2 * an];
+    } else if (ex == 0) {
+      eF = ey > 0 ? q[an] : -q[an];
+      eQ = q[3 * an];
+    } else {
+      eF = (ex > 0 ? q[0] : -q[0]) + (ey > 0 ? q[an] : -q[an]);
+      eQ = (q[2 * an] + q[3 * an]) + (ex * ey > 0 ? q[4 * an] : -q[4 * an]);
+    }
+    pb = pb + c * w * eF + pre * w * eQ * (c + Ap);
     ub = ub - m.A * w * eF;
   }
-  const bool fluid = !m.solid_row(y);
-  if (fluid) {
-    // own terms: dF/dpsi_0 = (1-A) s_psi (+ Eq. 14), dQ_ii/dpsi_0 = pre ((1-A) q1_ii - psi_0),
-    // dQ_xy/dpsi_0 = pre (1-A) q1_xy
-    R spx = 0, spy = 0, ssx = 0, ssy = 0, qxx1 = 0, qyy1 = 0, qxy1 = 0;
+  // own terms: dF/dpsi_0 = (1-A) s_psi (+ Eq. 14), dQ_ii/dpsi_0 = pre ((1-A) q1_ii - psi_0),
+  // dQ_xy/dpsi_0 = pre (1-A) q1_xy
+  R spx = (R)0, spy = (R)0, qxx1 = (R)0, qyy1 = (R)0, qxy1 = (R)0;
 #pragma unroll
-    for (int a = 1; a < 9; ++a) {
-      const R w = wgt<R>(a);
-      const R pn = psi[nb(EX(a), EY(a))];
-      const R sol = m.solid_row(m.wy(y + EY(a))) ? (R)1 : (R)0;
-      spx = spx + w * pn * (R)EX(a);
-      spy = spy + w * pn * (R)EY(a);
-      ssx = ssx + w * sol * (R)EX(a);
-      ssy = ssy + w * sol * (R)EY(a);
-      const R t1 = w * (pn - psi_p);
-      qxx1 = qxx1 + t1 * (R)(EX(a) * EX(a));
-      qyy1 = qyy1 + t1 * (R)(EY(a) * EY(a));
-      qxy1 = qxy1 + t1 * (R)(EX(a) * EY(a));
+  for (int a = 1; a < 9; ++a) {
+    const int ex = EX(a), ey = EY(a);
+    const R w = wgt<R>(a), pn = psi[nb(ex, ey)], tp = w * pn, t1 = w * (pn - psi_p);
+    if (ex) {
+      spx = ex > 0 ? spx + tp : spx - tp;
+      qxx1 = qxx1 + t1;
     }
-    const R *o = aux + ax(0, 0);
-    const R Fxb = o[0], Fyb = o[an];
-    pb = pb + omA * (Fxb * spx + Fyb * spy);
-    if (m.wetting == LBM_WET_MARTYS_CHEN) pb = pb - m.Gw * (Fxb * ssx + Fyb * ssy);
-    pb = pb + pre * (omA * (o[2 * an] * qxx1 + o[3 * an] * qyy1 + o[4 * an] * qxy1) - psi_p * (o[2 * an] + o[3 * an]));
+    if (ey) {
+      spy = ey > 0 ? spy + tp : spy - tp;
+      qyy1 = qyy1 + t1;
+    }
+    if (ex && ey) qxy1 = ex * ey > 0 ? qxy1 + t1 : qxy1 - t1;
   }
+  const R *o = aux + ax(0, 0);
+  const R Fxb = o[0], Fyb = o[an];
+  const bool fluid = !m.solid_row(y);
+  pb = pb + omA * (Fxb * spx + Fyb * spy);
+  if (m.wetting == LBM_WET_MARTYS_CHEN && fluid) {
+    R ssx, ssy;
+    solid_sums(m, y, ssx, ssy);
+    pb = pb - m.Gw * (Fxb * ssx + Fyb * ssy);
+  }
+  pb = pb + pre * (omA * (o[2 * an] * qxx1 + o[3 * an] * qyy1 + o[4 * an] * qxy1) - psi_p * (o[2 * an] + o[3 * an]));
   // to dL/drho (and dL/dT) through U = p(rho) - rho/3 and psi = sqrt(-2U)
-  rb = (R)0;
-  tb = 0.0;
+  rb = tb = (R)0;
   const bool ghost = !fluid && m.wetting == LBM_WET_GEOMETRIC;
   if (fluid || (ghost && rho < m.rho_max)) {
     R dp, dpT;
     eos_derivs(m, rho, dp, dpT);
     const R ut = ub - (psi_p > (R)0 ? pb / psi_p : (R)0);
     rb = ut * (dp - (R)1 / (R)3);
-    tb = (double)(ut * dpT);
+    tb = ut * dpT;
   }
 }
 
 // Transpose of the ghost rule at one wall node, from gb = dL/d(its density):
 // part = dL/d(rho(x-1), rho(x+1), rho(x) of the boundary row, rho(x) of the
-// second row); returns dL/dtheta.  dc, dcot: derivatives of c and cot in theta.
-template <typename R>
-__device__ __forceinline__ double adj_ghost(const Mdl<R> &m, R rim1, R ri1, R rip1, R ri2, R c, R cot, double dc,
-                                            double dcot, R gb, double (&part)[4]) {
-  R a = rip1 - rim1;
-  // forward again, keeping the iterates
-  R d[kMaxIter];
+// second row); cb, cotb: dL/d(c, cot).  MAX: most iterations of Eq. 20.
+template <int MAX, typename R>
+__device__ __forceinline__ void adj_ghost(int n_iter, R ghost_max, R rim1, R ri1, R rip1, R ri2, R c, R cot, R gb, R (&part)[4],
+                                          R &cb, R &cotb) {
+  const R a = rip1 - rim1;
+  // forward again, keeping the iterates: g_{k+1} = ri2 + c s_k, s_k = sqrt(a^2 + d_k^2), d_k = ri2 - g_k
+  R d[MAX], sq[MAX];
   R g;
-  const int nit = m.n_iter < kMaxIter ? m.n_iter : kMaxIter;
-  if (nit <= 0) {
+  if (n_iter <= 0) {
     g = ri2 + cot * fabs(a);
   } else {
-    d[0] = (R)2 * (ri2 - ri1);
     g = ri2;
-    for (int k = 0; k < nit; ++k) {
-      R s = a * a + d[k] * d[k];
-      g = ri2 + c * sqrt(s);
-      if (k + 1 < nit) d[k + 1] = ri2 - g;
+    R dk = (R)2 * (ri2 - ri1);
+#pragma unroll(MAX <= 4 ? MAX : 1)
+    for (int k = 0; k < MAX; ++k) {
+      if (k >= n_iter) break;
+      d[k] = dk;
+      sq[k] = sqrt(a * a + dk * dk);
+      g = ri2 + c * sq[k];
+      dk = ri2 - g;
     }
   }
-  if (!(g > (R)0 && g < m.ghost_max)) gb = (R)0;  // clamped: no gradient
-  R ab = 0, ri1b = 0, ri2b = 0, cb = 0, cotb = 0;
-  if (nit <= 0) {
+  if (!(g > (R)0 && g < ghost_max)) gb = (R)0;  // clamped: no gradient
+  R ab = (R)0, ri1b = (R)0, ri2b = (R)0;
+  cb = cotb = (R)0;
+  if (n_iter <= 0) {
     ri2b = gb;
     cotb = gb * fabs(a);
     ab = a > (R)0 ? gb * cot : (a < (R)0 ? -(gb * cot) : (R)0);
   } else {
     R gbar = gb;
-    for (int k = nit - 1; k >= 0; --k) {
-      // g_{k+1} = ri2 + c sqrt(a^2 + d_k^2)
-      R s = a * a + d[k] * d[k];
-      R sq = sqrt(s);
+#pragma unroll(MAX <= 4 ? MAX : 1)
+    for (int k = MAX - 1; k >= 0; --k) {
+      if (k >= n_iter) continue;
       ri2b = ri2b + gbar;
-      cb = cb + gbar * sq;
-      R sb = s > (R)0 ? (gbar * c) * (R)0.5 / sq : (R)0;
-      ab = ab + sb * (R)2 * a;
-      R db = sb * (R)2 * d[k];
+      cb = cb + gbar * sq[k];
+      const R t = sq[k] > (R)0 ? (gbar * c) / sq[k] : (R)0;
+      const R db = t * d[k];
+      ab = ab + t * a;
       if (k >= 1) {  // d_k = ri2 - g_k
         ri2b = ri2b + db;
         gbar = -db;
@@ -274,11 +372,16 @@ __device__ __forceinline__ double adj_ghost(const Mdl<R> &m, R rim1, R ri1, R ri
       }
     }
   }
-  part[0] = -(double)ab;
-  part[1] = (double)ab;
-  part[2] = (double)ri1b;
-  part[3] = (double)ri2b;
-  return (double)cb * dc + (double)cotb * dcot;
+  part[0] = -ab;
+  part[1] = ab;
+  part[2] = ri1b;
+  part[3] = ri2b;
+}
+// the general count, out of the way of the code that runs
+template <typename R>
+__device__ __noinline__ void adj_ghost_any(int n_iter, R ghost_max, R rim1, R ri1, R rip1, R ri2, R c, R cot, R gb,
+                                           R (&part)[4], R &cb, R &cotb) {
+  adj_ghost<kMaxIter>(n_iter, ghost_max, rim1, ri1, rip1, ri2, c, cot, gb, part, cb, cotb);
 }
 
 // ---- one reverse step in one kernel -----------------------------------------------
@@ -294,22 +397,28 @@ constexpr int kStepThreads = 480;                // one node per thread in every
 // collision of every node whose aux the tile reads (threads of the tile keep
 // the part that passes through the moments in registers); dL/drho through psi
 // and U, and at the ghost nodes the transpose of the ghost rule; the sums.
-// Small domains are bound by the latency of a kernel, and five kernels with
-// four global round trips of fields, aux and dL/drho took 19 us (captured; 28
-// launched directly) where this one takes 9; its repeated work at the tiles'
-// edges (1.8 times the fields, 1.4 times the collisions) is paid for at any size
-// by the 170 bytes a node that are not moved: reverse step with its replay, us,
-// five kernels -> one, 256 x 128 21.9 -> 12.0, 800 x 400 61 -> 55, 1600 x 800
-// 245 -> 238.  In FP64 the repeated work costs more than it saves (800 x 400
-// 816 -> 1040; the FP64 pipe is the limit), so FP64 keeps the kernels below.
+// Small domains are bound by the latency of a kernel and by its one CTA per SM,
+// whose 15 warps issue 30% of the time: five kernels with four global round trips
+// of fields, aux and dL/drho took longer than the repeated work at the tiles'
+// edges (1.8 times the fields, 1.4 times the collisions), which at any size is
+// also paid for by the 170 bytes a node that are not moved.  The arithmetic was
+// then cut without a change of its bits (no products with the zeros of e and M,
+// shared and constant divisors as in quot(), factors of the rates from the host),
+// and what a thread adds to (tacc, dtheta) is loaded ahead.  Reverse step with
+// its replay, us, five kernels -> one -> now: 256 x 128 21.9 -> 12.0 -> 9.9,
+// 800 x 400 61 -> 55 -> 43, 1600 x 800 245 -> 238 -> 159.  In FP64 the repeated
+// work costs more than it saves (the FP64 pipe is the limit: 800 x 400 816 us,
+// in one kernel 1040), so FP64 keeps the kernels below: 682 now; 256 x 128
+// 129 -> 111.
 template <typename R>
 __global__ void __launch_bounds__(kStepThreads)
-    k_adj_step(Mdl<R> m, int strips, int bands, const R *__restrict__ f, const R *__restrict__ lam_in,
+    k_adj_step(Mdl<R> m, AdjRates<R> K, int strips, int bands, const R *__restrict__ f, const R *__restrict__ lam_in,
                R *__restrict__ lam_out, const double *__restrict__ coef, const double *__restrict__ dcoef,
                double *__restrict__ tacc, double *__restrict__ dtheta, int *flag) {
+  constexpr int kAN = (kAH + 2) * kAW;  // aux: a row of zeros beyond each wall
   __shared__ R srho[kFH * kFW], spsi[kFH * kFW], sU[kFH * kFW];
-  __shared__ R saux[5 * kAH * kAW];
-  __shared__ double sgp[2][4][kAW];  // ghost-rule parts by wall, part, column (as in aux)
+  __shared__ R saux[5 * kAN];
+  __shared__ R sgp[2][4][kAW];  // ghost-rule parts by wall, part, column (as in aux)
   const int band = (int)(blockIdx.x / (unsigned)strips);
   const int x0 = ((int)blockIdx.x - band * strips) * kTW, wr = min(kTW, m.nx - x0);
   const int first = m.walls ? 1 : 0, rows = m.walls ? m.ny - 2 : m.ny;
@@ -319,17 +428,26 @@ __global__ void __launch_bounds__(kStepThreads)
   const size_t n = (size_t)m.nx * m.ny;
   const bool geo = m.walls && m.wetting == LBM_WET_GEOMETRIC;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
 
   // this thread's node: rows ya - 1 .. yb, columns x0 - 2 .. x0 + wr + 1
   const int cy = threadIdx.x / kAW, cx = threadIdx.x - cy * kAW, v = ya - 1 + cy;
   const bool on = cy < hr + 2 && cx < wr + 4;  // (in a walled domain all these rows exist)
-  const int y = m.wy(v), x = m.wx(x0 - 2 + cx);
+  const int y = m.wy(v), x = m.wx(x0 - 2 + cx), w = y == 0 ? 0 : 1;
   const bool solid = m.solid_row(y), own = on && cx >= 2 && cx < wr + 2 && (solid || (cy >= 1 && cy <= hr));
+  const bool wall = on && solid && geo && cx >= 1 && cx < wr + 3;  // a ghost node whose transposed rule is needed
   const size_t i = (size_t)y * m.nx + x;
-  const int jf = (cy + 1) * kFW + cx + 1, ja = cy * kAW + cx;  // its place among the fields and aux
+  const int jf = (cy + 1) * kFW + cx + 1, ja = (cy + 1) * kAW + cx;  // its place among the fields and aux
   auto nb = [&](int ex, int ey) { return jf + ey * kFW + ex; };
   auto ax = [&](int ex, int ey) { return ja + ey * kAW + ex; };
+  R c = (R)0, cot = (R)0;
+  double dc = 0.0, dcot = 0.0;
+  if (wall) {
+    c = (R)coef[w * m.nx + x];
+    cot = (R)coef[2 * m.nx + w * m.nx + x];
+    dc = dcoef[w * m.nx + x];
+    dcot = dcoef[2 * m.nx + w * m.nx + x];
+  }
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   R ls[9], fl[9], cl[9];
   if (on && !solid) {
 #pragma unroll
@@ -339,51 +457,61 @@ __global__ void __launch_bounds__(kStepThreads)
       fl[a] = f[a * n + i];
     }
   }
+  // the sums this thread adds to, loaded ahead of their use
+  const double t0 = own ? tacc[i] : 0.0, th0 = own && wall ? dtheta[w * m.nx + x] : 0.0;
   // fields: rows ya - 2 .. yb + 1, columns x0 - 3 .. x0 + wr + 2
   bool bad = false;
   const int t = threadIdx.x, fy = t / kFW, fx = t - fy * kFW, fv = ya - 2 + fy;
-  if (fy < hr + 4 && fx < wr + 6 && !(m.walls && (fv < 0 || fv >= m.ny))) {
-    const int y = m.wy(fv), x = m.wx(x0 - 3 + fx);
-    R r, psi = (R)0, U = (R)0;
-    if (!m.solid_row(y)) {
-      r = node_rho(f, n, (size_t)y * m.nx + x);
-      psi_U(m, r, psi, U);
-      bad |= !(r > (R)0) || r > m.rho_max;
-    } else if (geo) {
-      const int w = y == 0 ? 0 : 1;
-      const size_t b1 = (size_t)(w == 0 ? 1 : m.ny - 2) * m.nx, b2 = (size_t)(w == 0 ? 2 : m.ny - 3) * m.nx;
-      r = ghost_rho(m, node_rho(f, n, b1 + m.wx(x - 1)), node_rho(f, n, b1 + x), node_rho(f, n, b1 + m.wx(x + 1)),
-                    node_rho(f, n, b2 + x), (R)coef[w * m.nx + x], (R)coef[2 * m.nx + w * m.nx + x]);
-      if (r < m.rho_max) psi_U(m, r, psi, U);
-    } else {
-      r = (R)0;
+  if (fy < hr + 4 && fx < wr + 6) {
+    R r = (R)0, psi = (R)0, U = (R)0;
+    if (!(m.walls && (fv < 0 || fv >= m.ny))) {
+      const int y = m.wy(fv), x = m.wx(x0 - 3 + fx);
+      if (!m.solid_row(y)) {
+        r = node_rho(f, n, (size_t)y * m.nx + x);
+        node_eos(m, r, psi, U);
+        bad |= !(r > (R)0) || r > m.rho_max;
+      } else if (geo) {
+        const int w = y == 0 ? 0 : 1;
+        const size_t b1 = (size_t)(w == 0 ? 1 : m.ny - 2) * m.nx, b2 = (size_t)(w == 0 ? 2 : m.ny - 3) * m.nx;
+        r = ghost_rho(m, node_rho(f, n, b1 + m.wx(x - 1)), node_rho(f, n, b1 + x), node_rho(f, n, b1 + m.wx(x + 1)),
+                      node_rho(f, n, b2 + x), (R)coef[w * m.nx + x], (R)coef[2 * m.nx + w * m.nx + x]);
+        if (r < m.rho_max) node_eos(m, r, psi, U);
+      }
     }
     srho[t] = r;
     spsi[t] = psi;
     sU[t] = U;
   }
   if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(flag, 1);
-  if (on && !solid) {
-    R Fx, Fy, Qxx, Qyy, Qxy, a5[5];
-    force_Q(m, spsi, sU, y, nb, Fx, Fy, Qxx, Qyy, Qxy);
-    adj_collide(m, fl, ls, srho[jf], Fx, Fy, cl, a5);
+  if (on) {
+    R a5[5] = {(R)0, (R)0, (R)0, (R)0, (R)0};
+    if (!solid) {
+      R Fx, Fy;
+      force(m, spsi, sU, y, nb, Fx, Fy);
+      adj_collide(m, K, fl, ls, srho[jf], Fx, Fy, cl, a5);
+    }
 #pragma unroll
-    for (int k = 0; k < 5; ++k) saux[k * kAH * kAW + ja] = a5[k];
+    for (int k = 0; k < 5; ++k) {
+      saux[k * kAN + ja] = a5[k];
+      if (solid) saux[k * kAN + ja + (cy == 0 ? -kAW : kAW)] = (R)0;
+    }
   }
   __syncthreads();
   // dL/drho: the tile's nodes, and the ghost nodes of one more column each side
   R rb = (R)0;
-  if (own || (on && solid && geo && cx >= 1 && cx < wr + 3)) {
-    double tb;
-    adj_psi(m, spsi, saux, kAH * kAW, y, srho[jf], nb, ax, rb, tb);
-    if (own) tacc[i] += tb;
-    if (solid && geo) {
-      const int w = y == 0 ? 0 : 1, s = w == 0 ? kFW : -kFW;
-      double part[4];
-      const double dth = adj_ghost(m, srho[jf + s - 1], srho[jf + s], srho[jf + s + 1], srho[jf + 2 * s],
-                                   (R)coef[w * m.nx + x], (R)coef[2 * m.nx + w * m.nx + x], dcoef[w * m.nx + x],
-                                   dcoef[2 * m.nx + w * m.nx + x], rb, part);
-      if (own) dtheta[w * m.nx + x] += dth;
+  if (own || wall) {
+    R tb;
+    adj_psi(m, spsi, saux, kAN, y, srho[jf], nb, ax, rb, tb);
+    if (own) tacc[i] = t0 + (double)tb;
+    if (wall) {
+      const int s = w == 0 ? kFW : -kFW;
+      R part[4], cb, cotb;
+      if (m.n_iter <= 4)
+        adj_ghost<4>(m.n_iter, m.ghost_max, srho[jf + s - 1], srho[jf + s], srho[jf + s + 1], srho[jf + 2 * s], c, cot, rb, part, cb, cotb);
+      else
+        adj_ghost_any(m.n_iter, m.ghost_max, srho[jf + s - 1], srho[jf + s], srho[jf + s + 1], srho[jf + 2 * s], c, cot, rb, part, cb,
+                      cotb);
+      if (own) dtheta[w * m.nx + x] = th0 + (m.n_iter > 0 ? (double)cb * dc : (double)cotb * dcot);
 #pragma unroll
       for (int k = 0; k < 4; ++k) sgp[w][k][cx] = part[k];
     }
@@ -401,8 +529,8 @@ __global__ void __launch_bounds__(kStepThreads)
     for (int w = 0; w < 2; ++w) {
       const int y1 = w == 0 ? 1 : m.ny - 2, y2 = w == 0 ? 2 : m.ny - 3;
       // boundary row: this node is x-1 of wall node x+1, x+1 of wall node x-1, and x of wall node x
-      if (y == y1) r += sgp[w][0][cx + 1] + sgp[w][1][cx - 1] + sgp[w][2][cx];
-      if (y == y2) r += sgp[w][3][cx];
+      if (y == y1) r += (double)sgp[w][0][cx + 1] + (double)sgp[w][1][cx - 1] + (double)sgp[w][2][cx];
+      if (y == y2) r += (double)sgp[w][3][cx];
     }
     rb = (R)r;
   }
@@ -413,13 +541,17 @@ __global__ void __launch_bounds__(kStepThreads)
 // ---- the four kernels of a reverse step on whole fields (FP64, see reverse_step) --
 
 template <typename R>
-__global__ void k_adj_collide(Mdl<R> m, const R *__restrict__ f, const R *__restrict__ fields,
+__global__ void k_adj_collide(Mdl<R> m, AdjRates<R> K, const R *__restrict__ f, const R *__restrict__ fields,
                               const R *__restrict__ lam_in, R *__restrict__ lam_out, R *__restrict__ aux) {
   size_t n = (size_t)m.nx * m.ny;
   size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   int y = (int)(i / m.nx), x = (int)(i - (size_t)y * m.nx);
-  if (m.solid_row(y)) return;
+  if (m.solid_row(y)) {
+#pragma unroll
+    for (int k = 0; k < 5; ++k) aux[k * n + i] = (R)0;
+    return;
+  }
   // adjoint of the post-collision populations (transpose of the push streaming)
   R ls[9], fl[9], cl[9], ax[5];
 #pragma unroll
@@ -428,9 +560,9 @@ __global__ void k_adj_collide(Mdl<R> m, const R *__restrict__ f, const R *__rest
     ls[a] = m.solid_row(yt) ? lam_in[OPP(a) * n + i] : lam_in[a * n + (size_t)yt * m.nx + m.wx(x + EX(a))];
     fl[a] = f[a * n + i];
   }
-  R Fx, Fy, Qxx, Qyy, Qxy;
-  force_Q(m, fields + n, fields + 2 * n, y, FieldNb<R>{m, y, x}, Fx, Fy, Qxx, Qyy, Qxy);
-  adj_collide(m, fl, ls, fields[i], Fx, Fy, cl, ax);
+  R Fx, Fy;
+  force(m, fields + n, fields + 2 * n, y, FieldNb<R>{m, y, x}, Fx, Fy);
+  adj_collide(m, K, fl, ls, fields[i], Fx, Fy, cl, ax);
 #pragma unroll
   for (int a = 0; a < 9; ++a) lam_out[a * n + i] = cl[a];
 #pragma unroll
@@ -445,8 +577,7 @@ __global__ void k_adj_psi(Mdl<R> m, const R *__restrict__ fields, const R *__res
   if (i >= n) return;
   int y = (int)(i / m.nx), x = (int)(i - (size_t)y * m.nx);
   const FieldNb<R> nb{m, y, x};
-  R rb;
-  double tb;
+  R rb, tb;
   adj_psi(m, fields + n, aux, n, y, fields[i], nb, nb, rb, tb);
   rhob_out[i] = rb;
   tacc[i] += tb;
@@ -461,12 +592,16 @@ __global__ void k_adj_ghost(Mdl<R> m, const R *__restrict__ fields, const double
   int w = t / m.nx, x = t - w * m.nx;
   int yg = w == 0 ? 0 : m.ny - 1, y1 = w == 0 ? 1 : m.ny - 2, y2 = w == 0 ? 2 : m.ny - 3;
   const R *r1 = fields + (size_t)y1 * m.nx, *r2 = fields + (size_t)y2 * m.nx;
-  double part[4];
-  dtheta[w * m.nx + x] += adj_ghost(m, r1[m.wx(x - 1)], r1[x], r1[m.wx(x + 1)], r2[x], (R)coef[w * m.nx + x],
-                                    (R)coef[2 * m.nx + w * m.nx + x], dcoef[w * m.nx + x],
-                                    dcoef[2 * m.nx + w * m.nx + x], rhob[(size_t)yg * m.nx + x], part);
+  R part[4], cb, cotb;
+  const R c = (R)coef[w * m.nx + x], cot = (R)coef[2 * m.nx + w * m.nx + x], gb = rhob[(size_t)yg * m.nx + x];
+  if (m.n_iter <= 4)
+    adj_ghost<4>(m.n_iter, m.ghost_max, r1[m.wx(x - 1)], r1[x], r1[m.wx(x + 1)], r2[x], c, cot, gb, part, cb, cotb);
+  else
+    adj_ghost_any(m.n_iter, m.ghost_max, r1[m.wx(x - 1)], r1[x], r1[m.wx(x + 1)], r2[x], c, cot, gb, part, cb, cotb);
+  dtheta[w * m.nx + x] +=
+      m.n_iter > 0 ? (double)cb * dcoef[w * m.nx + x] : (double)cotb * dcoef[2 * m.nx + w * m.nx + x];
 #pragma unroll
-  for (int k = 0; k < 4; ++k) gpart[((size_t)w * 4 + k) * m.nx + x] = part[k];
+  for (int k = 0; k < 4; ++k) gpart[((size_t)w * 4 + k) * m.nx + x] = (double)part[k];
 }
 
 template <typename R>
@@ -554,7 +689,7 @@ int reverse_step(lbm_ctx *C, lbm_tape *T, const void *f, int lin) {
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = C->capturing ? 0 : 1;
-    ACK(cudaLaunchKernelEx(&cfg, k_adj_step<R>, m, strips, bands, (const R *)f, (const R *)lam_in, lam_out,
+    ACK(cudaLaunchKernelEx(&cfg, k_adj_step<R>, m, AdjRates<R>(C->dp), strips, bands, (const R *)f, (const R *)lam_in, lam_out,
                            (const double *)C->d_coef, (const double *)C->d_dcoef, T->tacc, T->dtheta, C->d_flag));
     ++C->launches;
     return LBM_OK;
@@ -564,7 +699,7 @@ int reverse_step(lbm_ctx *C, lbm_tape *T, const void *f, int lin) {
     const unsigned g = (unsigned)((n + B - 1) / B), gw = (unsigned)((2 * C->nx + B - 1) / B);
     const R *fields = (const R *)C->d_fields;
     ACK(lbm_ref_fields(C, (const double *)f, (double *)C->d_fields, &C->launches));
-    k_adj_collide<R><<<g, B, 0, C->stream>>>(m, (const R *)f, fields, lam_in, lam_out, (R *)T->aux);
+    k_adj_collide<R><<<g, B, 0, C->stream>>>(m, AdjRates<R>(C->dp), (const R *)f, fields, lam_in, lam_out, (R *)T->aux);
     k_adj_psi<R><<<g, B, 0, C->stream>>>(m, fields, (const R *)T->aux, (R *)T->rhob, T->tacc);
     C->launches += 2;
     const int geo = C->walls && m.wetting == LBM_WET_GEOMETRIC;
