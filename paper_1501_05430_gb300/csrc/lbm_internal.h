@@ -127,6 +127,9 @@ cudaError_t lbm_tile_pair(const lbm_ctx *C, const void *src, void *dst, unsigned
 void lbm_adjoint_free_tape(lbm_ctx *C);
 
 // ---- lbm_measure.cu: reductions -------------------------------------------
+// n values between FP32 and double
+cudaError_t lbm_widen(const lbm_ctx *C, const float *in, double *out, size_t n, unsigned long long *launches);
+cudaError_t lbm_narrow(const lbm_ctx *C, const double *in, float *out, size_t n, unsigned long long *launches);
 cudaError_t lbm_rho64(const lbm_ctx *C, const void *f, double *rho, unsigned long long *launches);
 // the same for rows [row0, row1) only (rho indexed like the whole field)
 cudaError_t lbm_rho64_rows(const lbm_ctx *C, const void *f, double *rho, int row0, int row1,

@@ -458,7 +458,25 @@ __global__ void __launch_bounds__(kAThreads) k_angle(lbm_angle_args A, const lbm
 
 inline unsigned nblk(size_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
+// FP32 populations to and from the caller's doubles.
+template <typename From, typename To>
+__global__ void k_convert(const From *__restrict__ in, To *__restrict__ out, size_t n) {
+  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) out[i] = (To)in[i];
+}
+
 }  // namespace
+
+cudaError_t lbm_widen(const lbm_ctx *C, const float *in, double *out, size_t n, unsigned long long *launches) {
+  k_convert<<<(unsigned)((n + 255) / 256), 256, 0, C->stream>>>(in, out, n);
+  ++*launches;
+  return cudaGetLastError();
+}
+cudaError_t lbm_narrow(const lbm_ctx *C, const double *in, float *out, size_t n, unsigned long long *launches) {
+  k_convert<<<(unsigned)((n + 255) / 256), 256, 0, C->stream>>>(in, out, n);
+  ++*launches;
+  return cudaGetLastError();
+}
 
 cudaError_t lbm_rho64_rows(const lbm_ctx *C, const void *f, double *rho, int row0, int row1,
                            unsigned long long *launches) {

@@ -103,3 +103,18 @@ def test_fp32_mass_is_the_exact_sum(nx, ny, walls):
         f[3, 2, 1] = np.inf
         s.set_f(f)
         assert s.mass() == math.inf
+
+
+@pytest.mark.parametrize("nx,ny", [(33, 7), (64, 40)])
+def test_populations_through_doubles(nx, ny):
+    """lbm_set_f rounds to nearest, lbm_get_f is exact, through either buffer
+    (the field queries' is there after the first of them)."""
+    sim, (rv, rl) = _sim(nx, ny, 32)
+    with sim as s:
+        for seed in (1, 2):
+            f = np.random.default_rng(seed).uniform(1e-3, 1.0, (9, ny, nx))
+            f[:, 3, 3] = (1e-42, 1e-46, 3e38, 0.0, -0.0, -1.5, 1 / 3, 2.0**-127, 1 + 2.0**-24)
+            s.set_f(f)
+            assert np.array_equal(s.f(), f.astype(np.float32).astype(np.float64))
+            s.set_f(I.random_distributions(np.full((ny, nx), rv), seed))
+            s.u()
