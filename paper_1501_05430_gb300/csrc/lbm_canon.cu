@@ -43,8 +43,20 @@ __device__ __forceinline__ F2 operator/(F2 a, F2 b) { return {make_float2(a.v.x 
 __device__ __forceinline__ F2 vfma(F2 a, F2 b, F2 c) { return {__ffma2_rn(a.v, b.v, c.v)}; }
 __device__ __forceinline__ double vfma(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float vfma(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ F2 both(float c) { return {make_float2(c, c)}; }
+// sqrt(max(0, a)), the bits of sqrtf, from the hardware's approximation y by one
+// coupled Newton step for sqrt and 1/(2 sqrt) and a last one with the exact
+// remainder (Markstein, IBM J. Res. Dev. 34, 1990; compared with sqrtf over
+// every significand): packed, where sqrtf is a branch and nine instructions for
+// each lane.
 __device__ __forceinline__ F2 root0(F2 a) {
-  return {make_float2(sqrtf(fmaxf(0.0f, a.v.x)), sqrtf(fmaxf(0.0f, a.v.y)))};
+  const float x = fmaxf(0.0f, a.v.x), z = fmaxf(0.0f, a.v.y);
+  float yx, yz;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(yx) : "f"(fmaxf(x, 1.17549435e-38f)));
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(yz) : "f"(fmaxf(z, 1.17549435e-38f)));
+  const F2 s = {make_float2(x, z)}, y = {make_float2(yx, yz)}, g = s * y, nh = both(-0.5f) * y;
+  const F2 e = vfma(nh, g, both(0.5f)), g1 = vfma(g, e, g), nh1 = vfma(nh, e, nh);
+  return vfma(vfma(g1, g1, -s), nh1, g1);
 }
 __device__ __forceinline__ double root0(double a) { return sqrt(fmax(0.0, a)); }
 __device__ __forceinline__ float root0(float a) { return sqrtf(fmaxf(0.0f, a)); }
@@ -52,6 +64,32 @@ __device__ __forceinline__ float root0(float a) { return sqrtf(fmaxf(0.0f, a)); 
 __device__ __forceinline__ F2 where_le(F2 x, float lim, F2 a, F2 b) {
   return {make_float2(x.v.x <= lim ? a.v.x : b.v.x, x.v.y <= lim ? a.v.y : b.v.y)};
 }
+// Quotients by one divisor.  A lane pair takes two corrections of a y with y = 1/b
+// and the exact remainders, the bits of a division (Markstein, as above), packed:
+// the divisions of two lanes were a fifth of the FP32 step's instructions.  Where
+// the divisor is 0 (a state that counts as unstable) it gives NaN; what the field
+// queries return of the velocity is divided plainly.
+template <class V>
+struct Divisor {
+  V b;
+  __device__ __forceinline__ explicit Divisor(V d) : b(d) {}
+  __device__ __forceinline__ V under(V a) const { return a / b; }
+};
+template <>
+struct Divisor<F2> {
+  F2 nb, y;
+  __device__ __forceinline__ explicit Divisor(F2 b) : nb(-b) {
+    float x, z;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(x) : "f"(b.v.x));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(z) : "f"(b.v.y));
+    y = {make_float2(x, z)};
+    y = vfma(vfma(nb, y, both(1.0f)), y, y);
+  }
+  __device__ __forceinline__ F2 under(F2 a) const {
+    const F2 q = a * y, q1 = vfma(vfma(nb, q, a), y, q);
+    return vfma(vfma(nb, q1, a), y, q1);
+  }
+};
 template <class R>
 __device__ __forceinline__ R where_le(R x, R lim, R a, R b) {
   return x <= lim ? a : b;
@@ -144,7 +182,7 @@ __device__ __forceinline__ void psi_U(const Canon<R> &m, V rho, V &psi, V &U) {
   if (m.kind == LBM_EOS_CARNAHAN_STARLING) {
     const V eta = bc(m.b4) * rho, e2 = eta * eta, one = bc((R)1), om = one - eta;
     const V num = ((one + eta) + e2) - e2 * eta, den = (om * om) * om;
-    p = (((rho * bc(m.Rg)) * bc(m.T)) * num) / den - (bc(m.a) * rho) * rho;
+    p = Divisor<V>(den).under(((rho * bc(m.Rg)) * bc(m.T)) * num) - (bc(m.a) * rho) * rho;
   } else {
     p = where_le(rho, m.r1, rho * bc(m.thv),
                  where_le(rho, m.r2, bc(m.p1) + (rho - bc(m.r1)) * bc(m.thm),
@@ -295,7 +333,8 @@ __device__ __forceinline__ void collide(const Canon<R> &m, const W &win, int row
   const V qy = ((vfma(m2, d24, f[5]) + f[6]) - f[7]) - f[8];
   const V nn = ((f[1] - f[2]) + f[3]) - f[4];
   const V no = ((f[5] - f[6]) + f[7]) - f[8];
-  const V vx = vfma(half, Fx, jx) / rho, vy = vfma(half, Fy, jy) / rho;
+  const Divisor<V> by(rho);
+  const V vx = by.under(vfma(half, Fx, jx)), vy = by.under(vfma(half, Fy, jy));
   const V vx2 = vx * vx, vy2 = vy * vy, v3 = bc((R)3) * (vx2 + vy2);
   const V vxF = vx * Fx, vyF = vy * Fy, S1 = bc((R)6) * (vxF + vyF);
   const V rvx = rho * vx, rvy = rho * vy;
