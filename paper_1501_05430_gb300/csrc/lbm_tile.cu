@@ -83,18 +83,23 @@ TileKernel kernel_ptr(const lbm_ctx *C, int rows) {
 
 }  // namespace
 
-// Which kernel runs a domain, from measurements of both (us per step, general
-// rates, ring / tile of 6 rows):
-//  - while both state arrays (72 bytes per node) stay in the 126 MB L2 the tile
-//    kernel wins: 1280 x 1280 28.5 / 26.8, 1400 x 1200 28.4 / 27.4; past it the
-//    ring's deep prefetch does: 2048 x 1024 31.3 / 33.2, 4096 x 2048 107 / 119;
-//  - at any size where the ring's 256-column strips hold over a ninth more
-//    columns than the tile's 64-column ones (its threads past nx idle):
-//    128 x 32000 98.8 / 59.1, 300 x 8000 56.7 / 39.5, 640 x 8000 82.4 / 76.5,
-//    1344 x 2048 44.5 / 43.2; at 720 x 6000, equal columns, 64.8 / 67.5.
-// Tiles of 4 rows up to 2^20 nodes (more CTAs, a shorter CTA: 256 x 128 2.95
-// against 3.26 us, 1024 x 512 9.1 / 9.4), of 6 rows above (fewer repeated
-// loads: 1200 x 1200 23.9 against 22.9).
+// Which kernel runs a domain, by the columns x rows each works through (the ring's
+// strips of 256 columns, the tile's of 64), from measurements of both.  While the
+// two state arrays (72 bytes per node) mostly stay in the 126 MB L2 the tile kernel
+// wins, past it the ring's deep prefetch does; the ring waits ~1.4 us for the ghost
+// rows of a walled domain, and general rates cost it more than the tile.  us per
+// step, ring / tile (6 rows), unit | general rates:
+//    walled    1280 x 1100 22.2 / 21.0 | 22.9 / 21.3, 1280 x 1200 23.0 / 24.8 | 23.7 / 23.5,
+//              1792 x 960 26.3 / 27.7 | 27.3 / 26.4, 2048 x 960 28.8 / 31.2 | 30.0 / 30.4,
+//              4096 x 2048 101 / 122 | 107 / 117;
+//    periodic  1024 x 1300 19.3 / 19.2 | 20.7 / 20.1, 1536 x 900 19.6 / 20.3 | 20.9 / 21.3.
+// Beyond, the tile wins where the ring's strips hold so many more columns than the
+// domain (threads past nx idle): walled 448 x 3600 25.6 / 25.9 | 27.6 / 24.8,
+// 1344 x 1344 29.5 / 29.5 | 29.9 / 27.9, 2624 x 1500 54.6 / 59.2 | 55.6 / 57.2,
+// 320 x 8000 52 / 39 | 56 / 38.
+// Tiles of 4 rows up to a million nodes (more CTAs, a shorter CTA: 256 x 128 2.95
+// against 3.26 us, 1024 x 512 9.1 / 9.4), of 6 rows above (fewer repeated loads:
+// 1024 x 1024 14.8 against 14.2, 1280 x 1000 19.3 / 18.4).
 // Two steps per launch up to 50,000 nodes, where the launch and the loads are
 // most of a step and two thirds of the collisions can be made twice: us per step,
 // one / two, 64 x 32 2.65 / 2.07, 256 x 128 2.92 / 2.49, 300 x 100 2.91 / 2.20;
@@ -106,8 +111,9 @@ void lbm_tile_plan(lbm_ctx *C) {
   const long long nodes = (long long)C->nx * C->ny;
   const int strips = (C->nx + kW - 1) / kW, ring_cols = (C->nx + 255) / 256 * 256;
   const int nrows = C->walls ? C->ny - 2 : C->ny;
-  if (nodes > 1600000 && 10LL * strips * kW > 9LL * ring_cols) return;
-  const int R = nodes <= (1 << 20) ? 4 : 6, bands = (nrows + R - 1) / R;
+  const long long limit = C->walls ? (C->fused_unit ? 1420000 : 1720000) : (C->fused_unit ? 1360000 : 1420000);
+  if (1LL * strips * kW * C->ny > limit && 100LL * strips * kW > (C->fused_unit ? 85LL : 90LL) * ring_cols) return;
+  const int R = nodes <= 1000000 ? 4 : 6, bands = (nrows + R - 1) / R;
   if (bands > 65535) return;  // grid.y
   C->tile_rows = R;
   C->tile_pairs = nodes <= 50000 && C->nx >= 8;

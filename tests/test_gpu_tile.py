@@ -25,8 +25,9 @@ MODELS = {
 }
 # one and several strips with a ragged last one (64 columns a tile, 58 with two
 # steps per launch, which 4 columns are too few for), bands with every remainder
-# (walled: ny - 2 rows), the smallest grids
-SIZES = [(4, 5), (8, 5), (8, 6), (56, 6), (60, 7), (64, 6), (68, 8), (116, 10), (132, 9), (260, 24), (128, 13)]
+# (walled: ny - 2 rows), the smallest grids, seven strips of the ring kernel (whose
+# CTAs are then a multiple of seven)
+SIZES = [(4, 5), (8, 5), (8, 6), (56, 6), (60, 7), (64, 6), (68, 8), (116, 10), (132, 9), (260, 24), (128, 13), (1700, 100)]
 
 
 def _context(c, f, monkeypatch, ring):
