@@ -8,13 +8,15 @@
 //    freely through roundings (4 f_0 - 2 f_1 is twice 2 f_0 - f_1);
 //  - x / 3, x / 9, x / 36, x / 6, x / 12: one product and one fused
 //    multiply-add (div_const below) instead of a general division;
+//  - other FP32 quotients and square roots are corrected approximations, packed
+//    (Divisor and root0 below);
 //  - values that several sums use in the same order are formed once (prefixes
 //    of the inverse transform, psi^2, and, per node instead of per neighbour,
 //    the weighted psi and U of the FP64 kernel).
 // About 350 FP64 operations per node instead of 700, and one pass over the
 // populations instead of two and a pass over three fields (FP32: 72 bytes per
 // node instead of 132).  us per step, before -> now: FP64 100 x 60 29.6 -> 16.7,
-// 400 x 200 104 -> 79; FP32 1001 x 501 30.4 -> 15.6, 2047 x 1025 131 -> 56.
+// 400 x 200 104 -> 79; FP32 1001 x 501 30.4 -> 11.3, 2047 x 1025 131 -> 45.
 // FP64 is bound by the FP64 pipe (0.5 lanes per clock and SM quarter), FP32 by
 // instruction issue and the FMA pipe.
 #include <math.h>
@@ -623,7 +625,7 @@ cudaError_t lbm_canon_step(const lbm_ctx *C, const void *src, void *dst, unsigne
 
 // The getters' fields and the largest speed, in one pass over the populations
 // (before: fields, then seven planes of doubles, then the reduction of two of
-// them).  4096 x 2048: largest speed 590 -> 200 us.
+// them).  4096 x 2048: largest speed, a call, 609 -> 169 us.
 cudaError_t lbm_canon_fields(const lbm_ctx *C, const void *f, double *const (&o)[10], unsigned long long *launches) {
   ++*launches;
   Fields out;

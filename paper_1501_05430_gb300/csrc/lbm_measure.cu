@@ -204,7 +204,8 @@ __device__ __forceinline__ void two_sum(float2 &s, float2 &e, float2 v) {
 // The same for four nodes at once (nx % 4 == 0; groups [q0, q1)): 16-byte loads,
 // and per group a sum in single precision with its rounding errors beside it (48
 // bits), which takes a fifth of the instructions of nine exact sums: 4096 x 2048
-// 134 us (density field and sum) -> 60 us; the populations alone take 45.
+// the kernels 134 us (density field and sum) -> 54, a call 161 -> 75; the
+// populations alone take 45.
 __global__ void k_mass_x4(const float4 *__restrict__ f, size_t n4, size_t q0, size_t q1, double *partial,
                           unsigned *counter, double *out) {
   sum_range(q0, q1, partial, counter, out, [&](size_t i) {
