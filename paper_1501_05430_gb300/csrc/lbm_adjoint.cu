@@ -148,7 +148,8 @@ __device__ __forceinline__ void solid_sums(const Mdl<R> &m, int y, R &ssx, R &ss
   }
 }
 
-// Eq. 9 force (+ Eq. 14) at a fluid node: the F of force_Q.
+// Eq. 9 force (+ Eq. 14) at a fluid node of row y; nb(ex, ey) is the index of a
+// neighbour in psi and U.
 template <typename R, typename Nb>
 __device__ __forceinline__ void force(const Mdl<R> &m, const R *__restrict__ psi, const R *__restrict__ U, int y, Nb nb,
                                       R &Fx, R &Fy) {

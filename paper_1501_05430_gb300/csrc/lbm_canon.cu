@@ -1,8 +1,8 @@
-// lbm_canon.cu -- the step in the canonical evaluation order (the one of
-// lbm_ref_node.cuh), one kernel per step: FP64 domains, and FP32 domains whose
-// width the fused kernels do not take.  Every result has the bits of the
-// plain form in lbm_ref_node.cuh (compiled, like it, without contraction); the
-// operations that cost most are only arranged anew:
+// lbm_canon.cu -- the step in the canonical evaluation order (the oracle's: the
+// equations term by term, sums left to right, no contraction), one kernel per
+// step: FP64 domains, and FP32 domains whose width the fused kernels do not take.
+// Every result has the bits of that plain form; the operations that cost most are
+// only arranged anew:
 //  - a product by a power of two is exact, so the sum it goes into takes it as
 //    a fused multiply-add with the same single rounding, and such factors move
 //    freely through roundings (4 f_0 - 2 f_1 is twice 2 f_0 - f_1);

@@ -1,5 +1,5 @@
 // lbm_ref_node.cuh -- per-node arithmetic in the canonical order (model
-// constants, EOS, Eq. 9 / Eq. 17 stencil), shared by the field kernels
+// constants, EOS, ghost rule), shared by the field kernels
 // (lbm_ref.cu) and the adjoint kernels (lbm_adjoint.cu), which recompute the
 // forward quantities of a step.  Both translation units are compiled with
 // -fmad=false.
@@ -122,55 +122,5 @@ struct FieldNb {
     return (size_t)m.wy(y + ey) * m.nx + m.wx(x + ex);
   }
 };
-
-// Eq. 9 force (+ Eq. 14) and Eq. 17 tensor at a fluid node of row y; nb(ex, ey)
-// is the index of a neighbour in psi and U.
-template <typename R, typename Nb>
-__device__ __forceinline__ void force_Q(const Mdl<R> &m, const R *__restrict__ psi, const R *__restrict__ U, int y,
-                                        Nb nb, R &Fx, R &Fy, R &Qxx, R &Qyy, R &Qxy) {
-  R psi0 = psi[nb(0, 0)];
-  R spx = 0, spy = 0, sUx = 0, sUy = 0, ssx = 0, ssy = 0;
-  R qxx1 = 0, qyy1 = 0, qxy1 = 0, qxx2 = 0, qyy2 = 0, qxy2 = 0;
-#pragma unroll
-  for (int a = 1; a < 9; ++a) {
-    const auto j = nb(EX(a), EY(a));
-    R pn = psi[j], un = U[j];
-    R w = wgt<R>(a);
-    R solid = m.solid_row(m.wy(y + EY(a))) ? (R)1 : (R)0;
-    if (EX(a) != 0) {
-      R tp = w * pn, tu = w * un, ts = w * solid;
-      if (EX(a) > 0) { spx = spx + tp; sUx = sUx + tu; ssx = ssx + ts; }
-      else { spx = spx - tp; sUx = sUx - tu; ssx = ssx - ts; }
-    }
-    if (EY(a) != 0) {
-      R tp = w * pn, tu = w * un, ts = w * solid;
-      if (EY(a) > 0) { spy = spy + tp; sUy = sUy + tu; ssy = ssy + ts; }
-      else { spy = spy - tp; sUy = sUy - tu; ssy = ssy - ts; }
-    }
-    R t1 = w * (pn - psi0);
-    R t2 = w * (pn * pn - psi0 * psi0);
-    int exx = EX(a) * EX(a), eyy = EY(a) * EY(a), exy = EX(a) * EY(a);
-    if (exx) { qxx1 = qxx1 + t1; qxx2 = qxx2 + t2; }
-    if (eyy) { qyy1 = qyy1 + t1; qyy2 = qyy2 + t2; }
-    if (exy > 0) { qxy1 = qxy1 + t1; qxy2 = qxy2 + t2; }
-    if (exy < 0) { qxy1 = qxy1 - t1; qxy2 = qxy2 - t2; }
-  }
-  const R G = (R)-1;
-  R cpsi = (((R)1 - m.A) * G) * psi0;
-  R fx = -(m.A * sUx) - cpsi * spx;
-  R fy = -(m.A * sUy) - cpsi * spy;
-  if (m.wetting == LBM_WET_MARTYS_CHEN) {
-    R gp = m.Gw * psi0;
-    fx = fx + (-(gp * ssx));
-    fy = fy + (-(gp * ssy));
-  }
-  R pre = m.kappa * (G * (R)0.5);
-  R c1 = ((R)1 - m.A) * psi0, c2 = m.A * (R)0.5;
-  Fx = fx;
-  Fy = fy;
-  Qxx = pre * ((c1 * qxx1) + (c2 * qxx2));
-  Qyy = pre * ((c1 * qyy1) + (c2 * qyy2));
-  Qxy = pre * ((c1 * qxy1) + (c2 * qxy2));
-}
 
 }  // namespace lbm_ref
