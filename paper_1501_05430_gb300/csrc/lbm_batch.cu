@@ -561,9 +561,10 @@ __global__ void __launch_bounds__(kTileThreads, 5) k_batch_tile(TileArgs A) {
   const int *src = (const int *)(A.inst + t.inst);
   for (int k = threadIdx.x; k < (int)(sizeof(BInst) / sizeof(int)); k += kTileThreads) ((int *)&P)[k] = src[k];
   const int par = A.cur[t.inst] ^ A.phase;
-  __syncthreads();
   if (A.pdl) asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (*(volatile const int *)(A.iflag + t.inst) & 1) return;  // a blown-up instance is frozen
+  // a blown-up instance is frozen; one thread looks, since CTAs of this launch may
+  // be raising the flag and a tile is made by all of its warps or by none
+  if (__syncthreads_or(threadIdx.x == 0 && (*(volatile const int *)(A.iflag + t.inst) & 1))) return;
   auto ready = [] {};
   auto unstable = [&] {
     atomicOr(A.iflag + t.inst, 1);

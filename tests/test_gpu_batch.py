@@ -352,3 +352,54 @@ def test_tile_form_freezes_an_unstable_instance():
         assert np.array_equal(b[1].f(), f, equal_nan=True)
         assert b.node_updates()[1] == upd[1]
     _close(cases)
+
+
+EX, EY, OPP = (0, 1, 0, -1, 0, 1, -1, -1, 1), (0, 0, 1, 0, -1, 1, 1, -1, -1), (0, 3, 4, 1, 2, 7, 8, 5, 6)
+
+
+def _streamed(nx, ny, xs, ys):
+    """Indices (a, y, x) that the nodes ys x xs of a walled domain stream to."""
+    a, y, x = (v.ravel() for v in np.meshgrid(np.arange(9), ys, xs, indexing="ij"))
+    yt = y + np.take(EY, a)
+    wall = (yt == 0) | (yt == ny - 1)
+    return np.where(wall, np.take(OPP, a), a), np.where(wall, y, yt), np.where(wall, x, (x + np.take(EX, a)) % nx)
+
+
+@pytest.mark.parametrize("on_stream", [False, True])
+def test_tiles_of_an_instance_that_blows_up_are_made_whole_or_left_out(on_stream):
+    """Other tiles of the launch that finds a density of NaN may see the flag or
+    not; each has either streamed all of its nodes, and counted them, or none."""
+    import torch
+
+    nx, ny, n = 132, 34, 24
+    c = _cases([(nx, ny, dict(theta="random"))])[0]
+    tiles = [(np.arange(x, min(x + 64, nx)), np.arange(y, min(y + 4, ny - 1)))
+             for y in range(1, ny - 1, 4) for x in range(0, nx, 64)]
+    index = [_streamed(nx, ny, xs, ys) for xs, ys in tiles]
+    nodes = np.array([len(xs) * len(ys) for xs, ys in tiles])
+    rng = np.random.default_rng(4)
+    starts, want = [], []
+    for _ in range(n):
+        f = c.f0.copy()
+        f[:, rng.integers(1, ny - 1), rng.integers(0, nx)] = np.nan
+        with L.Lbm(nx, ny, c.geos, c.T, c.tau, theta=c.theta, params=c.params, torch_state=False) as one:
+            one.set_f(f)
+            one.step(1)
+            starts.append(f)
+            want.append(one.f())
+    stream = torch.cuda.Stream() if on_stream else None
+    for _ in range(4):
+        with L.LbmBatch([c.desc()] * n, stream=stream) as b:
+            assert b.plan()["items"] == n * len(tiles)
+            for inst, f in zip(b.instances, starts):
+                inst.set_f(f)
+            b.step(1)
+            assert (b.status()[1] == L.LBM_EUNSTABLE).all()
+            upd = b.node_updates()
+            for k in range(n):
+                got = b[k].f()
+                made = np.array([np.array_equal(got[i], want[k][i], equal_nan=True) for i in index])
+                left = np.array([not got[i].any() for i in index])
+                assert (made ^ left).all() and made.any()
+                assert upd[k] == nodes[made].sum()
+    c.orc.close()
