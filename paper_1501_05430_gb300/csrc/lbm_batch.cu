@@ -701,30 +701,34 @@ bool default_shape(const lbm_batch_config &c) {
          c.hold_instance == -1;
 }
 
-// Tile list of the whole batch, made once.
+// Tile list of the whole batch, made once.  LBM_ENOMEM leaves the batch without it.
 int plan_tiles(lbm_batch *B) {
-  if (!B->tiles.empty()) return LBM_OK;
+  if (B->d_tiles) return LBM_OK;
   B->tile_kind = -2;
-  for (int i = 0; i < B->n; ++i) {
-    const lbm_ctx *C = B->ctx[i];
-    const int k = C->dp.wetting == LBM_WET_GEOMETRIC ? C->dp.eos_kind : -1;
-    B->tile_kind = B->tile_kind == -2 || B->tile_kind == k ? k : -1;
-    for (int y = 1; y < C->ny - 1; y += kTileRows)
-      for (int x = 0; x < C->nx; x += lbm_tile::kW) B->tiles.push_back(BTile{i, x, y, 0});
+  try {
+    B->tiles.clear();
+    for (int i = 0; i < B->n; ++i) {
+      const lbm_ctx *C = B->ctx[i];
+      const int k = C->dp.wetting == LBM_WET_GEOMETRIC ? C->dp.eos_kind : -1;
+      B->tile_kind = B->tile_kind == -2 || B->tile_kind == k ? k : -1;
+      for (int y = 1; y < C->ny - 1; y += kTileRows)
+        for (int x = 0; x < C->nx; x += lbm_tile::kW) B->tiles.push_back(BTile{i, x, y, 0});
+    }
+  } catch (const std::bad_alloc &) {
+    return LBM_ENOMEM;
   }
-  cudaError_t e = cudaMalloc(&B->d_tiles, B->tiles.size() * sizeof(BTile));
+  BTile *dev = nullptr;
+  cudaError_t e = cudaMalloc(&dev, B->tiles.size() * sizeof(BTile));
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(B->d_tiles, B->tiles.data(), B->tiles.size() * sizeof(BTile), cudaMemcpyHostToDevice,
-                        B->stream);
+    e = cudaMemcpyAsync(dev, B->tiles.data(), B->tiles.size() * sizeof(BTile), cudaMemcpyHostToDevice, B->stream);
   if (e == cudaSuccess)
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&B->tile_occ, tile_kernel(B->tile_kind), kTileThreads, 0);
   if (e != cudaSuccess) {
     cudaGetLastError();
-    cudaFree(B->d_tiles);
-    B->d_tiles = nullptr;
-    B->tiles.clear();
+    cudaFree(dev);
     return e == cudaErrorMemoryAllocation ? LBM_ENOMEM : LBM_ECUDA;
   }
+  B->d_tiles = dev;
   return LBM_OK;
 }
 
@@ -969,13 +973,17 @@ int run_steps(lbm_batch *B, int nsteps) {
 // advances 50 whatever the width.  Measured, us per step, persistent / tile:
 // 6 of 300 x 100 47 / 6.4, 32 of 256 x 128 45 / 20, 64 of them 53 / 44, 128 of
 // them 69 / 83, 16 of 512 x 256 49 / 42, 32 of them 64 / 80, 1024 of 128 x 64
-// 236 / 162, 100 of the four sizes 102 / 122.
+// 236 / 162, 100 of the four sizes 102 / 122.  Without memory for the list of
+// tiles the persistent kernel runs.
 int choose_tiles(lbm_batch *B, const lbm_batch_config &asked) {
   double narrow = 0.0, wide = 0.0;
   for (int i = 0; i < B->n; ++i)
     (B->ctx[i]->nx <= 128 ? narrow : wide) += (double)B->ctx[i]->nx * (B->ctx[i]->ny - 2);
-  B->tile = default_shape(asked) && (narrow + wide) / 50e3 < std::max(45.0, narrow / 34e3 + wide / 68e3);
-  return B->tile ? plan_tiles(B) : LBM_OK;
+  B->tile = false;
+  if (!default_shape(asked) || (narrow + wide) / 50e3 >= std::max(45.0, narrow / 34e3 + wide / 68e3)) return LBM_OK;
+  const int st = plan_tiles(B);
+  B->tile = st == LBM_OK;
+  return st == LBM_ENOMEM ? LBM_OK : st;
 }
 
 }  // namespace
@@ -1247,9 +1255,14 @@ int lbm_batch_autotune(lbm_batch *B, int trial_steps, lbm_batch_config *best) {
     }
     cur = best_cfg;
     // the tile form last: *best stays the best persistent shape
-    if (st == LBM_OK && (st = plan_tiles(B)) == LBM_OK) {
-      B->tile = true;
-      st = trial(cur);
+    if (st == LBM_OK) {
+      const int pt = plan_tiles(B);
+      if (pt == LBM_OK) {
+        B->tile = true;
+        st = trial(cur);
+      } else if (pt != LBM_ENOMEM) {
+        st = pt;
+      }
     }
   } else {
     cudaGetLastError();
