@@ -365,7 +365,10 @@ typedef struct {
 /* Launch shape.  Zero fields take the defaults in brackets.  With every field
  * at its default (or no config) the library may run a small batch with one
  * launch per step instead (tiles of 64 columns x 4 rows, no waits); results
- * are the same. */
+ * are the same.  lbm_batch_get_config then reports a persistent shape in full,
+ * and lbm_batch_set_config on the same batch takes that shape, whatever its
+ * graph_launches and wait_seconds (which tiles do not use), for one launch per
+ * step again. */
 typedef struct {
   int threads;           /* 256 [default]: every instance in one launch of 256-thread
                             CTAs; 128: the instances up to 256 wide in a launch of their
@@ -428,7 +431,9 @@ int lbm_batch_contact_angles(lbm_batch *b, int wall, double *theta, double *H, d
  * configurations on a copy of the current state (threads x stages, then the
  * band height of each size class present, then steps_per_launch), install the
  * fastest and put the state back.  best (may be NULL) receives the fastest
- * shape; when one launch per step is faster still, that is what is installed.
+ * shape; when one launch per step is faster still, that is what is installed,
+ * and what lbm_batch_set_config with best installs on this batch (another batch
+ * takes best as the persistent shape that it is).
  * Needs one extra state-sized device allocation while it runs. */
 int lbm_batch_autotune(lbm_batch *b, int trial_steps, lbm_batch_config *best);
 

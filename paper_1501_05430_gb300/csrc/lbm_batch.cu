@@ -639,8 +639,12 @@ struct lbm_batch {
   unsigned long long *d_work;  // [n] fluid-node updates computed per instance
   int *d_cur;
   int nsm;
-  // small batches with the default shape: one launch of tile CTAs per step
+  // small batches: one launch of tile CTAs per step
   bool tile;
+  // the shape that lbm_batch_get_config and the autotuner report while it steps
+  // in tiles (has_tile_shape): given back in full, it stands for the tiles
+  bool has_tile_shape;
+  lbm_batch_config tile_shape;
   int tile_kind, tile_occ;
   std::vector<BTile> tiles;
   BTile *d_tiles;
@@ -699,6 +703,11 @@ bool default_shape(const lbm_batch_config &c) {
   return !c.threads && !c.ctas_per_sm && !c.stages && !c.band_rows[0] && !c.band_rows[1] && !c.band_rows[2] &&
          !c.band_rows[3] && !c.steps_per_launch && !c.graph_launches && c.wait_seconds == 0.0 &&
          c.hold_instance == -1;
+}
+
+bool same_shape(const lbm_batch_config &a, const lbm_batch_config &b) {
+  return a.threads == b.threads && a.ctas_per_sm == b.ctas_per_sm && a.stages == b.stages &&
+         !memcmp(a.band_rows, b.band_rows, sizeof(a.band_rows)) && a.steps_per_launch == b.steps_per_launch;
 }
 
 // Tile list of the whole batch, made once.  LBM_ENOMEM leaves the batch without it.
@@ -966,8 +975,10 @@ int run_steps(lbm_batch *B, int nsteps) {
   return LBM_OK;
 }
 
-// Whether the batch steps in tiles; only an all-default shape leaves it to the
-// library.  The persistent kernel's step lasts at least as long as a band of 32
+// The form that a shape asks for, once B->cfg holds it in full: tiles where it is
+// all default and the batch is small, or where it is the shape reported for the
+// tiles (as the autotuner's result, however its graph and wait fields were set).
+// The rule: the persistent kernel's step lasts at least as long as a band of 32
 // rows sweeps (45 us) and advances 34 nodes per ns in instances up to 128 wide
 // (three quarters of a CTA idle), about 68 in wider ones; the tile kernel
 // advances 50 whatever the width.  Measured, us per step, persistent / tile:
@@ -980,9 +991,15 @@ int choose_tiles(lbm_batch *B, const lbm_batch_config &asked) {
   for (int i = 0; i < B->n; ++i)
     (B->ctx[i]->nx <= 128 ? narrow : wide) += (double)B->ctx[i]->nx * (B->ctx[i]->ny - 2);
   B->tile = false;
-  if (!default_shape(asked) || (narrow + wide) / 50e3 >= std::max(45.0, narrow / 34e3 + wide / 68e3)) return LBM_OK;
+  const bool small = default_shape(asked) && (narrow + wide) / 50e3 < std::max(45.0, narrow / 34e3 + wide / 68e3);
+  const bool again = B->has_tile_shape && same_shape(asked, B->tile_shape) && asked.hold_instance == -1;
+  if (!small && !again) return LBM_OK;
   const int st = plan_tiles(B);
   B->tile = st == LBM_OK;
+  if (B->tile) {
+    B->has_tile_shape = true;
+    B->tile_shape = B->cfg;
+  }
   return st == LBM_ENOMEM ? LBM_OK : st;
 }
 
@@ -1268,7 +1285,11 @@ int lbm_batch_autotune(lbm_batch *B, int trial_steps, lbm_batch_config *best) {
     cudaGetLastError();
     st = LBM_ECUDA;
   }
-  B->tile = st == LBM_OK ? best_tile : tile0;
+  B->tile = st == LBM_OK ? best_tile && start.hold_instance == -1 : tile0;
+  if (st == LBM_OK) {
+    B->has_tile_shape = best_tile;
+    B->tile_shape = cur;
+  }
   // restore the state and install the winner (with the caller's graph and wait settings)
   if (st == LBM_OK) {
     cur.graph_launches = start.graph_launches;

@@ -403,3 +403,39 @@ def test_tiles_of_an_instance_that_blows_up_are_made_whole_or_left_out(on_stream
                 assert (made ^ left).all() and made.any()
                 assert upd[k] == nodes[made].sum()
     c.orc.close()
+
+
+def test_the_shape_reported_for_tiles_installs_tiles():
+    """What get_config and the autotuner report while a batch steps in tiles,
+    with other graph and wait fields (the autotuner's result is used like that),
+    keeps the tiles; any other shape, and a held instance, do not."""
+    cases = _cases([(300, 100, dict(theta="random"))] * 6)
+    with _batch(cases) as b, _batch(cases, stages=3) as ref:
+        tiles = b.plan()
+        assert tiles["smem_bytes"] == 0
+        b.set_config(b.config)
+        assert b.plan() == tiles
+        cfg = b.config
+        cfg.graph_launches, cfg.wait_seconds = 4, 1.0
+        b.set_config(cfg)
+        assert b.plan() == tiles
+        b.step(35)
+        cfg.hold_instance = 2
+        b.set_config(cfg)
+        assert b.plan()["smem_bytes"] > 0
+        cfg.hold_instance = -1
+        cfg.steps_per_launch += 1
+        b.set_config(cfg)
+        assert b.plan()["smem_bytes"] > 0
+        b.step(3)
+        best = b.autotune(trial_steps=8)
+        tuned = b.plan()
+        assert tuned == tiles  # (a persistent step of this batch takes seven times as long)
+        best.graph_launches = 2
+        b.set_config(best)
+        assert b.plan() == tiles
+        b.step(2)
+        ref.step(40)
+        for x, y in zip(b.instances, ref.instances):
+            assert np.array_equal(x.f(), y.f())
+    _close(cases)
