@@ -192,36 +192,63 @@ __global__ void k_mass(const R *__restrict__ f, size_t n, size_t i0, size_t i1, 
   sum_range(i0, i1, partial, counter, out, [&](size_t i) { return node_rho64(f, n, i); });
 }
 
-// s + e += v for lane pairs, without loss: e takes the rounding error of the sum
-// (Knuth's two-sum).
-__device__ __forceinline__ void two_sum(float2 &s, float2 &e, float2 v) {
-  const float2 m1 = make_float2(-1.0f, -1.0f);
-  const float2 t = __fadd2_rn(s, v), b = __ffma2_rn(s, m1, t);
-  e = __fadd2_rn(e, __fadd2_rn(__ffma2_rn(__ffma2_rn(b, m1, t), m1, s), __ffma2_rn(b, m1, v)));
-  s = t;
+// The sum of the populations of four nodes, rounded once.  Where all 36 are normal
+// numbers within 31 binades, each is an integer below 2^54 times the last place of
+// the smallest ones, and the sum of the integers stays below 2^60: one widening
+// multiply-add per value.  Otherwise (zeros among them too) the sum of the four
+// densities.
+__device__ __forceinline__ double sum36(const float4 (&v)[9]) {
+  unsigned lo = 0xffffffffu, hi = 0u;
+  auto span = [&](float x) {
+    const unsigned u = __float_as_uint(x) & 0x7fffffffu;
+    lo = min(lo, u);
+    hi = max(hi, u);
+  };
+#pragma unroll
+  for (int a = 0; a < 9; ++a) {
+    span(v[a].x);
+    span(v[a].y);
+    span(v[a].z);
+    span(v[a].w);
+  }
+  const int emin = (int)(lo >> 23), emax = (int)(hi >> 23);
+  if (emin >= 1 && emax <= 254 && emax - emin <= 30) {
+    long long S = 0;
+    auto add = [&](float x) {
+      const unsigned u = __float_as_uint(x);
+      const int m = (int)((u & 0x7fffffu) | 0x800000u);
+      S += (long long)((int)u < 0 ? -m : m) * (1 << (((int)(u >> 23) - emin) & 31));
+    };
+#pragma unroll
+    for (int a = 0; a < 9; ++a) {
+      add(v[a].x);
+      add(v[a].y);
+      add(v[a].z);
+      add(v[a].w);
+    }
+    return (double)S * __longlong_as_double((long long)(emin - 150 + 1023) << 52);
+  }
+  double r = 0.0;
+#pragma unroll 1
+  for (int k = 0; k < 4; ++k) {
+    float q[9];
+#pragma unroll
+    for (int a = 0; a < 9; ++a) q[a] = k == 0 ? v[a].x : (k == 1 ? v[a].y : (k == 2 ? v[a].z : v[a].w));
+    r += sum9(q);
+  }
+  return r;
 }
 
-// The same for four nodes at once (nx % 4 == 0; groups [q0, q1)): 16-byte loads,
-// and per group a sum in single precision with its rounding errors beside it (48
-// bits), which takes a fifth of the instructions of nine exact sums: 4096 x 2048
-// the kernels 134 us (density field and sum) -> 54, a call 161 -> 75; the
-// populations alone take 45.
+// Mass of four nodes at once (nx % 4 == 0; groups [q0, q1)): 16-byte loads.
+// 4096 x 2048, a call: the densities and their sum in two kernels 161 us, each
+// node's density by itself 128, so 75; the populations alone take 45.
 __global__ void k_mass_x4(const float4 *__restrict__ f, size_t n4, size_t q0, size_t q1, double *partial,
                           unsigned *counter, double *out) {
   sum_range(q0, q1, partial, counter, out, [&](size_t i) {
     float4 v[9];
 #pragma unroll
     for (int a = 0; a < 9; ++a) v[a] = f[a * n4 + i];
-    float2 s = make_float2(v[0].x, v[0].y), e = make_float2(0.0f, 0.0f);
-#pragma unroll
-    for (int a = 1; a < 9; ++a) two_sum(s, e, make_float2(v[a].x, v[a].y));
-#pragma unroll
-    for (int a = 0; a < 9; ++a) two_sum(s, e, make_float2(v[a].z, v[a].w));
-    // (an infinite or NaN sum stands by itself)
-    float2 lo = make_float2(s.y, 0.0f), le = make_float2(0.0f, 0.0f);
-    two_sum(lo, le, make_float2(s.x, 0.0f));
-    const float err = (e.x + e.y) + le.x;
-    return (double)lo.x + (fabsf(err) <= FLT_MAX ? (double)err : 0.0);
+    return sum36(v);
   });
 }
 

@@ -105,6 +105,34 @@ def test_fp32_mass_is_the_exact_sum(nx, ny, walls):
         assert s.mass() == math.inf
 
 
+@pytest.mark.parametrize("nx,ny,walls", [(4, 5, True), (8, 6, False), (64, 9, True), (33, 7, True)])
+def test_fp32_mass_in_double_precision(nx, ny, walls):
+    """Populations added in double: a term passes through at most 9 roundings in
+    its density (none where their span allows an exact sum), 4 in a group of four
+    nodes, 10 in the block and 10 over the blocks.  The sum may exceed the
+    largest float; zeros, negative and subnormal populations count."""
+    eos = L.carnahan_starling()
+    T = 0.7 * L.lbm_eos_critical(eos)[0]
+    p = L.lbm_params_default(precision=32, check_every=0)
+    with L.Lbm(nx, ny, eos, T, 1.0, walls=walls, params=p, torch_state=False) as s:
+        for seed in range(7):
+            rng = np.random.default_rng(seed)
+            f = (rng.uniform(0.01, 2.0, (9, ny, nx)) * 10.0 ** rng.uniform(-3, 3, (9, ny, nx))).astype(np.float32)
+            if seed == 4:
+                f *= rng.choice(np.array([-1.0, 0.0, 1e-40, 1.0], np.float32), f.shape)
+            if seed == 5:
+                f *= np.float32(1e35)
+            if seed == 6:
+                f *= np.where(rng.random(f.shape) < 0.05, np.float32(-1e-6), np.float32(1))
+            if walls:
+                f[:, 0] = f[:, -1] = 0.0
+            s.set_f(f.astype(float))
+            g = f.astype(float).ravel()
+            want, size = math.fsum(g), math.fsum(abs(g))
+            assert size < 3.4e38 or seed == 5
+            assert abs(s.mass() - want) <= 33 * 2.0**-53 * size
+
+
 @pytest.mark.parametrize("nx,ny", [(33, 7), (64, 40)])
 def test_populations_through_doubles(nx, ny):
     """lbm_set_f rounds to nearest, lbm_get_f is exact, through either buffer
