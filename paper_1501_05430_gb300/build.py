@@ -32,7 +32,8 @@ UNITS = {
     "lbm_batch.cu": [],
     "lbm_adjoint.cu": ["-fmad=false"],
 }
-HEADERS = [os.path.join(CSRC, h) for h in ("lbm_internal.h", "lbm_fused.h", "lbm_tile.cuh", "lbm_node.cuh", "lbm_ref_node.cuh")] + [
+HEADERS = [os.path.join(CSRC, h) for h in ("lbm_internal.h", "lbm_fused.h", "lbm_tile.cuh", "lbm_node.cuh", "lbm_ref_node.cuh",
+                                           "lbm_round.cuh")] + [
     os.path.join(ROOT, "include", "lbm.h")]
 
 

@@ -7,9 +7,9 @@
 //    a fused multiply-add with the same single rounding, and such factors move
 //    freely through roundings (4 f_0 - 2 f_1 is twice 2 f_0 - f_1);
 //  - x / 3, x / 9, x / 36, x / 6, x / 12: one product and one fused
-//    multiply-add (div_const below) instead of a general division;
+//    multiply-add (div_const) instead of a general division;
 //  - other FP32 quotients and square roots are corrected approximations, packed
-//    (Divisor and root0 below);
+//    (quotients and root0_in_range, lbm_round.cuh);
 //  - values that several sums use in the same order are formed once (prefixes
 //    of the inverse transform, psi^2, and, per node instead of per neighbour,
 //    the weighted psi and U of the FP64 kernel).
@@ -20,105 +20,25 @@
 // FP64 is bound by the FP64 pipe (0.5 lanes per clock and SM quarter), FP32 by
 // instruction issue and the FMA pipe.
 #include <math.h>
+#include <string.h>
 
 #include <type_traits>
 
 #include "lbm_internal.h"
+#include "lbm_round.cuh"
 
 namespace {
 
-// ---- values: one double, or a lane pair of floats -------------------------------
-// F2 holds two nodes of a row; its operations are the packed FP32 instructions,
-// each lane rounded like the scalar operation.
-struct F2 {
-  float2 v;
-};
-// The assembler joins a packed product and the packed sum it goes into to one
-// fused operation whatever their rounding modifiers say, so sums are written as
-// fused operations themselves, a * 1 + b with a factor that it cannot know.
-__constant__ float2 c_one = {1.0f, 1.0f}, c_minus = {-1.0f, -1.0f};
-__device__ __forceinline__ F2 operator+(F2 a, F2 b) { return {__ffma2_rn(a.v, c_one, b.v)}; }
-__device__ __forceinline__ F2 operator-(F2 a, F2 b) { return {__ffma2_rn(b.v, c_minus, a.v)}; }
-__device__ __forceinline__ F2 operator-(F2 a) { return F2{make_float2(0.0f, 0.0f)} - a; }
-__device__ __forceinline__ F2 operator*(F2 a, F2 b) { return {__fmul2_rn(a.v, b.v)}; }
-__device__ __forceinline__ F2 operator/(F2 a, F2 b) { return {make_float2(a.v.x / b.v.x, a.v.y / b.v.y)}; }
-__device__ __forceinline__ F2 vfma(F2 a, F2 b, F2 c) { return {__ffma2_rn(a.v, b.v, c.v)}; }
-__device__ __forceinline__ double vfma(double a, double b, double c) { return fma(a, b, c); }
-__device__ __forceinline__ float vfma(float a, float b, float c) { return fmaf(a, b, c); }
-__device__ __forceinline__ F2 both(float c) { return {make_float2(c, c)}; }
-// sqrt(max(0, a)), the bits of sqrtf, from the hardware's approximation y by one
-// coupled Newton step for sqrt and 1/(2 sqrt) and a last one with the exact
-// remainder (Markstein, IBM J. Res. Dev. 34, 1990; compared with sqrtf over
-// every significand): packed, where sqrtf is a branch and nine instructions for
-// each lane.
-__device__ __forceinline__ F2 root0(F2 a) {
-  const float x = fmaxf(0.0f, a.v.x), z = fmaxf(0.0f, a.v.y);
-  float yx, yz;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(yx) : "f"(fmaxf(x, 1.17549435e-38f)));
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(yz) : "f"(fmaxf(z, 1.17549435e-38f)));
-  const F2 s = {make_float2(x, z)}, y = {make_float2(yx, yz)}, g = s * y, nh = both(-0.5f) * y;
-  const F2 e = vfma(nh, g, both(0.5f)), g1 = vfma(g, e, g), nh1 = vfma(nh, e, nh);
-  return vfma(vfma(g1, g1, -s), nh1, g1);
-}
-__device__ __forceinline__ double root0(double a) { return sqrt(fmax(0.0, a)); }
-__device__ __forceinline__ float root0(float a) { return sqrtf(fmaxf(0.0f, a)); }
+using namespace lbm_round;
+
 // a where x <= lim, else b
 __device__ __forceinline__ F2 where_le(F2 x, float lim, F2 a, F2 b) {
   return {make_float2(x.v.x <= lim ? a.v.x : b.v.x, x.v.y <= lim ? a.v.y : b.v.y)};
 }
-// Quotients by one divisor.  A lane pair takes two corrections of a y with y = 1/b
-// and the exact remainders, the bits of a division (Markstein, as above), packed:
-// the divisions of two lanes were a fifth of the FP32 step's instructions.  Where
-// the divisor is 0 (a state that counts as unstable) it gives NaN; what the field
-// queries return of the velocity is divided plainly.
-template <class V>
-struct Divisor {
-  V b;
-  __device__ __forceinline__ explicit Divisor(V d) : b(d) {}
-  __device__ __forceinline__ V under(V a) const { return a / b; }
-};
-template <>
-struct Divisor<F2> {
-  F2 nb, y;
-  __device__ __forceinline__ explicit Divisor(F2 b) : nb(-b) {
-    float x, z;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(x) : "f"(b.v.x));
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(z) : "f"(b.v.y));
-    y = {make_float2(x, z)};
-    y = vfma(vfma(nb, y, both(1.0f)), y, y);
-  }
-  __device__ __forceinline__ F2 under(F2 a) const {
-    const F2 q = a * y, q1 = vfma(vfma(nb, q, a), y, q);
-    return vfma(vfma(nb, q1, a), y, q1);
-  }
-};
 template <class R>
 __device__ __forceinline__ R where_le(R x, R lim, R a, R b) {
   return x <= lim ? a : b;
 }
-
-template <class V>
-struct Val;
-template <>
-struct Val<double> {
-  typedef double R;
-  static constexpr int N = 1;
-  __device__ __forceinline__ static double bc(double c) { return c; }
-  __device__ __forceinline__ static double lane(double v, int) { return v; }
-  __device__ __forceinline__ static void set(double &v, int, double x) { v = x; }
-};
-template <>
-struct Val<float> {
-  __device__ __forceinline__ static float bc(float c) { return c; }
-};
-template <>
-struct Val<F2> {
-  typedef float R;
-  static constexpr int N = 2;
-  __device__ __forceinline__ static F2 bc(float c) { return {make_float2(c, c)}; }
-  __device__ __forceinline__ static float lane(F2 v, int k) { return k ? v.v.y : v.v.x; }
-  __device__ __forceinline__ static void set(F2 &v, int k, float x) { (k ? v.v.y : v.v.x) = x; }
-};
 
 // Model constants, evaluated on the host in the kernel's precision in the order
 // in which the plain form evaluates them.
@@ -132,11 +52,8 @@ struct Canon {
   R s1, s2, s3, s4, s7, h1, h2, h3, h4, h7, h7x2, c15;  // rates, 1 - s/2, 2 (1 - s_7/2), 1.5 s_1
   R rho_max, ghost_max;
   R z3h, z3l, z9h, z9l, z36h, z36l, z6h, z6l, z12h, z12l;  // 1/d as a sum of two numbers
+  unsigned plain_lo, plain_len;           // bits of the densities [lo, hi] of plain(), hi - lo
 
-  static void split(R d, R *h, R *l) {
-    *h = (R)1 / d;
-    *l = (R)fma(-d, *h, (R)1) / d;  // the remainder is exact
-  }
   explicit Canon(const lbm_ctx *C) {
     const lbm_dev_params &P = C->dp;
     nx = P.nx, ny = P.ny, walls = P.walls, kind = P.eos_kind, n_iter = P.n_iter, wetting = P.wetting;
@@ -157,41 +74,68 @@ struct Canon {
     };
     h1 = half(s1), h2 = half(s2), h3 = half(s3), h4 = half(s4), h7 = half(s7), h7x2 = (R)2 * h7, c15 = (R)1.5 * s1;
     rho_max = (R)P.rho_max, ghost_max = (R)P.ghost_max;
-    split((R)3, &z3h, &z3l);
-    split((R)9, &z9h, &z9l);
-    split((R)36, &z36h, &z36l);
-    split((R)6, &z6h, &z6l);
-    split((R)12, &z12h, &z12l);
+    const_reciprocal((R)3, &z3h, &z3l);
+    const_reciprocal((R)9, &z9h, &z9l);
+    const_reciprocal((R)36, &z36h, &z36l);
+    const_reciprocal((R)6, &z6h, &z6l);
+    const_reciprocal((R)12, &z12h, &z12l);
+    // Densities whose quotients and square root stay where lbm_round.cuh takes the
+    // corrected approximations: rho itself in [2^-40, 2^30]; for Carnahan-Starling
+    // (1 - eta)^3 >= 2^-24, the numerator in [2^-80, 2^14] and the parts of U below
+    // 2^38, for Eq. 11 U below 2^38.  U = p - rho/3, where p and rho/3 cancel, is a
+    // multiple of their last place, 2^-66 or more, or 0.
+    double lo = 0x1p-40, hi = 0x1p30;
+    if (kind == LBM_EOS_CARNAHAN_STARLING) {
+      lo = fmax(lo, 0x1p-78 / (P.R * P.T));
+      hi = fmin(fmin(hi, (1.0 - 0x1p-7) * 4.0 / P.b), fmin(0x1p12 / (P.R * P.T), sqrt(0x1p36 / P.a)));
+    } else {
+      hi = fmin(hi, 0x1p34 / fmax(1.0, fmax(fmax(fabs(P.thv), fabs(P.thm)), fabs(P.thl))));
+    }
+    const float l = (float)lo, h = (float)hi;
+    unsigned hb;
+    memcpy(&plain_lo, &l, sizeof(l));
+    memcpy(&hb, &h, sizeof(h));
+    plain_len = hb - plain_lo;
+    if (!(l < h)) plain_lo = 0x7fffffffu, plain_len = 0u;  // none (the bits of a NaN)
   }
 };
 
-// x / d for d = 3, 6, 9, 12, 36, correctly rounded, from 1/d = h + l (Brisebarre,
-// Muller, Raina, "Accelerating correctly rounded floating-point division when
-// the divisor is known in advance", IEEE Trans. Computers 53, 2004).  Before its
-// rounding x h + RN(x l) is within 2^-2p (relative; p = 53 or 24) of x / d, and
-// x / d, whose odd denominator part is 3 or 9, is never nearer than 1/18 of a
-// last place to a midpoint between two numbers.
-template <class V, class R>
-__device__ __forceinline__ V div_const(V x, R h, R l) {
-  return vfma(x, Val<V>::bc(h), x * Val<V>::bc(l));
+// Both lanes of rho lie in [lo, hi]: positive numbers order like their bits.
+__device__ __forceinline__ bool plain(const Canon<float> &m, F2 rho) {
+  return __float_as_uint(rho.v.x) - m.plain_lo <= m.plain_len && __float_as_uint(rho.v.y) - m.plain_lo <= m.plain_len;
+}
+template <class R>
+__device__ __forceinline__ bool plain(const Canon<R> &, R) {
+  return true;
 }
 
-// psi and U of Eqs. 10-11.
-template <class V, class R>
-__device__ __forceinline__ void psi_U(const Canon<R> &m, V rho, V &psi, V &U) {
+// psi and U of Eqs. 10-11; over(a, b) is a / b and root(a) is sqrt(max(0, a)).
+template <class V, class R, class Over, class Root>
+__device__ __forceinline__ void psi_U(const Canon<R> &m, V rho, V &psi, V &U, Over over, Root root) {
   auto bc = [](R c) { return Val<V>::bc(c); };
   V p;
   if (m.kind == LBM_EOS_CARNAHAN_STARLING) {
     const V eta = bc(m.b4) * rho, e2 = eta * eta, one = bc((R)1), om = one - eta;
     const V num = ((one + eta) + e2) - e2 * eta, den = (om * om) * om;
-    p = Divisor<V>(den).under(((rho * bc(m.Rg)) * bc(m.T)) * num) - (bc(m.a) * rho) * rho;
+    p = over(((rho * bc(m.Rg)) * bc(m.T)) * num, den) - (bc(m.a) * rho) * rho;
   } else {
     p = where_le(rho, m.r1, rho * bc(m.thv),
                  where_le(rho, m.r2, bc(m.p1) + (rho - bc(m.r1)) * bc(m.thm),
                           bc(m.p2) + (rho - bc(m.r2)) * bc(m.thl)));
   }
   U = p - div_const(rho, m.z3h, m.z3l);
-  psi = root0(bc((R)-2) * U);
+  psi = root(bc((R)-2) * U);
+}
+template <class V, class R>
+__device__ __forceinline__ void psi_U(const Canon<R> &m, V rho, V &psi, V &U) {
+  psi_U(m, rho, psi, U, [](V a, V b) { return a / b; }, [](V a) { return root0(a); });
+}
+// The same for a rho that is plain(m, rho).
+__device__ __forceinline__ void psi_U_plain(const Canon<float> &m, F2 rho, F2 &psi, F2 &U) {
+  psi_U(m, rho, psi, U, [](F2 a, F2 b) { return Reciprocal(b).under(a); }, [](F2 a) { return root0_in_range(a); });
+}
+__device__ __forceinline__ void psi_U_plain(const Canon<double> &m, double rho, double &psi, double &U) {
+  psi_U(m, rho, psi, U);
 }
 
 // Ghost density, psi and U (Eqs. 19-21) from the densities around column x.
@@ -319,7 +263,7 @@ __device__ __forceinline__ void momentum(const V (&f)[9], V &d13, V &d24, V &jx,
 // rho: density, fs: post-collision populations.
 template <class V, class R, class W>
 __device__ __forceinline__ void collide(const Canon<R> &m, const W &win, int row, int i, const V (&f)[9], V rho,
-                                        R ss, V (&fs)[9]) {
+                                        bool ok, R ss, V (&fs)[9]) {
   auto bc = [](R c) { return Val<V>::bc(c); };
   V Fx, Fy, Qxx, Qyy, Qxy, d13, d24, jx, jy;
   force(m, win, row, i, ss, Fx, Fy, Qxx, Qyy, Qxy);
@@ -335,8 +279,8 @@ __device__ __forceinline__ void collide(const Canon<R> &m, const W &win, int row
   const V qy = ((vfma(m2, d24, f[5]) + f[6]) - f[7]) - f[8];
   const V nn = ((f[1] - f[2]) + f[3]) - f[4];
   const V no = ((f[5] - f[6]) + f[7]) - f[8];
-  const Divisor<V> by(rho);
-  const V vx = by.under(vfma(half, Fx, jx)), vy = by.under(vfma(half, Fy, jy));
+  V vx, vy;
+  quotients(vfma(half, Fx, jx), vfma(half, Fy, jy), rho, ok, vx, vy);
   const V vx2 = vx * vx, vy2 = vy * vy, v3 = bc((R)3) * (vx2 + vy2);
   const V vxF = vx * Fx, vyF = vy * Fy, S1 = bc((R)6) * (vxF + vyF);
   const V rvx = rho * vx, rvy = rho * vy;
@@ -388,13 +332,13 @@ struct Fields {
 template <class V, int R, class real>
 __device__ __forceinline__ void emit(const Canon<real> &m, const Step<real> &out, const Window<V, R> &win,
                                      const real (&)[R + 2][Val<V>::N * kH + 4], int w, int lane, int, int y, int x0,
-                                     const bool (&act)[Val<V>::N], bool node, bool, real ss, const V (&f)[9], V r) {
+                                     const bool (&act)[Val<V>::N], bool node, bool, real ss, const V (&f)[9], V r, bool ok) {
   constexpr int N = Val<V>::N;
   if (!node) return;
   const size_t n = (size_t)m.nx * m.ny;
   const bool dn = m.walls && y == 1, up = m.walls && y == m.ny - 2;
   V fs[9];
-  collide(m, win, w, lane + 2, f, r, ss, fs);
+  collide(m, win, w, lane + 2, f, r, ok, ss, fs);
   // streaming with half-way bounce-back
   const size_t ry = (size_t)y * m.nx, rd = (size_t)(y == 0 ? m.ny - 1 : y - 1) * m.nx,
                ru = (size_t)(y == m.ny - 1 ? 0 : y + 1) * m.nx;
@@ -423,7 +367,7 @@ __device__ __forceinline__ void emit(const Canon<real> &m, const Step<real> &out
 template <class V, int R, class real>
 __device__ __forceinline__ void emit(const Canon<real> &m, const Speed &out, const Window<V, R> &win,
                                      const real (&)[R + 2][Val<V>::N * kH + 4], int w, int lane, int, int, int,
-                                     const bool (&act)[Val<V>::N], bool node, bool, real ss, const V (&f)[9], V r) {
+                                     const bool (&act)[Val<V>::N], bool node, bool, real ss, const V (&f)[9], V r, bool) {
   constexpr int N = Val<V>::N;
   V Fx, Fy, Qxx, Qyy, Qxy, d13, d24, jx, jy;
   if (node) {
@@ -458,7 +402,7 @@ template <class V, int R, class real>
 __device__ __forceinline__ void emit(const Canon<real> &m, const Fields &out, const Window<V, R> &win,
                                      const real (&wrho)[R + 2][Val<V>::N * kH + 4], int w, int lane, int, int y,
                                      int x0, const bool (&act)[Val<V>::N], bool node, bool solid, real ss,
-                                     const V (&f)[9], V r) {
+                                     const V (&f)[9], V r, bool) {
   constexpr int N = Val<V>::N;
   if (!node && !solid) return;
   V v[7];
@@ -539,8 +483,13 @@ __global__ void __launch_bounds__((R + 3) * 32)
     for (int j = 0; j < N; ++j)
       if (row_warp ? act[j] : j == 0) kc[j] = c[row_warp ? x0 + lane + j * kH : gx];
   }
-  bool bad = false;
+  bool bad = false, ok = true;
   V f[9], r = Val<V>::bc((real)0);
+  auto put = [&](V psi, V U) {
+#pragma unroll
+    for (int j = 0; j < N; ++j)
+      if (row_warp ? act[j] : j == 0) win.put(w, row_warp ? lane + j * kH : hc, Val<V>::lane(psi, j), Val<V>::lane(U, j));
+  };
   if (on && (row_warp ? act[0] : true)) {
     if (!solid) {
       const real *q = fin + (size_t)y * m.nx + (row_warp ? x0 + lane : gx);
@@ -552,16 +501,16 @@ __global__ void __launch_bounds__((R + 3) * 32)
       r = f[0];
 #pragma unroll
       for (int a = 1; a < 9; ++a) r = r + f[a];
+      ok = plain(m, r);
       V psi, U;
-      psi_U(m, r, psi, U);
+      psi_U_plain(m, r, psi, U);
+      put(psi, U);
 #pragma unroll
       for (int j = 0; j < N; ++j) {
         if (row_warp ? act[j] : j == 0) {
-          const int c = row_warp ? lane + j * kH : hc;
           const real rj = Val<V>::lane(r, j);
           bad |= !(rj > (real)0) || rj > m.rho_max;
-          wrho[w][c + 2] = rj;
-          win.put(w, c, Val<V>::lane(psi, j), Val<V>::lane(U, j));
+          wrho[w][(row_warp ? lane + j * kH : hc) + 2] = rj;
         }
       }
     } else if (!geo) {  // Martys-Chen: psi = U = 0 on the solid rows
@@ -570,7 +519,22 @@ __global__ void __launch_bounds__((R + 3) * 32)
         if (row_warp ? act[j] : j == 0) win.put(w, row_warp ? lane + j * kH : hc, (real)0, (real)0);
     }
   }
-  __syncthreads();
+  // densities out of the ordinary (none in a stable state) take the plain division
+  // and root; decided for the CTA at the barrier, a branch for each thread in the
+  // load phase cost 2 of 44 us at 2047 x 1025
+  if (std::is_same<V, double>::value) {
+    __syncthreads();
+  } else if (__syncthreads_or(!ok)) {
+    if (!ok) {
+      V psi, U;
+      psi_U(m, r, psi, U);
+      put(psi, U);
+    }
+    ok = false;
+    __syncthreads();
+  } else {
+    ok = true;
+  }
   if (low || high) {  // uniform in the CTA
     if (on && solid) {
       // v == 0 from window rows 1, 2; v == ny - 1 from the two rows below it
@@ -592,7 +556,7 @@ __global__ void __launch_bounds__((R + 3) * 32)
   const bool dn = m.walls && y == 1, up = m.walls && y == m.ny - 2;
   const real ss = dn ? m.ss_dn : (up ? m.ss_up : (real)0);
   const bool node = warp >= 1 && warp <= nr && act[0];
-  emit(m, out, win, wrho, w, lane, warp, y, x0, act, node, solid && row_warp && on, ss, f, r);
+  emit(m, out, win, wrho, w, lane, warp, y, x0, act, node, solid && row_warp && on, ss, f, r, ok);
 }
 
 template <class V, int R, class OUT>
