@@ -56,13 +56,14 @@ inline RateK rate_consts(const double *s) {
   return k;
 }
 
-// Reciprocal square root, quotient and reciprocal.  CUDA's forms spend a few
-// instructions on subnormal operands; a parameter block that declares `short_math`
-// (the tile kernels') takes the bare hardware instructions, which give the same
-// bits for normal operands and are shorter in the chain that small domains wait
-// for (256 x 128: 3.0 -> 2.8 us per step).  No operand is subnormal in a stable
-// state.  The ring kernel, which overlaps that chain, keeps CUDA's: 4096 x 2048
-// ran 107.3 -> 110.8 us with the bare ones, for 5% fewer instructions.
+// Reciprocal square root and quotient of operands that are never subnormal: sqrt0
+// bounds its argument from below, and eos_node's quotient has the divisor (1 - e)^3
+// with 1 - e a multiple of 2^-24 near 0, and a numerator between 1 and 2 (for e < 1).
+// A parameter block that declares `short_math` (the tile kernels') takes the bare
+// hardware instructions for them, the same bits with a shorter chain, which small
+// domains wait for (256 x 128: 3.0 -> 2.8 us per step).  The ring kernel, which
+// overlaps that chain, keeps CUDA's functions: 4096 x 2048 ran 107.3 -> 110.8 us
+// with the bare ones.  (1/rho takes CUDA's everywhere: a density may be subnormal.)
 template <class PT, class = void>
 struct ShortMath {
   static constexpr bool value = false;
@@ -85,14 +86,6 @@ __device__ __forceinline__ float quotient(float a, float b) {
   asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
   return r;
 }
-template <class PT>
-__device__ __forceinline__ float reciprocal(float x) {
-  if (!ShortMath<PT>::value) return __fdividef(1.0f, x);
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-
 // sqrt for x >= 0 through the hardware reciprocal square root; exactly 0 at 0.
 template <class PT>
 __device__ __forceinline__ float sqrt0(const PT &, float x) {
@@ -246,7 +239,7 @@ __device__ __forceinline__ void collide_node2(const PT &P, const float2 *f, cons
   const float2 d57 = sub2(f[5], f[7]), d86 = sub2(f[8], f[6]);
   const float2 jx = add2(s13, add2(d57, d86));
   const float2 jy = add2(s24, sub2(d57, d86));
-  const float2 ir = make_float2(reciprocal<PT>(rho.x), reciprocal<PT>(rho.y));
+  const float2 ir = make_float2(__fdividef(1.0f, rho.x), __fdividef(1.0f, rho.y));
   const float2 half = bc2(0.5f);
   const float2 vx = mul2(fma2(half, Fx, jx), ir), vy = mul2(fma2(half, Fy, jy), ir);
   const float2 rvx = mul2(rho, vx), rvy = mul2(rho, vy);

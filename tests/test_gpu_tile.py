@@ -76,6 +76,23 @@ def test_narrow_domains_above_2_20_nodes(nx, ny, monkeypatch):
     assert np.array_equal(out[0], out[1])
 
 
+@pytest.mark.parametrize("rho", [2.0**-125, 2.0**-126, 0.9 * 2.0**-126, 2.0**-127, 1.001 * 2.0**-128])
+@pytest.mark.parametrize("nx,ny", [(64, 12), (400, 200), (1024, 1030)])
+def test_subnormal_densities(nx, ny, rho, monkeypatch):
+    """A uniform vapour of a density whose reciprocal is finite stays at rest (the
+    three sizes: two steps per launch, tiles of four and of six rows)."""
+    c, _ = _case(nx, ny, 1, walls=False, tau=0.9)
+    f = rho * np.array([4 / 9] + [1 / 9] * 4 + [1 / 36] * 4)[:, None, None] * np.ones((9, ny, nx))
+    out = []
+    for ring in (False, True):
+        with _context(c, f, monkeypatch, ring) as g:
+            g.step(5)
+            out.append((g.f(), g.status()))
+    c.orc.close()
+    assert np.array_equal(out[0][0], out[1][0]) and out[0][0].min() > 0
+    assert out[0][1] == out[1][1] == 0
+
+
 @pytest.mark.parametrize("y,x", [(1, 0), (3, 63), (4, 64), (8, 67)])
 def test_tile_kernel_flags_an_unstable_node(y, x, monkeypatch):
     """A density of 0 in the first and last row and column of tiles."""
