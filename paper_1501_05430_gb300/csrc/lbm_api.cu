@@ -766,10 +766,16 @@ int lbm_contact_angle(lbm_ctx *C, int wall, int x0, int x1, double *theta, doubl
   if (!C || (wall != 0 && wall != 1) || x0 < 0 || x1 > C->nx || x0 >= x1) return LBM_EINVAL;
   if (!C->walls) return LBM_EINVAL;
   if (C->status == LBM_ECUDA) return C->status;
-  CK(lbm_angle(C, lbm_make_angle_args(C, wall, x0, x1, C->d_res), &C->launches));
+  const lbm_angle_args A = lbm_make_angle_args(C, wall, x0, x1, C->d_res);
   lbm_angle_cut r;
+  CK(lbm_angle(C, A, &C->launches));
   CK(cudaMemcpyAsync(&r, C->d_res, sizeof(r), cudaMemcpyDeviceToHost, C->stream));
   CK(cudaStreamSynchronize(C->stream));
+  if (r.contact < 0) {
+    CK(lbm_angle_ties(C, A, &C->launches));
+    CK(cudaMemcpyAsync(&r, C->d_res, sizeof(r), cudaMemcpyDeviceToHost, C->stream));
+    CK(cudaStreamSynchronize(C->stream));
+  }
   double t, h, l;
   const int st = lbm_angle_of(r, C->rho_mid, &t, &h, &l);
   if (st) return st;

@@ -1167,8 +1167,16 @@ int lbm_batch_contact_angles(lbm_batch *B, int wall, double *theta, double *H, d
   BCK(cudaMemcpyAsync(B->d_angles, tab.data(), n * sizeof(lbm_angle_args), cudaMemcpyHostToDevice, B->stream));
   for (int i = 0; i < B->n; i += 65535)
     BCK(lbm_angle_many(B->d_angles, i, std::min(65535, B->n - i), blocks, B->stream));
-  BCK(cudaMemcpyAsync(r.data(), res, n * sizeof(lbm_angle_cut), cudaMemcpyDeviceToHost, B->stream));
-  BCK(cudaStreamSynchronize(B->stream));
+  for (bool again = true; again;) {
+    BCK(cudaMemcpyAsync(r.data(), res, n * sizeof(lbm_angle_cut), cudaMemcpyDeviceToHost, B->stream));
+    BCK(cudaStreamSynchronize(B->stream));
+    again = false;
+    for (int i = 0; i < B->n; ++i)
+      if (r[i].contact < 0) {
+        BCK(lbm_angle_ties(B->ctx[i], tab[i], &B->ctx[i]->launches));
+        again = true;
+      }
+  }
   for (int i = 0; i < B->n; ++i) {
     double t = NAN, h = NAN, l = NAN;
     const int st = lbm_angle_of(r[i], B->ctx[i]->rho_mid, &t, &h, &l);

@@ -143,14 +143,15 @@ cudaError_t lbm_mass_of(const lbm_ctx *C, const void *f, double *res, unsigned l
 // state f: the kernel finds where the contour cuts the boundary row and the
 // centre column, lbm_angle_of interpolates there.
 struct lbm_angle_cut {
-  int contact, xl, xr, steps;  // cuts right of xl and of xr, and above row `steps` from the boundary row
+  int contact;                 // 1: cuts found, 0: no contact line, -1: columns tie, lbm_angle_ties decides
+  int xl, xr, steps;           // cuts right of xl and of xr, and above row `steps` from the boundary row
   double rho[6];               // at xl, xl + 1; xr, xr + 1; the last liquid node up the centre column, the next
 };
 struct lbm_angle_args {
   const void *f;
   int nx, ny, wall, x0, x1;
   double rho_mid;
-  double *partial;    // scratch: a row of x1 - x0 doubles per 64 rows
+  double *partial;    // scratch: a row of x1 - x0 doubles per chunk of rows
   unsigned *counter;  // 0 before and after
   lbm_angle_cut *res;
 };
@@ -159,6 +160,8 @@ lbm_angle_args lbm_make_angle_args(const lbm_ctx *C, int wall, int x0, int x1, v
 int lbm_angle_of(const lbm_angle_cut &r, double rho_mid, double *theta, double *H, double *L);
 int lbm_angle_blocks(const lbm_angle_args &A);
 cudaError_t lbm_angle(const lbm_ctx *C, const lbm_angle_args &A, unsigned long long *launches);
+// the cuts of a domain that lbm_angle or lbm_angle_many left undecided
+cudaError_t lbm_angle_ties(const lbm_ctx *C, const lbm_angle_args &A, unsigned long long *launches);
 // the same for entries [first, first + count) (at most 65535) of a device table
 // of FP32 domains; blocks: the largest lbm_angle_blocks among them
 cudaError_t lbm_angle_many(const lbm_angle_args *tab, int first, int count, int blocks, cudaStream_t stream);

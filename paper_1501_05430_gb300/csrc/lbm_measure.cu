@@ -276,12 +276,20 @@ __device__ int block_reduce_int(int v, bool is_max, int *sh) {
 
 // ---- apparent contact angle ---------------------------------------------------
 // The centre column is the one with the largest sum over the wall's half, each
-// sum taken bottom to top, one addition after the other: a chain that no single
-// block shortens (1023 rows: 198 us, after 110 us for the densities of the
-// whole field).  Here all blocks sum chunks of rows in parallel, which places
-// every column's sum within a proven distance of the sequential one; only
-// columns within twice that distance of the largest (nearly always one) still
-// need the sequential sum to tell them apart, and the last block takes it.
+// sum taken bottom to top, one addition after the other: a chain of 35 ns a row.
+// In a half of few rows a block takes the sums of 32 columns so, from densities that
+// it forms in parallel.  In a higher one the blocks sum chunks of rows in parallel,
+// which places every column's sum within a proven distance of the sequential one;
+// only columns within twice that distance of the largest still need the sequential
+// sum to tell them apart.  Usually that is one column, or two (a droplet with a
+// mirror axis between columns): up to four are summed by the last block.  With more
+// (a wall without droplets, where all are equal) it leaves the domain undecided, and
+// a second pass (k_angle_ties) takes the sums of all columns in parallel.
+// us a call, FP32, one block over a density field / this, one column the largest | all
+// equal: 300 x 100 49 / 37 | 42 / 35, 400 x 200 50 / 48 | 50 / 50, 512 x 400 73 / 47 |
+// 75 / 50, 1001 x 501 122 / 47 | 114 / 97, 4096 x 2048 1365 / 182 | 1360 / 365.  A
+// low half ends at 200 rows: at 249 (1001 x 501) its chain costs the call of one
+// largest column 58 instead of 47, at 199 nothing (512 x 400).
 // Everything else (the boundary row's liquid run, the walk up the centre column)
 // reads its densities straight from the populations.  The last block's phases
 // follow one another, so they are kept short: comparisons of positive doubles
@@ -290,7 +298,10 @@ __device__ int block_reduce_int(int v, bool is_max, int *sh) {
 
 constexpr int kACols = 32, kALanes = 8, kARows = 64;  // columns, row lanes, rows of a block
 constexpr int kAThreads = kACols * kALanes;
-constexpr int kAFew = 16;  // candidates evaluated one after the other by the whole block
+constexpr int kALow = 200, kLCols = 8, kLLanes = 32;  // rows of a low half; columns and row lanes of a block there
+static_assert(kLCols * kLLanes == kAThreads, "one thread per column and lane");
+constexpr int kAFew = 4;                              // columns that the last block may sum from the populations
+constexpr int kTThreads = 128;                        // of a block of k_angle_ties
 
 __device__ __forceinline__ long long bits(double v) { return __double_as_longlong(v); }
 constexpr long long kInfBits = 0x7ff0000000000000ll;
@@ -314,144 +325,51 @@ __device__ __forceinline__ long long block_max_key(long long k, long long *sh) {
   return k;
 }
 
-// Blocks (kACols columns x kARows rows) of one domain along x, domains of a
-// table along y (tab == NULL: the one in A).
+// Rows [lo, hi) of the wall's half.
+__host__ __device__ __forceinline__ int half_lo(int ny, int wall) { return wall == 0 ? 1 : ny / 2; }
+__host__ __device__ __forceinline__ int half_hi(int ny, int wall) { return wall == 0 ? ny / 2 : ny - 1; }
+
+// Column of the largest sum (the lowest of equal ones) over the block's threads, in
+// every thread; INT_MAX where no thread has one.
+template <int THREADS>
+__device__ __forceinline__ int block_argmax(double best, int x) {
+  __shared__ double shv[THREADS / 32];
+  __shared__ int shx[THREADS / 32];
+  for (int o = 16; o > 0; o >>= 1) {
+    const double ov = __shfl_down_sync(0xffffffffu, best, o);
+    const int ox = __shfl_down_sync(0xffffffffu, x, o);
+    if (ov > best || (ov == best && ox < x)) best = ov, x = ox;
+  }
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) shv[threadIdx.x >> 5] = best, shx[threadIdx.x >> 5] = x;
+  __syncthreads();
+  best = shv[0], x = shx[0];
+  for (int j = 1; j < THREADS / 32; ++j)
+    if (shv[j] > best || (shv[j] == best && shx[j] < x)) best = shv[j], x = shx[j];
+  __syncthreads();
+  return x;
+}
+
+// The cuts of the contour with the boundary row and the centre column xc, by one block.
 template <typename R>
-__global__ void __launch_bounds__(kAThreads) k_angle(lbm_angle_args A, const lbm_angle_args *__restrict__ tab) {
-  if (tab) A = tab[blockIdx.y];
-  const int nx = A.nx, ny = A.ny, wall = A.wall, x0 = A.x0, x1 = A.x1, cols = x1 - x0;
+__device__ __forceinline__ void cut_at(const lbm_angle_args &A, int xc) {
+  __shared__ int shi[33];
+  const int nx = A.nx, ny = A.ny, wall = A.wall, x0 = A.x0, x1 = A.x1;
   const long long mid = bits(A.rho_mid);
   const R *f = (const R *)A.f;
   const size_t n = (size_t)nx * ny;
-  const int ylo = wall == 0 ? 1 : ny / 2, yhi = wall == 0 ? ny / 2 : ny - 1, half = yhi - ylo;
-  const int groups = (cols + kACols - 1) / kACols, chunks = (half + kARows - 1) / kARows;
-  if ((int)blockIdx.x >= groups * chunks) return;
-
-  // the block's part of its columns' sums; NaN where a density is negative or
-  // not finite (the bound below is for positive terms)
-  __shared__ double sh[kALanes][kACols];
-  {
-    const int g = (int)blockIdx.x % groups, k = (int)blockIdx.x / groups;
-    const int tx = threadIdx.x % kACols, ty = threadIdx.x / kACols, c = g * kACols + tx;
-    double s = 0.0;
-    if (c < cols) {
-      const int ya = ylo + k * kARows, yb = min(yhi, ya + kARows);
-      bool odd = false;
-#pragma unroll 2
-      for (int y = ya + ty; y < yb; y += kALanes) {
-        const double r = node_rho64(f, n, (size_t)y * nx + x0 + c);
-        odd |= (unsigned long long)bits(r) >= (unsigned long long)kInfBits;
-        s += r;
-      }
-      if (odd) s = (double)NAN;
-    }
-    sh[ty][tx] = s;
-    __syncthreads();
-    if (ty == 0 && c < cols) {
-      for (int j = 1; j < kALanes; ++j) s += sh[j][tx];
-      A.partial[(size_t)k * cols + c] = s;
-    }
-  }
-  if (!arrives_last(A.counter, (unsigned)(groups * chunks))) return;
-
-  // ---- the last block ----
   auto rho = [&](int y, int x) { return rho_at(f, n, (size_t)y * nx + x); };
-  __shared__ int shi[33];
-  __shared__ long long shk[kAThreads / 32];
-  // bits of a column's sum (NaN: above kInfBits)
-  auto total = [&](int c) {
-    double s = __ldcg(A.partial + c);
-    for (int k = 1; k < chunks; ++k) s += __ldcg(A.partial + (size_t)k * cols + c);
-    return bits(s);
-  };
-  long long top = -1;
-  for (int c = threadIdx.x; c < cols; c += kAThreads) {
-    const long long t = total(c);
-    if (t <= kInfBits) top = max(top, t);
-  }
-  top = block_max_key(top, shk);
-  // A sum of m positive terms, in any order, is within m 2^-53 of the true one
-  // (relative, to first order), so two sums of a column differ by at most
-  // m 2^-52 or m units in the last place; the largest sequential sum is among
-  // the columns within twice that of the largest of these (here eight times, as
-  // the units halve below a power of two).
-  const long long near = top - (8LL * half + 64LL);
-  // candidates: their first column and their number
-  int first = INT_MAX, count = 0;
-  for (int c = threadIdx.x; c < cols; c += kAThreads)
-    if (total(c) >= near) {
-      first = min(first, c);
-      ++count;
-    }
-  first = block_reduce_int(first, false, shi);
-  __shared__ int found;
-  if (threadIdx.x == 0) found = 0;
-  __syncthreads();
-  if (count) atomicAdd(&found, count);
-  __syncthreads();
-  int xc = INT_MAX;
-  if (found == 1) {
-    xc = x0 + first;
-  } else if (found <= kAFew) {
-    __shared__ int cand[kAFew];
-    __shared__ double line[kAThreads];
-    for (int j = 0, c = first; j < found; ++j) {
-      if (threadIdx.x == 0) cand[j] = c;
-      int next = INT_MAX;
-      for (int q = threadIdx.x; q < cols; q += kAThreads)
-        if (q > c && total(q) >= near) next = min(next, q);
-      c = block_reduce_int(next, false, shi);
-    }
-    double best = -DBL_MAX;
-    for (int j = 0; j < found; ++j) {
-      // sequential sum: densities of 256 rows at a time in parallel, added by one thread
-      double s = 0.0;
-      for (int y = ylo; y < yhi; y += kAThreads) {
-        if (y + (int)threadIdx.x < yhi) line[threadIdx.x] = rho(y + threadIdx.x, x0 + cand[j]);
-        __syncthreads();
-        if (threadIdx.x == 0)
-          for (int k = 0; k < min(kAThreads, yhi - y); ++k) s = s + line[k];
-        __syncthreads();
-      }
-      if (threadIdx.x == 0 && s > best) best = s, xc = x0 + cand[j];  // (ties: the lower column came first)
-    }
-    if (threadIdx.x == 0) shi[0] = xc;
-    __syncthreads();
-    xc = shi[0];
-    __syncthreads();
-  } else {  // many equal columns: a sequential sum per thread
-    __shared__ double shv[kAThreads / 32];
-    double best = -DBL_MAX;
-    for (int c = threadIdx.x; c < cols; c += kAThreads) {
-      if (total(c) < near) continue;
-      double s = 0.0;
-      for (int y = ylo; y < yhi; ++y) s = s + rho(y, x0 + c);
-      if (s > best || (s == best && x0 + c < xc)) best = s, xc = x0 + c;
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-      const double ov = __shfl_down_sync(0xffffffffu, best, o);
-      const int ox = __shfl_down_sync(0xffffffffu, xc, o);
-      if (ov > best || (ov == best && ox < xc)) best = ov, xc = ox;
-    }
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) shv[threadIdx.x >> 5] = best, shi[threadIdx.x >> 5] = xc;
-    __syncthreads();
-    best = shv[0], xc = shi[0];
-    for (int j = 1; j < kAThreads / 32; ++j)
-      if (shv[j] > best || (shv[j] == best && shi[j] < xc)) best = shv[j], xc = shi[j];
-    __syncthreads();
-  }
   lbm_angle_cut *res = A.res;
   if (xc < x0 || xc >= x1) {  // no column has a sum at all (NaN everywhere)
     if (threadIdx.x == 0) res->contact = 0;
     return;
   }
-
+  const int ylo = half_lo(ny, wall), yhi = half_hi(ny, wall);
   const int base = wall == 0 ? 1 : ny - 2, dir = wall == 0 ? 1 : -1;
   // liquid run of the boundary row containing xc
   int jl = INT_MIN, jr = INT_MAX;
   bool dry = false;
-  for (int x = x0 + threadIdx.x; x < x1; x += kAThreads) {
+  for (int x = x0 + threadIdx.x; x < x1; x += blockDim.x) {
     const bool vap = !at_least(rho(base, x), mid);
     if (vap && x < xc) jl = max(jl, x);
     if (vap && x > xc) jr = min(jr, x);
@@ -461,7 +379,7 @@ __global__ void __launch_bounds__(kAThreads) k_angle(lbm_angle_args A, const lbm
   const int ymax = wall == 0 ? yhi : ylo - 1;
   const int nwalk = wall == 0 ? (ymax - base - 1) : (base - ymax - 1);
   int kmin = INT_MAX;
-  for (int k = 1 + threadIdx.x; k <= nwalk; k += kAThreads)
+  for (int k = 1 + threadIdx.x; k <= nwalk; k += blockDim.x)
     if (!at_least(rho(base + k * dir, xc), mid)) {
       kmin = k;
       break;
@@ -482,6 +400,154 @@ __global__ void __launch_bounds__(kAThreads) k_angle(lbm_angle_args A, const lbm
     res->steps = kmin - 1;
     res->contact = 1;
   }
+}
+
+// Blocks of a domain: groups of columns x chunks of rows (a low half in one).
+struct AngleGrid {
+  bool low;
+  int groups, chunks;
+  __host__ __device__ __forceinline__ AngleGrid(int cols, int half) : low(half <= kALow) {
+    groups = low ? (cols + kLCols - 1) / kLCols : (cols + kACols - 1) / kACols;
+    chunks = low ? 1 : (half + kARows - 1) / kARows;
+  }
+};
+
+// The blocks of one domain along x, domains of a table along y (tab == NULL: the one
+// in A).
+template <typename R>
+__global__ void __launch_bounds__(kAThreads) k_angle(lbm_angle_args A, const lbm_angle_args *__restrict__ tab) {
+  if (tab) A = tab[blockIdx.y];
+  const int nx = A.nx, ny = A.ny, wall = A.wall, x0 = A.x0, x1 = A.x1, cols = x1 - x0;
+  const int ylo = half_lo(ny, wall), yhi = half_hi(ny, wall), half = yhi - ylo;
+  const AngleGrid G(cols, half);
+  const int chunks = G.chunks;
+  if ((int)blockIdx.x >= G.groups * chunks) return;
+
+  __shared__ double tile[kALow * kLCols];
+  {
+    const R *f = (const R *)A.f;
+    const size_t n = (size_t)nx * ny;
+    const int g = (int)blockIdx.x % G.groups, k = (int)blockIdx.x / G.groups, w = G.low ? kLCols : kACols;
+    const int tx = threadIdx.x % w, ty = threadIdx.x / w, c = g * w + tx;
+    double s = 0.0;
+    if (G.low) {  // the columns' sums in order
+      if (c < cols)
+#pragma unroll 2
+        for (int y = ty; y < half; y += kLLanes) tile[y * kLCols + tx] = node_rho64(f, n, (size_t)(ylo + y) * nx + x0 + c);
+      __syncthreads();
+      if (ty == 0 && c < cols)
+#pragma unroll 8
+        for (int y = 0; y < half; ++y) s = s + tile[y * kLCols + tx];
+    } else {  // the block's part of them; NaN where a density is negative or not finite
+              // (the bound below is for positive terms)
+      if (c < cols) {
+        const int ya = ylo + k * kARows, yb = min(yhi, ya + kARows);
+        bool odd = false;
+#pragma unroll 2
+        for (int y = ya + ty; y < yb; y += kALanes) {
+          const double r = node_rho64(f, n, (size_t)y * nx + x0 + c);
+          odd |= (unsigned long long)bits(r) >= (unsigned long long)kInfBits;
+          s += r;
+        }
+        if (odd) s = (double)NAN;
+      }
+      tile[ty * kACols + tx] = s;
+      __syncthreads();
+      if (ty == 0 && c < cols)
+        for (int j = 1; j < kALanes; ++j) s += tile[j * kACols + tx];
+    }
+    if (ty == 0 && c < cols) A.partial[(size_t)k * cols + c] = s;
+  }
+  if (!arrives_last(A.counter, (unsigned)(G.groups * chunks))) return;
+
+  // ---- the last block ----
+  double best = -DBL_MAX;
+  int xc = INT_MAX;
+  if (G.low) {
+    for (int c = threadIdx.x; c < cols; c += kAThreads) {
+      const double s = __ldcg(A.partial + c);
+      if (s > best) best = s, xc = x0 + c;
+    }
+    cut_at<R>(A, block_argmax<kAThreads>(best, xc));
+    return;
+  }
+  __shared__ long long shk[kAThreads / 32];
+  // bits of a column's sum (NaN: above kInfBits)
+  auto total = [&](int c) {
+    double s = __ldcg(A.partial + c);
+    for (int k = 1; k < chunks; ++k) s += __ldcg(A.partial + (size_t)k * cols + c);
+    return bits(s);
+  };
+  long long top = -1;
+  for (int c = threadIdx.x; c < cols; c += kAThreads) {
+    const long long t = total(c);
+    if (t <= kInfBits) top = max(top, t);
+  }
+  top = block_max_key(top, shk);
+  // A sum of m positive terms, in any order, is within m 2^-53 of the true one
+  // (relative, to first order), so two sums of a column differ by at most
+  // m 2^-52 or m units in the last place; the largest sequential sum is among
+  // the columns within twice that of the largest of these (here eight times, as
+  // the units halve below a power of two).
+  const long long near = top - (8LL * half + 64LL);
+  // candidates: their number, and the first few to be found
+  __shared__ int found, cand[kAFew];
+  if (threadIdx.x == 0) found = 0;
+  __syncthreads();
+  for (int c = threadIdx.x; c < cols; c += kAThreads)
+    if (total(c) >= near) {
+      const int k = atomicAdd(&found, 1);
+      if (k < kAFew) cand[k] = c;
+    }
+  __syncthreads();
+  if (found > kAFew) {
+    if (threadIdx.x == 0) A.res->contact = -1;
+    return;
+  }
+  xc = x0 + cand[0];
+  if (found > 1) {
+    // one after the other: the densities of 256 rows in parallel, added by one thread
+    __shared__ double line[kAThreads];
+    xc = INT_MAX;
+    for (int j = 0; j < found; ++j) {
+      const int x = x0 + cand[j];
+      double s = 0.0;
+      for (int y = ylo; y < yhi; y += kAThreads) {
+        if (y + (int)threadIdx.x < yhi)
+          line[threadIdx.x] = rho_at((const R *)A.f, (size_t)nx * ny, (size_t)(y + threadIdx.x) * nx + x);
+        __syncthreads();
+        if (threadIdx.x == 0)
+          for (int k = 0; k < min(kAThreads, yhi - y); ++k) s = s + line[k];
+        __syncthreads();
+      }
+      if (threadIdx.x == 0 && (s > best || (s == best && x < xc))) best = s, xc = x;
+    }
+    xc = block_argmax<kAThreads>(best, xc);
+  }
+  cut_at<R>(A, xc);
+}
+
+// The same from the densities rho [ny][nx] of the wall's half: every column's sum
+// by one thread, sums[] and the largest of them by the last block.
+template <typename R>
+__global__ void __launch_bounds__(kTThreads) k_angle_ties(lbm_angle_args A, const double *rho, double *sums) {
+  const int ylo = half_lo(A.ny, A.wall), half = half_hi(A.ny, A.wall) - ylo, cols = A.x1 - A.x0;
+  const int c = blockIdx.x * kTThreads + threadIdx.x;
+  if (c < cols) {
+    const double *v = rho + (size_t)ylo * A.nx + A.x0 + c;
+    double s = 0.0;
+#pragma unroll 16
+    for (int y = 0; y < half; ++y) s = s + v[(size_t)y * A.nx];
+    sums[c] = s;
+  }
+  if (!arrives_last(A.counter, gridDim.x)) return;
+  double best = -DBL_MAX;
+  int xc = INT_MAX;
+  for (int k = threadIdx.x; k < cols; k += kTThreads) {
+    const double s = __ldcg(sums + k);
+    if (s > best) best = s, xc = A.x0 + k;
+  }
+  cut_at<R>(A, block_argmax<kTThreads>(best, xc));
 }
 
 inline unsigned nblk(size_t n, int t) { return (unsigned)((n + t - 1) / t); }
@@ -555,7 +621,7 @@ lbm_angle_args lbm_make_angle_args(const lbm_ctx *C, int wall, int x0, int x1, v
 }
 
 int lbm_angle_of(const lbm_angle_cut &r, double rho_mid, double *theta, double *H, double *L) {
-  if (!r.contact) return LBM_ENOCONTACT;
+  if (r.contact <= 0) return LBM_ENOCONTACT;
   const double *q = r.rho;
   const double left = (double)r.xl + (rho_mid - q[0]) / (q[1] - q[0]);
   const double right = (double)r.xr + (q[2] - rho_mid) / (q[2] - q[3]);
@@ -566,8 +632,8 @@ int lbm_angle_of(const lbm_angle_cut &r, double rho_mid, double *theta, double *
 }
 
 int lbm_angle_blocks(const lbm_angle_args &A) {
-  const int half = A.wall == 0 ? A.ny / 2 - 1 : A.ny - 1 - A.ny / 2;
-  return ((A.x1 - A.x0 + kACols - 1) / kACols) * ((half + kARows - 1) / kARows);
+  const AngleGrid G(A.x1 - A.x0, half_hi(A.ny, A.wall) - half_lo(A.ny, A.wall));
+  return G.groups * G.chunks;
 }
 
 cudaError_t lbm_angle(const lbm_ctx *C, const lbm_angle_args &A, unsigned long long *launches) {
@@ -576,6 +642,19 @@ cudaError_t lbm_angle(const lbm_ctx *C, const lbm_angle_args &A, unsigned long l
     k_angle<double><<<g, kAThreads, 0, C->stream>>>(A, nullptr);
   else
     k_angle<float><<<g, kAThreads, 0, C->stream>>>(A, nullptr);
+  ++*launches;
+  return cudaGetLastError();
+}
+
+cudaError_t lbm_angle_ties(const lbm_ctx *C, const lbm_angle_args &A, unsigned long long *launches) {
+  // the sums go where the density of the lower solid row would be
+  cudaError_t e = lbm_rho64_rows(C, A.f, C->d_rho64, half_lo(A.ny, A.wall), half_hi(A.ny, A.wall), launches);
+  if (e != cudaSuccess) return e;
+  const unsigned g = nblk(A.x1 - A.x0, kTThreads);
+  if (C->precision == 64)
+    k_angle_ties<double><<<g, kTThreads, 0, C->stream>>>(A, C->d_rho64, C->d_rho64);
+  else
+    k_angle_ties<float><<<g, kTThreads, 0, C->stream>>>(A, C->d_rho64, C->d_rho64);
   ++*launches;
   return cudaGetLastError();
 }

@@ -49,6 +49,71 @@ def test_ties_are_broken_like_the_sequential_measurement(nx, ny, columns, precis
         assert H == oH and Lb == oL and th == pytest.approx(ot, rel=1e-15)
 
 
+# low halves (200 rows) and higher ones, with up to four and more columns to tell apart
+@pytest.mark.parametrize("wall", [0, 1])
+@pytest.mark.parametrize("precision", [32, 64])
+@pytest.mark.parametrize("nx,ny,columns", [(513, 400, 2), (60, 404, 2), (70, 405, 40), (700, 200, 40), (100, 502, 4), (100, 502, 5), (500, 602, 90), (3000, 66, 1500)])
+def test_ties_in_large_domains(nx, ny, columns, precision, wall):
+    sim, (rv, rl) = _sim(nx, ny, precision)
+    with sim:
+        sim.set_rho(_block(nx, ny, rv, rl, nx + ny, columns, wall)[:, :nx])
+        mid = sim.info.rho_mid
+        for x0, x1 in ((0, nx), (1, nx - 3)):
+            ot, oH, oL, _ = O.contact_angle_field(sim.rho(), wall, x0, x1, mid)
+            if math.isnan(ot):
+                with pytest.raises(L.LbmError):
+                    sim.contact_angle(wall, x0, x1)
+                continue
+            th, H, Lb = sim.contact_angle(wall, x0, x1)
+            assert H == oH and Lb == oL and th == pytest.approx(ot, rel=1e-15)
+
+
+@pytest.mark.parametrize("precision", [32, 64])
+@pytest.mark.parametrize("nx,ny", [(131, 140), (200, 500)])
+def test_angle_over_columns_with_negative_densities(nx, ny, precision):
+    """Sums with negative terms have no bound from the parallel ones: such columns are
+    always summed in order.  They may hold the largest sum (a large positive density
+    beside the negative one) or not."""
+    sim, (rv, rl) = _sim(nx, ny, precision)
+    with sim:
+        rho = _block(nx, ny, rv, rl, 3, 9, 0)
+        for boost in (False, True):
+            f = I.random_distributions(rho, 1)
+            x = nx // 3 + 4
+            f[:, ny // 2 - 2, x] *= -0.5
+            f[:, 30, 5] *= -3.0
+            if boost:
+                f[:, 24, x] *= 50.0 * rl / rv
+            sim.set_f(f)
+            ot, oH, oL, oxc = O.contact_angle_field(sim.rho(), 0, 0, nx, sim.info.rho_mid)
+            th, H, Lb = sim.contact_angle(0, 0, nx)
+            assert H == oH and Lb == oL and th == pytest.approx(ot, rel=1e-15)
+
+
+def test_a_wall_without_droplets_takes_no_longer_than_a_few_angles():
+    """All columns tie there: their sums are taken in parallel (one block alone took
+    a hundred times as long as the angle of a droplet)."""
+    import time
+
+    nx, ny = 4096, 1024
+    sim, (rv, rl) = _sim(nx, ny, 32)
+    with sim:
+        sim.set_rho(I.droplet_field(nx, ny, [(nx * 0.3, ny * 0.3, 0)], rv, rl))
+
+        def best(wall):
+            t = []
+            for _ in range(8):
+                t0 = time.perf_counter()
+                try:
+                    sim.contact_angle(wall, 0, nx)
+                except L.LbmError as e:
+                    assert e.status == L.LBM_ENOCONTACT
+                t.append(time.perf_counter() - t0)
+            return min(t)
+
+        assert best(1) < 5 * best(0)
+
+
 @pytest.mark.parametrize("precision", [32, 64])
 def test_no_contact_line(precision):
     sim, (rv, rl) = _sim(40, 30, precision)
@@ -83,6 +148,24 @@ def test_batch_angles_are_the_instances_own():
                 assert st[k] == e.status == L.LBM_ENOCONTACT and math.isnan(th[k])
             else:
                 assert st[k] == 0 and (th[k], H[k], Lb[k]) == own
+
+
+def test_batch_angles_of_large_instances_with_ties():
+    """Instances that the batch's pass leaves undecided, among others."""
+    eos = L.carnahan_starling()
+    T = 0.7 * L.lbm_eos_critical(eos)[0]
+    rv, rl = L.lbm_coexistence(eos, T)
+    sizes = [(512, 500), (64, 60), (512, 430), (508, 470)]
+    with L.LbmBatch([dict(nx=nx, ny=ny, eos=eos, T=T, tau=1.0, theta=None) for nx, ny in sizes]) as b:
+        for k, ((nx, ny), inst) in enumerate(zip(sizes, b.instances)):
+            inst.set_rho(_block(nx, ny, rv, rl, k, (2, 3, 1, 200)[k], 0))
+        for wall in (0, 1):
+            th, H, Lb, st = b.contact_angles(wall)
+            assert (st == (L.LBM_OK if wall == 0 else L.LBM_ENOCONTACT)).all()
+            if wall == 0:
+                for k, inst in enumerate(b.instances):
+                    ot, oH, oL, _ = O.contact_angle_field(inst.rho(), 0, 0, inst.nx, inst.info.rho_mid)
+                    assert (H[k], Lb[k]) == (oH, oL) == inst.contact_angle(0, 0, inst.nx)[1:]
 
 
 @pytest.mark.parametrize("nx,ny,walls", [(4, 5, True), (64, 33, True), (30, 17, False), (1024, 300, True)])
