@@ -1149,16 +1149,29 @@ int lbm_batch_contact_angles(lbm_batch *B, int wall, double *theta, double *H, d
   for (int i = 0; i < B->n; ++i)
     if (B->ctx[i]->status == LBM_ECUDA) return LBM_ECUDA;
   const size_t n = B->n;
-  if (!B->d_angles) {
-    if (cudaMalloc(&B->d_angles, n * (sizeof(lbm_angle_args) + sizeof(lbm_angle_cut))) != cudaSuccess) {
-      cudaGetLastError();
-      B->d_angles = nullptr;
-      return LBM_ENOMEM;
+  std::vector<lbm_angle_args> tab;
+  std::vector<lbm_angle_cut> r;
+  try {
+    tab.resize(n);
+    r.resize(n);
+  } catch (const std::bad_alloc &) {
+    return LBM_ENOMEM;
+  }
+  if (!B->d_angles && cudaMalloc(&B->d_angles, n * (sizeof(lbm_angle_args) + sizeof(lbm_angle_cut))) != cudaSuccess) {
+    cudaGetLastError();
+    B->d_angles = nullptr;
+    for (int i = 0; i < B->n; ++i) {  // no memory for the table: one by one
+      double t = NAN, h = NAN, l = NAN;
+      const int st = lbm_contact_angle(B->ctx[i], wall, 0, B->ctx[i]->nx, &t, &h, &l);
+      if (st == LBM_ECUDA) return st;
+      theta[i] = t;
+      if (H) H[i] = h;
+      if (L) L[i] = l;
+      if (status) status[i] = st;
     }
+    return LBM_OK;
   }
   lbm_angle_cut *res = (lbm_angle_cut *)(B->d_angles + n);
-  std::vector<lbm_angle_args> tab(n);
-  std::vector<lbm_angle_cut> r(n);
   int blocks = 0;
   for (int i = 0; i < B->n; ++i) {
     tab[i] = lbm_make_angle_args(B->ctx[i], wall, 0, B->ctx[i]->nx, res + i);

@@ -1,6 +1,7 @@
 """A batch whose list of tiles gets no device memory runs the persistent kernel
-instead: the library linked anew from its objects, with a cudaMalloc that
-refuses allocations of one size."""
+instead, and one without memory for its table of angles measures one by one: the
+library linked anew from its objects, with a cudaMalloc that refuses allocations of
+one size."""
 import os
 import subprocess
 
@@ -67,3 +68,13 @@ def test_no_memory_for_the_tiles(refuse):
             assert b.plan()["smem_bytes"] > 0
             b.step(6)
             assert b.status()[0] == 0 and np.array_equal(b[1].f(), want)
+
+
+def test_no_memory_for_the_table_of_angles(refuse):
+    with _batch() as b, _batch() as c:
+        b.step(6)
+        c.step(6)
+        want = b.contact_angles(0)
+        refuse(2 * 128)  # (two entries of 64 bytes an instance)
+        got = c.contact_angles(0)
+        assert all(np.array_equal(x, y, equal_nan=True) for x, y in zip(want, got))
