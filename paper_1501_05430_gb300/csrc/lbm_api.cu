@@ -710,12 +710,16 @@ int lbm_get_u(lbm_ctx *C, double *ux, double *uy) {
   return get_fields(C, {nullptr, nullptr, nullptr, ux, uy, nullptr, nullptr, nullptr, nullptr, nullptr});
 }
 
-// FP32 populations to and from the caller's doubles: converted on the device,
-// through the buffer of the field queries where it is there (eight planes at a
-// time), else through the density buffer (one).  The host link takes the caller's
-// pages at ~175 GB/s, so twice the bytes cost less than a loop over a fresh host
-// array: 800 x 400, us, set_f 814 -> 294 (density buffer) or 191, get_f 1042 ->
-// 269 or 181 (the 23 MB alone 130).
+// FP32 populations to and from the caller's doubles.  Many are converted on the
+// device, through the buffer of the field queries where it is there (eight planes at
+// a time), else through the density buffer (one): the host link takes the caller's
+// pages at ~175 GB/s, so twice the bytes cost less than a loop on the host.  Few are
+// converted there, in one copy: a copy and a kernel for every plane take 12 us to
+// read and 5 to write.  us, host | density buffer | field queries' buffer:
+//   get_f  64 x 32 18 | 113 | 30, 100 x 100 38 | 120 | 32, 256 x 128 100 | 127 | 42,
+//          400 x 200 231 | 151 | 60, 800 x 400 908 | 241 | 160;
+//   set_f  64 x 32 17 | 57 | 26, 128 x 128 44 | 135 | 42, 256 x 128 82 | 137 | 49,
+//          400 x 200 190 | 159 | 72, 800 x 400 739 | 266 | 177.
 namespace {
 struct Convert {
   double *buf;
@@ -731,6 +735,17 @@ int lbm_get_f(lbm_ctx *C, double *f) {
   if (C->precision == 64) {
     CK(cudaMemcpyAsync(f, C->f[C->cur], cnt * sizeof(double), cudaMemcpyDeviceToHost, C->stream));
     CK(cudaStreamSynchronize(C->stream));
+    return LBM_OK;
+  }
+  if (cnt <= (C->d_aux ? 80000 : 400000)) {
+    float *tmp = (float *)malloc(cnt * sizeof(float));
+    if (!tmp) return LBM_ENOMEM;
+    cudaError_t e = cudaMemcpyAsync(tmp, C->f[C->cur], cnt * sizeof(float), cudaMemcpyDeviceToHost, C->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(C->stream);
+    if (e == cudaSuccess)
+      for (size_t i = 0; i < cnt; ++i) f[i] = (double)tmp[i];
+    free(tmp);
+    CK(e);
     return LBM_OK;
   }
   const Convert V(C);
@@ -750,6 +765,16 @@ int lbm_set_f(lbm_ctx *C, const double *f) {
   if (C->precision == 64) {
     CK(cudaMemcpyAsync(C->f[C->cur], f, cnt * sizeof(double), cudaMemcpyHostToDevice, C->stream));
     CK(cudaStreamSynchronize(C->stream));
+    return LBM_OK;
+  }
+  if (cnt <= (C->d_aux ? 140000 : 600000)) {
+    float *tmp = (float *)malloc(cnt * sizeof(float));
+    if (!tmp) return LBM_ENOMEM;
+    for (size_t i = 0; i < cnt; ++i) tmp[i] = (float)f[i];
+    cudaError_t e = cudaMemcpyAsync(C->f[C->cur], tmp, cnt * sizeof(float), cudaMemcpyHostToDevice, C->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(C->stream);
+    free(tmp);
+    CK(e);
     return LBM_OK;
   }
   const Convert V(C);

@@ -139,3 +139,30 @@ def test_large_field_readback_in_chunks(nx, ny, precision):
     for out in (None, _pinned((ny, nx))):
         assert _same_bits(L.lbm_get_rho(ctx, out), want)
     L.lbm_destroy(ctx)
+
+
+# values below and above the numbers that are converted on the host, without and with
+# the field queries' buffer (9 nx ny; reading 400,000 and 80,000, writing 600,000 and 140,000)
+@pytest.mark.parametrize("nx,ny", [(90, 90), (120, 120), (130, 121), (300, 150), (310, 210), (333, 211)])
+def test_distributions_of_any_size_through_doubles(nx, ny):
+    c = _ctx(nx, ny)
+    rng = np.random.default_rng(nx)
+    for _ in range(2):
+        f = rng.uniform(1e-3, 1.0, (9, ny, nx))
+        f[:, 3, 3] = (1e-42, 1e-46, 3e38, 0.0, -0.0, -1.5, 1 / 3, 2.0**-127, 1 + 2.0**-24)
+        L.lbm_set_f(c, f)
+        assert np.array_equal(L.lbm_get_f(c), f.astype(np.float32).astype(np.float64))
+        L.lbm_get_u(c)  # (makes the buffer)
+    L.lbm_destroy(c)
+
+
+@pytest.mark.parametrize("nx,ny", [(4, 5), (64, 32), (100, 90)])
+def test_distributions_of_small_domains_take_one_copy(nx, ny):
+    """No kernel and no copy for every plane, which took ten times as long."""
+    c = _ctx(nx, ny)
+    f = np.random.default_rng(1).uniform(1e-3, 1.0, (9, ny, nx))
+    before = L.lbm_launch_count(c)
+    L.lbm_set_f(c, f)
+    assert np.array_equal(L.lbm_get_f(c), f.astype(np.float32).astype(np.float64))
+    assert L.lbm_launch_count(c) == before
+    L.lbm_destroy(c)
