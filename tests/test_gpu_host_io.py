@@ -166,3 +166,49 @@ def test_distributions_of_small_domains_take_one_copy(nx, ny):
     assert np.array_equal(L.lbm_get_f(c), f.astype(np.float32).astype(np.float64))
     assert L.lbm_launch_count(c) == before
     L.lbm_destroy(c)
+
+
+@pytest.mark.parametrize("precision", [32, 64])
+@pytest.mark.parametrize("nx,ny", [(4, 5), (90, 88), (100, 81), (126, 111), (128, 110), (300, 100)])
+def test_fields_together_and_one_by_one(nx, ny, precision):
+    """All fields, a few and single ones (in one read-back where they are few)."""
+    from paper_1501_05430_gb300 import inputs as I
+
+    c = _ctx(nx, ny, precision)
+    rho = np.random.default_rng(1).uniform(0.05, 0.3, (ny, nx))
+    L.lbm_set_f(c, I.random_distributions(rho, 2))
+    all8 = list(L.lbm_get_fields(c).values())
+    lib = L.load()
+    for chosen in ([0, 1], [3, 4], [2], [1, 5, 7], [0, 2, 4, 6, 7]):
+        out = [np.full((ny, nx), np.nan) if k in chosen else None for k in range(8)]
+        assert lib.lbm_get_fields(c, *[None if o is None else L._dp(o) for o in out]) == L.LBM_OK
+        for k in chosen:
+            assert np.array_equal(out[k], all8[k])
+    assert lib.lbm_get_fields(c, *[None] * 8) == L.LBM_OK
+    ux, uy = L.lbm_get_u(c)
+    only = np.empty((ny, nx))
+    assert lib.lbm_get_u(c, None, L._dp(only)) == L.LBM_OK
+    assert np.array_equal(only, uy) and not np.array_equal(ux, uy)
+    L.lbm_destroy(c)
+
+
+def test_fields_of_a_small_domain_take_one_read_back():
+    """Eight fields of 4 x 5 nodes cost little more than one (a read-back for each
+    made it five times as long)."""
+    import time
+
+    c = _ctx(4, 5)
+    L.lbm_set_rho(c, np.full((5, 4), 0.1))
+    lib, out = L.load(), [np.empty((5, 4)) for _ in range(8)]
+
+    def best(args):
+        t = []
+        for _ in range(200):
+            t0 = time.perf_counter()
+            assert lib.lbm_get_fields(c, *args) == L.LBM_OK
+            t.append(time.perf_counter() - t0)
+        return min(t)
+
+    args = [L._dp(o) for o in out]
+    assert best(args) < 3 * best([args[0]] + [None] * 7)
+    L.lbm_destroy(c)
