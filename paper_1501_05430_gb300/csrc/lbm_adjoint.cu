@@ -1,6 +1,6 @@
-// lbm_adjoint.cu -- discrete adjoint (reverse-time) of the reference step.
+// lbm_adjoint.cu -- discrete adjoint (reverse-time) of the canonical step.
 //
-// Forward step n -> n+1 (lbm_ref.cu): rho, psi, U (Eqs. 1, 10-11); ghost rows
+// Forward step n -> n+1 (lbm_canon.cu): rho, psi, U (Eqs. 1, 10-11); ghost rows
 // (Eqs. 19-21); per fluid node the force F (Eq. 9 [+ Eq. 14]) and tensor Q
 // (Eq. 17) from the 3x3 stencil of (psi, U); the MRT collision with Guo
 // forcing and the Eq. 16 source (Eqs. 4-6, 15); push streaming with half-way
@@ -42,6 +42,7 @@
 
 #include "lbm_internal.h"
 #include "lbm_ref_node.cuh"
+#include "lbm_round.cuh"
 
 using namespace lbm_ref;
 
@@ -66,31 +67,11 @@ struct lbm_tape {
 
 namespace {
 
+using lbm_round::over;
+using lbm_round::quot;
+using lbm_round::vfma;
+
 constexpr int kMaxIter = 64;
-
-__device__ __forceinline__ float fma_(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-__device__ __forceinline__ double fma_(double a, double b, double c) { return __fma_rn(a, b, c); }
-
-// a / b from y = 1/b rounded to nearest: each correction with the exact remainder
-// brings the quotient to 1 ulp and then to the correctly rounded one (Markstein,
-// IBM J. Res. Dev. 34, 1990), the bits of a division, without its special cases:
-// five instructions where several quotients share a divisor.  (A remainder below
-// the normal range, |a| < 1e-30 in FP32, can leave it an ulp off.)
-template <typename R>
-__device__ __forceinline__ R quot(R a, R b, R y) {
-  const R q0 = a * y, q1 = fma_(fma_(-b, q0, a), y, q0);
-  return fma_(fma_(-b, q1, a), y, q1);
-}
-// a / N for a small integer N: in FP32 one correction is enough for 3, 9 and
-// their multiples by powers of two (true of every significand)
-template <int N, typename R>
-__device__ __forceinline__ R over(R a) {
-  constexpr R y = (R)1 / (R)N;
-  if constexpr ((N & (N - 1)) == 0) return a * y;
-  if constexpr (sizeof(R) == 8) return quot(a, (R)N, y);
-  const R q = a * y;
-  return fma_(fma_(-(R)N, q, a), y, q);
-}
 
 // Row k of M times v, left to right (the products by 2 and 4 are exact, so the
 // fused ones round as separate ones).
@@ -102,7 +83,7 @@ __device__ __forceinline__ R moment(int k, const R (&v)[9]) {
   for (int a = 0; a < 9; ++a) {
     const R c = (R)MC(k, a);
     if (c == (R)0) continue;
-    acc = first ? c * v[a] : (c == (R)1 ? acc + v[a] : (c == (R)-1 ? acc - v[a] : fma_(c, v[a], acc)));
+    acc = first ? c * v[a] : (c == (R)1 ? acc + v[a] : (c == (R)-1 ? acc - v[a] : vfma(c, v[a], acc)));
     first = false;
   }
   return acc;
@@ -245,7 +226,7 @@ __device__ __forceinline__ void adj_collide(const Mdl<R> &m, const AdjRates<R> &
     for (int k = 0; k < 9; ++k) {
       const R c = (R)MC(k, a);
       if (c == (R)0) continue;
-      acc = c == (R)1 ? acc + mb[k] : (c == (R)-1 ? acc - mb[k] : fma_(c, mb[k], acc));
+      acc = c == (R)1 ? acc + mb[k] : (c == (R)-1 ? acc - mb[k] : vfma(c, mb[k], acc));
     }
     cl[a] = acc;
   }

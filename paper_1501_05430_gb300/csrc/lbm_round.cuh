@@ -23,8 +23,8 @@ __device__ __forceinline__ F2 operator-(F2 a) { return {__ffma2_rn(a.v, c_minus,
 __device__ __forceinline__ F2 operator*(F2 a, F2 b) { return {__fmul2_rn(a.v, b.v)}; }
 __device__ __forceinline__ F2 operator/(F2 a, F2 b) { return {make_float2(a.v.x / b.v.x, a.v.y / b.v.y)}; }
 __device__ __forceinline__ F2 vfma(F2 a, F2 b, F2 c) { return {__ffma2_rn(a.v, b.v, c.v)}; }
-__device__ __forceinline__ double vfma(double a, double b, double c) { return fma(a, b, c); }
-__device__ __forceinline__ float vfma(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double vfma(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float vfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ F2 both(float c) { return {make_float2(c, c)}; }
 
 template <class V>
@@ -128,6 +128,26 @@ inline void const_reciprocal(R d, R *h, R *l) {
 template <class V, class R>
 __device__ __forceinline__ V div_const(V x, R h, R l) {
   return vfma(x, Val<V>::bc(h), x * Val<V>::bc(l));
+}
+
+// a / b from y = 1/b rounded to nearest by two corrections, as Reciprocal::under, in
+// FP32 or FP64 (five instructions where several quotients share a divisor).  Finite
+// operands in the normal range; a below 1e-30 in FP32 (its remainder leaves the normal
+// range) may be a last place off.
+template <typename R>
+__device__ __forceinline__ R quot(R a, R b, R y) {
+  const R q0 = a * y, q1 = vfma(vfma(-b, q0, a), y, q0);
+  return vfma(vfma(-b, q1, a), y, q1);
+}
+// a / N for a small integer N, for such a: in FP32 one correction is enough for 3, 9
+// and their multiples by powers of two (compared for every significand).
+template <int N, typename R>
+__device__ __forceinline__ R over(R a) {
+  constexpr R y = (R)1 / (R)N;
+  if constexpr ((N & (N - 1)) == 0) return a * y;
+  if constexpr (sizeof(R) == 8) return quot(a, (R)N, y);
+  const R q = a * y;
+  return vfma(vfma(-(R)N, q, a), y, q);
 }
 
 }  // namespace lbm_round

@@ -28,6 +28,12 @@ __global__ void k(int what, const float2 *a, const float2 *b, float2 *q, size_t 
   if (what == 2) quotients(w, u, d, plain(d), x, y), q[i] = y.v;
   if (what == 3) q[i] = u.v.x >= 0.0f && u.v.y >= 0.0f && in_range(u, u) ? root0_in_range(u).v : root0(u).v;
   if (what == 4) q[i] = div_const(u, z.h, z.l).v;
+  if (what == 5) q[i] = make_float2(quot(u.v.x, d.v.x, 1.0f / d.v.x), quot(u.v.y, d.v.y, 1.0f / d.v.y));
+  if (what == 103) q[i] = make_float2(over<3>(u.v.x), over<3>(u.v.y));
+  if (what == 106) q[i] = make_float2(over<6>(u.v.x), over<6>(u.v.y));
+  if (what == 109) q[i] = make_float2(over<9>(u.v.x), over<9>(u.v.y));
+  if (what == 112) q[i] = make_float2(over<12>(u.v.x), over<12>(u.v.y));
+  if (what == 136) q[i] = make_float2(over<36>(u.v.x), over<36>(u.v.y));
 }
 // numbers of the bit patterns [u0, u1) whose corrected reciprocal or root is not the rounded one
 __global__ void k_count(unsigned u0, unsigned u1, unsigned *bad) {
@@ -155,3 +161,13 @@ def test_every_quotient_by_a_small_integer(run, d):
     for scale in (1.0, -(2.0**-60), 2.0**-94, 2.0**120):
         x = (SIGNIFICANDS * np.float32(scale)).astype(np.float32)
         _same(run(4, x, d=float(d)), x / np.float32(d))
+        _same(run(100 + d, x), x / np.float32(d))
+
+
+def test_quotients_that_share_a_rounded_reciprocal(run):
+    rng = np.random.default_rng(4)
+    for scale in (1.0, 2.0**-11, 2.0**6):
+        b = (SIGNIFICANDS * np.float32(scale)).astype(np.float32)
+        for a in (np.ones_like(b), rng.permutation(SIGNIFICANDS), -rng.permutation(SIGNIFICANDS) * np.float32(1e-29)):
+            _same(run(5, a, b), a / b)
+    _same(run(5, SIGNIFICANDS.copy(), np.repeat(ALL_ONES, SIGNIFICANDS.size)), SIGNIFICANDS / ALL_ONES)
