@@ -433,8 +433,13 @@ __device__ __forceinline__ void emit(const Canon<real> &m, const Fields &out, co
 // Tile of m.sw columns x R rows per CTA of R + 3 warps: warps 0 .. R + 1 each
 // load one row (the tile's, the one above, the one below), the last one the
 // columns beside the tile.  Window row w holds row y0 - 1 + w.
+// CTAs per SM that the registers leave room for: 56 registers a thread in tiles of 8
+// rows (with 62 and two CTAs FP64 at 400 x 200 took 103 us a step instead of 79) and
+// of 4 (with 80 and three, FP32 at 2047 x 1025 59 instead of 45), 64 in those of 2.
+constexpr int min_ctas(int R) { return R == 8 ? 3 : (R == 4 ? 5 : 6); }
+
 template <class V, int R, class OUT>
-__global__ void __launch_bounds__((R + 3) * 32)
+__global__ void __launch_bounds__((R + 3) * 32, min_ctas(R))
     k_canon(Canon<typename Val<V>::R> m, const typename Val<V>::R *__restrict__ fin, OUT out,
             const double *__restrict__ coef, int *flag) {
   typedef typename Val<V>::R real;
@@ -485,11 +490,6 @@ __global__ void __launch_bounds__((R + 3) * 32)
   }
   bool bad = false, ok = true;
   V f[9], r = Val<V>::bc((real)0);
-  auto put = [&](V psi, V U) {
-#pragma unroll
-    for (int j = 0; j < N; ++j)
-      if (row_warp ? act[j] : j == 0) win.put(w, row_warp ? lane + j * kH : hc, Val<V>::lane(psi, j), Val<V>::lane(U, j));
-  };
   if (on && (row_warp ? act[0] : true)) {
     if (!solid) {
       const real *q = fin + (size_t)y * m.nx + (row_warp ? x0 + lane : gx);
@@ -504,13 +504,14 @@ __global__ void __launch_bounds__((R + 3) * 32)
       ok = plain(m, r);
       V psi, U;
       psi_U_plain(m, r, psi, U);
-      put(psi, U);
 #pragma unroll
       for (int j = 0; j < N; ++j) {
         if (row_warp ? act[j] : j == 0) {
+          const int c = row_warp ? lane + j * kH : hc;
           const real rj = Val<V>::lane(r, j);
           bad |= !(rj > (real)0) || rj > m.rho_max;
-          wrho[w][(row_warp ? lane + j * kH : hc) + 2] = rj;
+          wrho[w][c + 2] = rj;
+          win.put(w, c, Val<V>::lane(psi, j), Val<V>::lane(U, j));
         }
       }
     } else if (!geo) {  // Martys-Chen: psi = U = 0 on the solid rows
@@ -522,13 +523,15 @@ __global__ void __launch_bounds__((R + 3) * 32)
   // densities out of the ordinary (none in a stable state) take the plain division
   // and root; decided for the CTA at the barrier, a branch for each thread in the
   // load phase cost 2 of 44 us at 2047 x 1025
-  if (std::is_same<V, double>::value) {
+  if constexpr (std::is_same<V, double>::value) {
     __syncthreads();
   } else if (__syncthreads_or(!ok)) {
     if (!ok) {
       V psi, U;
       psi_U(m, r, psi, U);
-      put(psi, U);
+#pragma unroll
+      for (int j = 0; j < N; ++j)
+        if (row_warp ? act[j] : j == 0) win.put(w, row_warp ? lane + j * kH : hc, Val<V>::lane(psi, j), Val<V>::lane(U, j));
     }
     ok = false;
     __syncthreads();
