@@ -982,9 +982,9 @@ int run_steps(lbm_batch *B, int nsteps) {
 // rows sweeps (45 us) and advances 34 nodes per ns in instances up to 128 wide
 // (three quarters of a CTA idle), about 68 in wider ones; the tile kernel
 // advances 50 whatever the width.  Measured, us per step, persistent / tile:
-// 6 of 300 x 100 47 / 6.4, 32 of 256 x 128 45 / 20, 64 of them 53 / 44, 128 of
-// them 69 / 83, 16 of 512 x 256 49 / 42, 32 of them 64 / 80, 1024 of 128 x 64
-// 236 / 162, 100 of the four sizes 102 / 122.  Without memory for the list of
+// 6 of 300 x 100 50 / 5.1, 32 of 256 x 128 45 / 19, 64 of them 53 / 44, 128 of
+// them 68 / 84, 16 of 512 x 256 48 / 42, 32 of them 64 / 81, 1024 of 128 x 64
+// 236 / 164, 100 of the four sizes 98 / 117.  Without memory for the list of
 // tiles the persistent kernel runs.
 int choose_tiles(lbm_batch *B, const lbm_batch_config &asked) {
   double narrow = 0.0, wide = 0.0;

@@ -16,8 +16,8 @@
 // bit (lbm_node.cuh).
 //
 // Measured, us per step, Carnahan-Starling with general rates, ring -> tile:
-// 64 x 32 3.9 -> 1.9, 256 x 128 5.5 -> 2.3, 400 x 200 5.9 -> 3.1, 512 x 512
-// 7.9 -> 5.6, 1024 x 512 11.4 -> 8.5, 1024 x 1024 17.3 -> 15.0.
+// 64 x 32 3.9 -> 2.0, 256 x 128 5.5 -> 2.3, 400 x 200 5.9 -> 3.1, 512 x 512
+// 7.9 -> 5.4, 1024 x 512 11.4 -> 8.5, 1024 x 1024 17.3 -> 15.1.
 #include <stdlib.h>
 
 #include "lbm_fused.h"
@@ -87,23 +87,24 @@ TileKernel kernel_ptr(const lbm_ctx *C, int rows) {
 // strips of 256 columns, the tile's of 64), from measurements of both.  While the
 // two state arrays (72 bytes per node) mostly stay in the 126 MB L2 the tile kernel
 // wins, past it the ring's deep prefetch does; the ring waits ~1.4 us for the ghost
-// rows of a walled domain, and general rates cost it more than the tile.  us per
-// step, ring / tile (6 rows), unit | general rates:
-//    walled    1280 x 1100 22.2 / 21.0 | 22.9 / 21.3, 1280 x 1200 23.0 / 24.8 | 23.7 / 23.5,
-//              1792 x 960 26.3 / 27.7 | 27.3 / 26.4, 2048 x 960 28.8 / 31.2 | 30.0 / 30.4,
-//              4096 x 2048 101 / 122 | 107 / 117;
-//    periodic  1024 x 1300 19.3 / 19.2 | 20.7 / 20.1, 1536 x 900 19.6 / 20.3 | 20.9 / 21.3.
-// Beyond, the tile wins where the ring's strips hold so many more columns than the
-// domain (threads past nx idle): walled 448 x 3600 25.6 / 25.9 | 27.6 / 24.8,
-// 1344 x 1344 29.5 / 29.5 | 29.9 / 27.9, 2624 x 1500 54.6 / 59.2 | 55.6 / 57.2,
-// 320 x 8000 52 / 39 | 56 / 38.
-// Tiles of 4 rows up to a million nodes (more CTAs, a shorter CTA: 256 x 128 2.95
-// against 3.26 us, 1024 x 512 9.1 / 9.4), of 6 rows above (fewer repeated loads:
-// 1024 x 1024 14.8 against 14.2, 1280 x 1000 19.3 / 18.4).
+// rows of a walled domain.  us per step, ring / tile (6 rows), unit | general rates:
+//    walled    1280 x 1100 22.4 / 21.1 | 22.6 / 21.7, 1280 x 1200 23.4 / 24.2 | 23.5 / 24.4,
+//              1792 x 960 26.8 / 27.3 | 27.1 / 27.8, 2048 x 960 29.3 / 30.8 | 29.6 / 31.5,
+//              4096 x 2048 103 / 118 | 107 / 120;
+//    periodic  1024 x 1300 19.7 / 19.3 | 20.5 / 20.0, 1536 x 900 20.0 / 20.4 | 20.7 / 21.1.
+// Beyond, the tile wins where the ring's strips hold a tenth more columns than the
+// domain (threads past nx idle): walled 448 x 3600 26.2 / 25.2 | 27.6 / 25.7,
+// 1344 x 1344 30.1 / 28.5 | 29.8 / 29.6, 2624 x 1500 55.8 / 58.3 | 55.5 / 59.2,
+// 320 x 8000 53 / 39 | 56 / 40.
+// Tiles of 4 rows up to a million nodes (more CTAs, a shorter CTA: 400 x 200 3.08
+// against 3.30 us, 1000 x 800 11.7 / 12.0, 1024 x 960 13.6 / 13.7), of 6 rows above
+// (fewer repeated loads: 1024 x 1024 14.6 against 14.5, 1280 x 1000 19.4 / 18.4).
 // Two steps per launch up to 50,000 nodes, where the launch and the loads are
-// most of a step and two thirds of the collisions can be made twice: us per step,
-// one / two, 64 x 32 2.65 / 2.07, 256 x 128 2.92 / 2.49, 300 x 100 2.91 / 2.20;
-// 400 x 200 3.52 / 3.91.
+// most of a step and two thirds of the collisions can be made twice, as long as the
+// CTAs fit on the chip at once: us per step, one / two, 64 x 32 2.43 / 1.96, 256 x 128
+// 2.50 / 2.22, 300 x 150 2.75 / 2.34; still 256 x 200 2.79 / 2.18 and 348 x 200
+// 2.76 / 2.22, which the line leaves out, then 400 x 200 3.08 / 3.51; the other way
+// round for tall and narrow domains below it, 60 x 800 2.63 / 3.09.
 // The ring kernel's own tuning variables ask for the ring.
 void lbm_tile_plan(lbm_ctx *C) {
   C->tile_rows = C->tile_pairs = 0;
@@ -111,8 +112,7 @@ void lbm_tile_plan(lbm_ctx *C) {
   const long long nodes = (long long)C->nx * C->ny;
   const int strips = (C->nx + kW - 1) / kW, ring_cols = (C->nx + 255) / 256 * 256;
   const int nrows = C->walls ? C->ny - 2 : C->ny;
-  const long long limit = C->walls ? (C->fused_unit ? 1420000 : 1720000) : (C->fused_unit ? 1360000 : 1420000);
-  if (1LL * strips * kW * C->ny > limit && 100LL * strips * kW > (C->fused_unit ? 85LL : 90LL) * ring_cols) return;
+  if (1LL * strips * kW * C->ny > (C->walls ? 1420000 : 1360000) && 100LL * strips * kW > 90LL * ring_cols) return;
   const int R = nodes <= 1000000 ? 4 : 6, bands = (nrows + R - 1) / R;
   if (bands > 65535) return;  // grid.y
   C->tile_rows = R;

@@ -430,7 +430,7 @@ def test_the_shape_reported_for_tiles_installs_tiles():
         b.step(3)
         best = b.autotune(trial_steps=8)
         tuned = b.plan()
-        assert tuned == tiles  # (a persistent step of this batch takes seven times as long)
+        assert tuned == tiles  # (a persistent step of this batch takes ten times as long)
         best.graph_launches = 2
         b.set_config(best)
         assert b.plan() == tiles
