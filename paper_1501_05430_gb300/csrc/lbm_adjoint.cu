@@ -380,7 +380,8 @@ constexpr int kStepThreads = 480;                // one node per thread in every
 // the part that passes through the moments in registers); dL/drho through psi
 // and U, and at the ghost nodes the transpose of the ghost rule; the sums.
 // Small domains are bound by the latency of a kernel and by its one CTA per SM,
-// whose 15 warps issue 30% of the time: five kernels with four global round trips
+// whose 15 warps issue in 38% of the cycles (256 x 128, waiting for loads, fixed
+// latencies, barriers and shared memory in equal parts): five kernels with four global round trips
 // of fields, aux and dL/drho took longer than the repeated work at the tiles'
 // edges (1.8 times the fields, 1.4 times the collisions), which at any size is
 // also paid for by the 170 bytes a node that are not moved.  The arithmetic was

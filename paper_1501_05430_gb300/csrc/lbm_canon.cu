@@ -16,9 +16,11 @@
 // About 350 FP64 operations per node instead of 700, and one pass over the
 // populations instead of two and a pass over three fields (FP32: 72 bytes per
 // node instead of 132).  us per step, before -> now: FP64 100 x 60 29.6 -> 16.7,
-// 400 x 200 104 -> 79; FP32 1001 x 501 30.4 -> 11.3, 2047 x 1025 131 -> 45.
-// FP64 is bound by the FP64 pipe (0.5 lanes per clock and SM quarter), FP32 by
-// instruction issue and the FMA pipe.
+// 400 x 200 104 -> 80; FP32 1001 x 501 30.4 -> 11.4, 2047 x 1025 131 -> 44.
+// FP64 is bound by the FP64 pipe (0.5 lanes per clock and SM quarter): 55% of its
+// cycles at 400 x 200, and at 100 x 60 one warp's chain through it (25%, 2.8 warps on
+// an SM).  FP32 waits for its loads at 28 warps per SM, of which 60% of the cycles
+// issue an instruction (1001 x 501; 14% of DRAM throughput).
 #include <math.h>
 #include <string.h>
 

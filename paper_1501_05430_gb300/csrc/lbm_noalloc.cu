@@ -1,11 +1,10 @@
 // lbm_noalloc.cu -- lbm_mass_noalloc: the total-mass reduction for callers that
 // cannot allocate device memory.
 //
-// lbm_mass computes rho per node into a context-owned scratch field and sums it
-// through a context-owned array of block partials.  This variant takes the
-// caller's distribution-function array directly, forms rho on the fly and keeps
-// its block partials in a fixed file-scope device array, so a call allocates
-// nothing.  Host code must not pass the array's name to a kernel (in host code
+// lbm_mass sums the populations of a context through a context-owned array of block
+// partials.  This variant takes the caller's distribution-function array and keeps
+// its block partials in a fixed file-scope device array, so a call needs no context
+// and allocates nothing.  Host code must not pass the array's name to a kernel (in host code
 // it names a host-side stand-in); the device address is looked up once per
 // device with cudaGetSymbolAddress and cached here.
 #include <mutex>

@@ -4,8 +4,8 @@
 // the double instantiation is bit-identical to any IEEE FP64 evaluation in the
 // same order: the fields of a state (rho, psi, U; Eqs. 1, 10, 11, with the
 // ghost values of Eqs. 19-21 or the Martys-Chen zero potential on the solid
-// rows), the macroscopic getters and the initial states.  The step in this
-// order is lbm_canon.cu.
+// rows; for the FP64 reverse step) and the initial states.  The step in this
+// order and the getters' fields are lbm_canon.cu.
 #include <math.h>
 #include <stdint.h>
 
